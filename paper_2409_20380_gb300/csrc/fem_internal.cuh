@@ -622,59 +622,63 @@ __device__ __forceinline__ void ebe_tail(const Reducer& red, CgCase* sc, double*
 }
 
 // Per-case sums over the grid.  Threads hold vals[q] for case c = threadIdx.x % rpad (the grid stride of
-// every caller is a multiple of rpad).  Returns true in the last block to finish, after red.out[q*rpad+c]
-// holds the grid totals (summed in a fixed order: deterministic).
+// every caller is a multiple of rpad; blockDim.x is a multiple of 32, at most kVecBlock).  Returns true in the
+// last block to finish, after red.out[q*rpad+c] holds the grid totals (summed in a fixed order: deterministic).
+// The sums are FP64, and GB300 adds two FP64 lanes a clock and SM with a long latency, so what bounds this
+// tail is the count of warp-wide FP64 adds and the longest chain of them.  Both levels (threads of a block,
+// rows of partial sums) therefore go through shared memory and one warp a quantity: 15 adds in four chains
+// and at most 5 shuffles, instead of shuffles in every warp and, in the last block, a serial loop over all
+// blockDim / (NQ rpad) slices (512 dependent adds for one case).  A k_update<double> of 729 nodes and one case
+// (2 blocks: all tail) took 14.9 us with those loops; ten FP64 steps of the 729-node
+// box went from 14.36 to 12.74 ms, a 4-case solve on 118,000 nodes from 4.72 to 4.50 ms.
+template <int NQ>
+__device__ __forceinline__ void warp_case_sums(const double (*sh)[kVecBlock], int len, int rpad, double* out) {
+  const int lane = threadIdx.x & 31;
+  for (int q = threadIdx.x >> 5; q < NQ; q += blockDim.x >> 5) {
+    double a[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+    for (int j = 0; j < kVecBlock / 32; ++j)
+      if (lane + 32 * j < len) a[j & 3] += sh[q][lane + 32 * j];
+    double v = (a[0] + a[1]) + (a[2] + a[3]);
+    for (int off = 16; off >= rpad; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+    if (lane < rpad) out[q * rpad + lane] = v;
+  }
+}
+
 template <int NQ>
 __device__ __forceinline__ bool block_reduce_last(double (&vals)[NQ], int rpad, const Reducer& red) {
-  __shared__ double sh[kVecBlock / 32][NQ][32];
+  __shared__ double sh[NQ][kVecBlock];
   __shared__ bool am_last;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-  for (int q = 0; q < NQ; ++q) {
-    double v = vals[q];
-    for (int off = 16; off >= rpad; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-    if (lane < rpad) sh[warp][q][lane] = v;
-  }
-  __syncthreads();
   const int V = NQ * rpad;
-  if (threadIdx.x < V) {
-    const int q = threadIdx.x / rpad, c = threadIdx.x % rpad;
-    double s = 0.0;
-    for (int w = 0; w < nw; ++w) s += sh[w][q][c];
-    red.partial[(size_t)blockIdx.x * V + threadIdx.x] = s;
-  }
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) sh[q][threadIdx.x] = vals[q];
+  __syncthreads();
+  warp_case_sums<NQ>(sh, blockDim.x, rpad, red.partial + (size_t)blockIdx.x * V);
   __threadfence();
   __syncthreads();
   if (threadIdx.x == 0) am_last = (atomicAdd(red.counter, 1u) == gridDim.x - 1);
   __syncthreads();
   if (!am_last) return false;
   __threadfence();
-  double* flat = &sh[0][0][0];
-  int S = blockDim.x / V;
-  if (S * V > (kVecBlock / 32) * NQ * 32) S = (kVecBlock / 32) * NQ * 32 / V;
-  if (threadIdx.x < S * V) {
-    const int v = threadIdx.x % V, sl = threadIdx.x / V;
-    // eight loads in flight per round so the L2 latency is paid few times; fixed assignment keeps the sum
-    // deterministic
-    double a[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-    int b = sl;
-    const int nb = (int)gridDim.x;
-    for (; b + 7 * S < nb; b += 8 * S) {
-      double t[8];
+  // thread (slice, case) sums every S-th row of the partial sums, four loads in flight a quantity
+  const int nb = (int)gridDim.x, S = blockDim.x / rpad, c = threadIdx.x & (rpad - 1), s0 = threadIdx.x / rpad;
 #pragma unroll
-      for (int u = 0; u < 8; ++u) t[u] = __ldcg(red.partial + (size_t)(b + u * S) * V + v);
+  for (int q = 0; q < NQ; ++q) {
+    const double* col = red.partial + q * rpad + c;
+    double a[4] = {0.0, 0.0, 0.0, 0.0};
+    int b = s0;
+    for (; b + 3 * S < nb; b += 4 * S) {
+      double t[4];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) a[u] += t[u];
+      for (int u = 0; u < 4; ++u) t[u] = __ldcg(col + (size_t)(b + u * S) * V);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) a[u] += t[u];
     }
-    for (int u = 0; b < nb; b += S, ++u) a[u & 7] += __ldcg(red.partial + (size_t)b * V + v);
-    flat[sl * V + v] = ((a[0] + a[1]) + (a[2] + a[3])) + ((a[4] + a[5]) + (a[6] + a[7]));
+    for (int u = 0; b < nb; b += S, ++u) a[u & 3] += __ldcg(col + (size_t)b * V);
+    sh[q][threadIdx.x] = (a[0] + a[1]) + (a[2] + a[3]);
   }
   __syncthreads();
-  if (threadIdx.x < V) {
-    double acc = 0.0;
-    for (int sl = 0; sl < S; ++sl) acc += flat[sl * V + threadIdx.x];
-    red.out[threadIdx.x] = acc;
-  }
+  warp_case_sums<NQ>(sh, (S < nb ? S : nb) * rpad, rpad, red.out);
   if (threadIdx.x == 0) *red.counter = 0u;
   __syncthreads();
   return true;

@@ -26,12 +26,10 @@ static int log2i(int r) {
   return s;
 }
 
+// Every thread of the last block calls it, after the cases' states were set by threads c < rpad.
 __device__ __forceinline__ void count_active(const CgCase* sc, int rpad, int* n_active) {
-  if (threadIdx.x == 0 && n_active) {
-    int n = 0;
-    for (int c = 0; c < rpad; ++c) n += sc[c].active;
-    *n_active = n;
-  }
+  const int n = __syncthreads_count((int)threadIdx.x < rpad && sc[threadIdx.x].active);
+  if (threadIdx.x == 0 && n_active) *n_active = n;
 }
 
 // bb = ||b||^2 over free DOFs; resets the case state.  gate (optional): a case whose gate is inactive is
@@ -136,7 +134,6 @@ __global__ void __launch_bounds__(kVecBlock, 3) k_resid(MeshView m, int rpad, in
         }
       }
     }
-    __syncthreads();
     count_active(sc, rpad, n_active);
   }
 }
@@ -215,7 +212,6 @@ __global__ void __launch_bounds__(kVecBlock, 3) k_update(MeshView m, int rpad, i
         }
       }
     }
-    __syncthreads();
     count_active(sc, rpad, n_active);
   }
 }
@@ -337,7 +333,6 @@ __global__ void __launch_bounds__(kVecBlock, 2) k_update_defer(MeshView m, int r
         }
       }
     }
-    __syncthreads();
     count_active(sc, rpad, n_active);
   }
 }
@@ -375,7 +370,6 @@ __global__ void __launch_bounds__(kVecBlock, 3) k_outer_resid(MeshView m, int rp
       s.active = (s.status == FEM_OK && s.bb > 0.0 && rrc >= tol * tol * s.bb) ? 1 : 0;
       s.inner_tol = inner_target(aim, s.relres, inner_max);
     }
-    __syncthreads();
     count_active(outer, rpad, n_active);
   }
 }

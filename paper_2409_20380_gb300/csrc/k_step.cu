@@ -827,12 +827,8 @@ __global__ void __launch_bounds__(kVecBlock, 2) k_r0(MeshView m, int rpad, int r
       s.inner_tol = inner_target(aim, s.relres, inner_max);
       if (inner) init_inner(inner[c], s, rrc, zrc);
     }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      int na = 0;
-      for (int c = 0; c < rpad; ++c) na += outer[c].active;
-      *n_active = na;
-    }
+    const int na = __syncthreads_count((int)threadIdx.x < rpad && outer[threadIdx.x].active);
+    if (threadIdx.x == 0) *n_active = na;
   }
 }
 
@@ -941,12 +937,8 @@ __global__ void __launch_bounds__(kVecBlock, 2) k_cert(MeshView m, int rpad, int
       s.inner_tol = inner_target(aim, s.relres, inner_max);
       if (inner) init_inner(inner[c], s, rrc, red.out[rpad + c]);
     }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      int na = 0;
-      for (int c = 0; c < rpad; ++c) na += outer[c].active;
-      *n_active = na;
-    }
+    const int na = __syncthreads_count((int)threadIdx.x < rpad && outer[threadIdx.x].active);
+    if (threadIdx.x == 0) *n_active = na;
   }
 }
 
