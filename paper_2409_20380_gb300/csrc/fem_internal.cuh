@@ -674,7 +674,9 @@ __device__ __forceinline__ bool block_reduce_last(double (&vals)[NQ], int rpad, 
 #pragma unroll
       for (int u = 0; u < 4; ++u) a[u] += t[u];
     }
-    for (int u = 0; b < nb; b += S, ++u) a[u & 3] += __ldcg(col + (size_t)b * V);
+#pragma unroll
+    for (int u = 0; u < 3; ++u)
+      if (b + u * S < nb) a[u] += __ldcg(col + (size_t)(b + u * S) * V);
     sh[q][threadIdx.x] = (a[0] + a[1]) + (a[2] + a[3]);
   }
   __syncthreads();

@@ -205,38 +205,186 @@ template <> struct Vec4<double> {
   }
 };
 
-template <typename T, int A0, int A1, int A2, int A3>
-__device__ __forceinline__ void tet_acc(const T* __restrict__ re, T aM, T aK, const T (&P)[8][3], T (&Q)[8][3]) {
-  T r[12];
-  Vec4<T>::load12(re, r);
-  const T lam = aK * r[9], mu = aK * r[10], ms = aM * r[11];
-  T G[3][3];
+// One hex in FP64: q += (aM M + aK K) p over its six tets.  ld(slot, P) gives a corner's values, rc(t, r) the
+// record of tet t, fl(slot, Q) takes a corner's sums.  The tets are visited around the cycle of their middle
+// corners (the diagonal corners 0 and 3 are in all six): a middle corner's values are loaded just before its
+// first tet and its sums leave right after its second; corner 2, which closes the cycle, leaves after the first
+// tet and is loaded again for the last, so at most four corners are live.
+// The FP64 pipe (2 lanes a clock and SM) bounds the FP64 products, so the operations are counted (per tet, 97
+// instead of the 126 of six separate element products):
+//   * the gradient needs only differences to corner 0, which all six tets share: 7 per hex instead of 18;
+//   * sigma g_b is accumulated straight into corner b's sums, and corner 0's stiffness part is minus the sum of
+//     the others' (rows of K_e add up to zero), taken once a corner instead of once a tet and corner;
+//   * mass: with s_t = p_0 + .. + p_3 of tet t and m_t = rho V / 20, corner a gets sum_t m_t s_t + (sum_t m_t) p_a;
+//     corners 0 and 3 share the sum over all six tets.  (Their m_t p_a are added tet by tet: a rounded
+//     sum of six equal m_t would bias every product of a uniform mesh.)
+// Measured: the staged FP64 product of 4 cases on 663,558 tets 702 -> 588 us, ten FP64 steps of the 729-node box
+// 12.74 -> 11.10 ms.  In FP32 the same form has longer dependent chains and no pipe to relieve: 113.5 against 108.5 us (16 cases,
+// 786,432 tets, pairs of cases) and 28.7 against 26.6 us (2 cases, 413,478 tets); FP32 keeps tet_acc.
+template <bool DOT, typename LD, typename FL, typename RC>
+__device__ __forceinline__ void hex_apply(LD ld, FL fl, RC rc, double aM, double aK, double& hd) {
+  static_assert(kHexTet[0][1] == 1 && kHexTet[0][2] == 2 && kHexTet[0][3] == 3 && kHexTet[1][1] == 1 &&
+                    kHexTet[1][2] == 3 && kHexTet[1][3] == 4 && kHexTet[4][1] == 7 && kHexTet[4][2] == 4 &&
+                    kHexTet[5][1] == 7 && kHexTet[5][3] == 6 && kHexTet[3][1] == 5 && kHexTet[3][2] == 6 &&
+                    kHexTet[2][1] == 5 && kHexTet[2][3] == 2,
+                "the visiting order follows the corner table");
+  struct Mid {
+    double P[3], D[3], Q[3];
+  };
+  double P0[3], P3[3], D3[3], B[3], Q0[3], Q3[3], W[3], W0[3], W3[3];
+  ld(0, P0);
+  ld(3, P3);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    D3[k] = P3[k] - P0[k];
+    B[k] = fma(P0[k], 4.0, D3[k]);       // s_t = 4 p_0 + D_3 + D_a + D_b
+    Q0[k] = Q3[k] = W[k] = W0[k] = W3[k] = 0.0;
+  }
+  auto enter = [&](int sl, Mid& m) {
+    ld(sl, m.P);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      m.D[k] = m.P[k] - P0[k];
+      m.Q[k] = 0.0;
+    }
+  };
+  // tet t with middle corners a, b; their and corner 3's gradients at positions ga, gb, g3 of the record
+  auto tet = [&](int t, int ga, int gb, int g3, Mid& a, Mid& b, double (&F)[3], double& ms) {
+    double r[12];
+    rc(t, r);
+    const double lam = aK * r[9], mu = aK * r[10], mu2 = mu + mu;
+    ms = aM * r[11];
+    double G[3][3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+      for (int j = 0; j < 3; ++j)
+        G[i][j] = fma(D3[i], r[3 * g3 + j], fma(b.D[i], r[3 * gb + j], a.D[i] * r[3 * ga + j]));
+    const double ltr = (G[0][0] + G[1][1] + G[2][2]) * lam;
+    double T[3][3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) T[i][i] = fma(G[i][i], mu2, ltr);
+    T[0][1] = T[1][0] = (G[0][1] + G[1][0]) * mu;
+    T[0][2] = T[2][0] = (G[0][2] + G[2][0]) * mu;
+    T[1][2] = T[2][1] = (G[1][2] + G[2][1]) * mu;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+        a.Q[k] = fma(T[k][j], r[3 * ga + j], a.Q[k]);
+        b.Q[k] = fma(T[k][j], r[3 * gb + j], b.Q[k]);
+        Q3[k] = fma(T[k][j], r[3 * g3 + j], Q3[k]);
+      }
+      F[k] = B[k] + (a.D[k] + b.D[k]);
+      W[k] = fma(F[k], ms, W[k]);
+      W0[k] = fma(P0[k], ms, W0[k]);
+      W3[k] = fma(P3[k], ms, W3[k]);
+    }
+  };
+  auto leave = [&](int sl, Mid& m, const double (&F1)[3], double m1, const double (&F2)[3], double m2, bool two) {
+    const double mm = two ? m1 + m2 : m1;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      Q0[k] -= m.Q[k];
+      double v = fma(F1[k], m1, m.Q[k]);
+      if (two) v = fma(F2[k], m2, v);
+      m.Q[k] = fma(m.P[k], mm, v);
+      if (DOT) hd = fma(m.P[k], m.Q[k], hd);
+    }
+    fl(sl, m.Q);
+  };
+  Mid x, y;
+  double Fa[3], Fb[3];
+  double ma, mb;
+  enter(2, x), enter(1, y);
+  tet(0, 0, 1, 2, y, x, Fa, ma);
+  leave(2, x, Fa, ma, Fa, ma, false);
+  enter(4, x);
+  tet(1, 0, 2, 1, y, x, Fb, mb);
+  leave(1, y, Fa, ma, Fb, mb, true);
+  enter(7, y);
+  tet(4, 0, 1, 2, y, x, Fa, ma);
+  leave(4, x, Fb, mb, Fa, ma, true);
+  enter(6, x);
+  tet(5, 0, 2, 1, y, x, Fb, mb);
+  leave(7, y, Fa, ma, Fb, mb, true);
+  enter(5, y);
+  tet(3, 0, 1, 2, y, x, Fa, ma);
+  leave(6, x, Fb, mb, Fa, ma, true);
+  enter(2, x);
+  tet(2, 0, 2, 1, y, x, Fb, mb);
+  leave(5, y, Fa, ma, Fb, mb, true);
+  leave(2, x, Fb, mb, Fb, mb, false);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    Q0[k] = (Q0[k] - Q3[k]) + (W[k] + W0[k]);
+    Q3[k] += W[k] + W3[k];
+    if (DOT) hd = fma(P3[k], Q3[k], fma(P0[k], Q0[k], hd));
+  }
+  fl(0, Q0);
+  fl(3, Q3);
+}
+
+template <int A0, int A1, int A2, int A3>
+__device__ __forceinline__ void tet_acc(const float (&r)[12], float aM, float aK, const float (&P)[8][3],
+                                        float (&Q)[8][3]) {
+  const float lam = aK * r[9], mu = aK * r[10], ms = aM * r[11];
+  float G[3][3];
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
-    const T d1 = P[A1][i] - P[A0][i], d2 = P[A2][i] - P[A0][i], d3 = P[A3][i] - P[A0][i];
+    const float d1 = P[A1][i] - P[A0][i], d2 = P[A2][i] - P[A0][i], d3 = P[A3][i] - P[A0][i];
 #pragma unroll
     for (int j = 0; j < 3; ++j) G[i][j] = d1 * r[j] + d2 * r[3 + j] + d3 * r[6 + j];
   }
-  const T tr = G[0][0] + G[1][1] + G[2][2];
-  const T mu2 = mu + mu;
-  T S[3][3];
+  const float tr = G[0][0] + G[1][1] + G[2][2];
+  const float mu2 = mu + mu;
+  float S[3][3];
 #pragma unroll
   for (int i = 0; i < 3; ++i) S[i][i] = lam * tr + mu2 * G[i][i];
   S[0][1] = S[1][0] = mu * (G[0][1] + G[1][0]);
   S[0][2] = S[2][0] = mu * (G[0][2] + G[2][0]);
   S[1][2] = S[2][1] = mu * (G[1][2] + G[2][1]);
-  T F[3][3];
+  float F[3][3];
 #pragma unroll
   for (int b = 0; b < 3; ++b)
 #pragma unroll
     for (int i = 0; i < 3; ++i) F[b][i] = S[i][0] * r[3 * b] + S[i][1] * r[3 * b + 1] + S[i][2] * r[3 * b + 2];
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
-    const T sum = P[A0][k] + P[A1][k] + P[A2][k] + P[A3][k];
+    const float sum = P[A0][k] + P[A1][k] + P[A2][k] + P[A3][k];
     Q[A0][k] += ms * (P[A0][k] + sum) - (F[0][k] + F[1][k] + F[2][k]);
     Q[A1][k] += ms * (P[A1][k] + sum) + F[0][k];
     Q[A2][k] += ms * (P[A2][k] + sum) + F[1][k];
     Q[A3][k] += ms * (P[A3][k] + sum) + F[2][k];
+  }
+}
+
+// One hex of a tiled kernel: the FP64 form above, or six tet products on registers of all eight corners (FP32).
+template <bool DOT, typename T, typename LD, typename FL, typename RC>
+__device__ __forceinline__ void hex_elem(LD ld, FL fl, RC rc, T aM, T aK, T& hd) {
+  if constexpr (sizeof(T) == 8) {
+    hex_apply<DOT>(ld, fl, rc, aM, aK, hd);
+  } else {
+    T P[8][3], Q[8][3], r[12];
+#pragma unroll
+    for (int sl = 0; sl < 8; ++sl) {
+      ld(sl, P[sl]);
+#pragma unroll
+      for (int k = 0; k < 3; ++k) Q[sl][k] = (T)0;
+    }
+    rc(0, r), tet_acc<kHexTet[0][0], kHexTet[0][1], kHexTet[0][2], kHexTet[0][3]>(r, aM, aK, P, Q);
+    rc(1, r), tet_acc<kHexTet[1][0], kHexTet[1][1], kHexTet[1][2], kHexTet[1][3]>(r, aM, aK, P, Q);
+    rc(2, r), tet_acc<kHexTet[2][0], kHexTet[2][1], kHexTet[2][2], kHexTet[2][3]>(r, aM, aK, P, Q);
+    rc(3, r), tet_acc<kHexTet[3][0], kHexTet[3][1], kHexTet[3][2], kHexTet[3][3]>(r, aM, aK, P, Q);
+    rc(4, r), tet_acc<kHexTet[4][0], kHexTet[4][1], kHexTet[4][2], kHexTet[4][3]>(r, aM, aK, P, Q);
+    rc(5, r), tet_acc<kHexTet[5][0], kHexTet[5][1], kHexTet[5][2], kHexTet[5][3]>(r, aM, aK, P, Q);
+#pragma unroll
+    for (int sl = 0; sl < 8; ++sl) {
+      if (DOT)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) hd += P[sl][k] * Q[sl][k];
+      fl(sl, Q[sl]);
+    }
   }
 }
 
@@ -279,31 +427,19 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? 2 : 1) k_ebe_hex(HexT
       const uint4 lw = __ldg(ht.hex_local + hx);
       int ls[8] = {(int)(lw.x & 0xffff), (int)(lw.x >> 16), (int)(lw.y & 0xffff), (int)(lw.y >> 16),
                    (int)(lw.z & 0xffff), (int)(lw.z >> 16), (int)(lw.w & 0xffff), (int)(lw.w >> 16)};
-      T P[8][3], Q[8][3];
-#pragma unroll
-      for (int sl = 0; sl < 8; ++sl) {
-        const int64_t g = snode[ls[sl]] & 0x0fffffff;
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-          P[sl][k] = p[(g * 3 + k) * rpad + c];
-          Q[sl][k] = (T)0;
-        }
-      }
       const T* re = rec + hx * 6 * kRec;
-      tet_acc<T, kHexTet[0][0], kHexTet[0][1], kHexTet[0][2], kHexTet[0][3]>(re + 0 * kRec, aM, aK, P, Q);
-      tet_acc<T, kHexTet[1][0], kHexTet[1][1], kHexTet[1][2], kHexTet[1][3]>(re + 1 * kRec, aM, aK, P, Q);
-      tet_acc<T, kHexTet[2][0], kHexTet[2][1], kHexTet[2][2], kHexTet[2][3]>(re + 2 * kRec, aM, aK, P, Q);
-      tet_acc<T, kHexTet[3][0], kHexTet[3][1], kHexTet[3][2], kHexTet[3][3]>(re + 3 * kRec, aM, aK, P, Q);
-      tet_acc<T, kHexTet[4][0], kHexTet[4][1], kHexTet[4][2], kHexTet[4][3]>(re + 4 * kRec, aM, aK, P, Q);
-      tet_acc<T, kHexTet[5][0], kHexTet[5][1], kHexTet[5][2], kHexTet[5][3]>(re + 5 * kRec, aM, aK, P, Q);
       T hdot = 0;
+      hex_elem<DOT, T>(
+          [&](int sl, T (&P)[3]) {
+            const T* src = p + (int64_t)(snode[ls[sl]] & 0x0fffffff) * per_node + c;
 #pragma unroll
-      for (int sl = 0; sl < 8; ++sl)
+            for (int k = 0; k < 3; ++k) P[k] = src[k * rpad];
+          },
+          [&](int sl, const T (&Q)[3]) {
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
-          if (DOT) hdot += P[sl][k] * Q[sl][k];
-          atomicAdd(qs + ls[sl] * per_node + k * rpad + c, Q[sl][k]);
-        }
+            for (int k = 0; k < 3; ++k) atomicAdd(qs + ls[sl] * per_node + k * rpad + c, Q[k]);
+          },
+          [&](int t, T (&r)[12]) { Vec4<T>::load12(re + t * kRec, r); }, aM, aK, hdot);
       if (seg) {
         double v1[1] = {(double)hdot};
         seg_add<1>(sacc, m.nseg, m.seg[snode[ls[0]] & 0x0fffffff], v1);
@@ -388,41 +524,6 @@ template <> struct SVec4<double> {
   }
 };
 
-template <typename T, int A0, int A1, int A2, int A3>
-__device__ __forceinline__ void tet_acc_s(const T* re, T aM, T aK, const T (&P)[8][3], T (&Q)[8][3]) {
-  T r[12];
-  SVec4<T>::load12(re, r);
-  const T lam = aK * r[9], mu = aK * r[10], ms = aM * r[11];
-  T G[3][3];
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    const T d1 = P[A1][i] - P[A0][i], d2 = P[A2][i] - P[A0][i], d3 = P[A3][i] - P[A0][i];
-#pragma unroll
-    for (int j = 0; j < 3; ++j) G[i][j] = d1 * r[j] + d2 * r[3 + j] + d3 * r[6 + j];
-  }
-  const T tr = G[0][0] + G[1][1] + G[2][2];
-  const T mu2 = mu + mu;
-  T S[3][3];
-#pragma unroll
-  for (int i = 0; i < 3; ++i) S[i][i] = lam * tr + mu2 * G[i][i];
-  S[0][1] = S[1][0] = mu * (G[0][1] + G[1][0]);
-  S[0][2] = S[2][0] = mu * (G[0][2] + G[2][0]);
-  S[1][2] = S[2][1] = mu * (G[1][2] + G[2][1]);
-  T F[3][3];
-#pragma unroll
-  for (int b = 0; b < 3; ++b)
-#pragma unroll
-    for (int i = 0; i < 3; ++i) F[b][i] = S[i][0] * r[3 * b] + S[i][1] * r[3 * b + 1] + S[i][2] * r[3 * b + 2];
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    const T sum = P[A0][k] + P[A1][k] + P[A2][k] + P[A3][k];
-    Q[A0][k] += ms * (P[A0][k] + sum) - (F[0][k] + F[1][k] + F[2][k]);
-    Q[A1][k] += ms * (P[A1][k] + sum) + F[0][k];
-    Q[A2][k] += ms * (P[A2][k] + sum) + F[1][k];
-    Q[A3][k] += ms * (P[A3][k] + sum) + F[2][k];
-  }
-}
-
 // Two cases per thread on Blackwell's paired FP32 pipe operations (one instruction, two lanes of values):
 // the cases of a node are adjacent in memory, so a pair loads as one float2 and every operation of the
 // element arithmetic is the same for both; the element records are shared and broadcast to both halves.
@@ -432,7 +533,7 @@ __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 __device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
 
-// The tet_acc_s arithmetic for a pair of cases.
+// The tet_acc arithmetic for a pair of cases.
 template <int A0, int A1, int A2, int A3>
 __device__ __forceinline__ void tet_acc_p(const float* re, float aM, float aK, const float2 (&P)[8][3],
                                           float2 (&Q)[8][3]) {
@@ -778,29 +879,18 @@ __global__ void __launch_bounds__(kBlock, (sizeof(T) == 4 && PK != 2) ? 2 : 1) k
       if (it + (int)blockDim.x < items) lw_next = __ldg(ht.hex_local + h0 + ((it + blockDim.x) >> rshift));
       int ls[8] = {(int)(lw.x & 0xffff), (int)(lw.x >> 16), (int)(lw.y & 0xffff), (int)(lw.y >> 16),
                    (int)(lw.z & 0xffff), (int)(lw.z >> 16), (int)(lw.w & 0xffff), (int)(lw.w >> 16)};
-      T P[8][3], Q[8][3];
-#pragma unroll
-      for (int sl = 0; sl < 8; ++sl)
-#pragma unroll
-        for (int kk = 0; kk < 3; ++kk) {
-          P[sl][kk] = ps[ls[sl] * per_node + (kk << rshift) + c];
-          Q[sl][kk] = (T)0;
-        }
       const T* re = sr + hl * 6 * kRec;
-      tet_acc_s<T, kHexTet[0][0], kHexTet[0][1], kHexTet[0][2], kHexTet[0][3]>(re + 0 * kRec, aM, aK, P, Q);
-      tet_acc_s<T, kHexTet[1][0], kHexTet[1][1], kHexTet[1][2], kHexTet[1][3]>(re + 1 * kRec, aM, aK, P, Q);
-      tet_acc_s<T, kHexTet[2][0], kHexTet[2][1], kHexTet[2][2], kHexTet[2][3]>(re + 2 * kRec, aM, aK, P, Q);
-      tet_acc_s<T, kHexTet[3][0], kHexTet[3][1], kHexTet[3][2], kHexTet[3][3]>(re + 3 * kRec, aM, aK, P, Q);
-      tet_acc_s<T, kHexTet[4][0], kHexTet[4][1], kHexTet[4][2], kHexTet[4][3]>(re + 4 * kRec, aM, aK, P, Q);
-      tet_acc_s<T, kHexTet[5][0], kHexTet[5][1], kHexTet[5][2], kHexTet[5][3]>(re + 5 * kRec, aM, aK, P, Q);
       T hdot = 0;
+      hex_elem<DOT, T>(
+          [&](int sl, T (&P)[3]) {
 #pragma unroll
-      for (int sl = 0; sl < 8; ++sl)
+            for (int kk = 0; kk < 3; ++kk) P[kk] = ps[ls[sl] * per_node + (kk << rshift) + c];
+          },
+          [&](int sl, const T (&Q)[3]) {
 #pragma unroll
-        for (int kk = 0; kk < 3; ++kk) {
-          if (DOT) hdot += P[sl][kk] * Q[sl][kk];
-          atomicAdd(qs + ls[sl] * per_node + (kk << rshift) + c, Q[sl][kk]);
-        }
+            for (int kk = 0; kk < 3; ++kk) atomicAdd(qs + ls[sl] * per_node + (kk << rshift) + c, Q[kk]);
+          },
+          [&](int t, T (&r)[12]) { SVec4<T>::load12(re + t * kRec, r); }, aM, aK, hdot);
       if (seg) {
         double v1[1] = {(double)hdot};
         seg_add<1>(sacc, m.nseg, m.seg[snode[ls[0]] & 0x0fffffff], v1);
@@ -1019,28 +1109,17 @@ __global__ void __launch_bounds__(kBlockCM, 1) k_ebe_hex_cm(HexTiles ht, MeshVie
         const uint4 lw = hexl[hl];
         int ls[8] = {(int)(lw.x & 0xffff), (int)(lw.x >> 16), (int)(lw.y & 0xffff), (int)(lw.y >> 16),
                      (int)(lw.z & 0xffff), (int)(lw.z >> 16), (int)(lw.w & 0xffff), (int)(lw.w >> 16)};
-        T P[8][3], Q[8][3];
-#pragma unroll
-        for (int sl = 0; sl < 8; ++sl)
-#pragma unroll
-          for (int kk = 0; kk < 3; ++kk) {
-            P[sl][kk] = ps[ls[sl] * PN + (kk << rshift) + c];
-            Q[sl][kk] = (T)0;
-          }
         const T* re = sr + hl * 6 * kRec;
-        tet_acc_s<T, kHexTet[0][0], kHexTet[0][1], kHexTet[0][2], kHexTet[0][3]>(re + 0 * kRec, aM, aK, P, Q);
-        tet_acc_s<T, kHexTet[1][0], kHexTet[1][1], kHexTet[1][2], kHexTet[1][3]>(re + 1 * kRec, aM, aK, P, Q);
-        tet_acc_s<T, kHexTet[2][0], kHexTet[2][1], kHexTet[2][2], kHexTet[2][3]>(re + 2 * kRec, aM, aK, P, Q);
-        tet_acc_s<T, kHexTet[3][0], kHexTet[3][1], kHexTet[3][2], kHexTet[3][3]>(re + 3 * kRec, aM, aK, P, Q);
-        tet_acc_s<T, kHexTet[4][0], kHexTet[4][1], kHexTet[4][2], kHexTet[4][3]>(re + 4 * kRec, aM, aK, P, Q);
-        tet_acc_s<T, kHexTet[5][0], kHexTet[5][1], kHexTet[5][2], kHexTet[5][3]>(re + 5 * kRec, aM, aK, P, Q);
+        hex_elem<DOT, T>(
+            [&](int sl, T (&P)[3]) {
 #pragma unroll
-        for (int sl = 0; sl < 8; ++sl)
+              for (int kk = 0; kk < 3; ++kk) P[kk] = ps[ls[sl] * PN + (kk << rshift) + c];
+            },
+            [&](int sl, const T (&Q)[3]) {
 #pragma unroll
-          for (int kk = 0; kk < 3; ++kk) {
-            if (DOT) hdot += P[sl][kk] * Q[sl][kk];
-            atomicAdd(qs + ls[sl] * PN + (kk << rshift) + c, Q[sl][kk]);
-          }
+              for (int kk = 0; kk < 3; ++kk) atomicAdd(qs + ls[sl] * PN + (kk << rshift) + c, Q[kk]);
+            },
+            [&](int t, T (&r)[12]) { SVec4<T>::load12(re + t * kRec, r); }, aM, aK, hdot);
       }
       if (DOT) {   // the warp's lanes share one case: one shared-memory add per warp
         for (int off = 16; off > 0; off >>= 1) hdot += __shfl_xor_sync(0xffffffffu, hdot, off);
