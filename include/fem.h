@@ -234,7 +234,7 @@ fem_status fem_mesh_set_absorbing(fem_mesh* m, int64_t n_faces, const int32_t* f
  * product the paper compares the EBE with, Section 3.3; built on first use and shared with the
  * certification product), FP64 blocks for FP64 products and their FP32 rounding for FP32 ones, any mesh,
  * not fused groups (those use 5, or 1 without hex patches).  hex_per_tile: 0 = automatic (largest tile
- * whose shared memory fits), or 64/128/256/512 hexes per tile.  Errors: FEM_ERR_ARG for other values or
+ * whose shared memory fits and that leaves a tile for every SM), or 64/128/256/512 hexes per tile.  Errors: FEM_ERR_ARG for other values or
  * variants 2-7 on a mesh without hex patches.
  */
 fem_status fem_mesh_tune(fem_mesh* m, int ebe_variant, int hex_per_tile);

@@ -419,10 +419,30 @@ struct fem_mesh {
       const Tuned& t = tuned[elem_bytes == 4 ? 0 : 1][lg];
       if (t.variant) *variant = t.variant, *hpt = t.hpt;
     }
+    if (*variant == 0 && *hpt == 0 && hex && !seg) {
+      // Automatic choice on hex patches by the work H x r (hexes x cases), both sides measured alone:
+      //   FP32: packed staged tiles (5; 3, then 2, where it does not apply), but the element kernel up to H r =
+      //   8192 with at most 4 cases (H = 512, r = 1: 8.4 us against 12.2; 4096: 10.8 against 12.8; 15,283: 17.8
+      //   against 14.7), where the tiles would leave most SMs idle.
+      //   FP64 (bound by the FP64 pipe): tiles of at most 128 hexes from H r = 500,000 on (131,072 hexes, 4
+      //   cases: 711 us against 728 staged, 761 element kernel), the element kernel below, whose threads spread
+      //   over all SMs (512 hexes, 1 case: 12.5 us against 33.5 for 64-hex tiles and 103 for one 512-hex tile;
+      //   15,283 hexes, 16 cases: 359 against 401).
+      const int64_t work = (E / 6) * rpad;
+      if (elem_bytes == 4) {
+        if (rpad <= 4 && work <= 8192) *variant = 1;
+      } else {
+        *variant = work < 500000 ? 1 : 2;
+        *hpt = *variant == 2 ? 128 : 0;
+        if (*variant == 2 && !tiles_for(elem_bytes, rpad, 2, 128)) *hpt = 0;
+      }
+    }
     if (*variant == 0) *variant = hex ? 5 : 1;       // packed staged tiles where they apply (else 3, 2, 1)
     if (!hex && *variant != 8) *variant = 1;
   }
-  // Tiling for the resolved variant: the largest tile whose shared memory fits (or the requested size).
+  // Tiling for the resolved variant: the requested size, else the largest tile whose shared memory fits and that
+  // still gives every SM a tile (else the smallest that fits).  H = 68,913, FP32: 270 tiles of 256 hexes against
+  // 135 of 512, 16.8 against 19.0 us (1 case) and 21.8 against 28.1 (2 cases).
   const HexTiles* tiles_for(size_t elem_bytes, int rpad, int variant, int hpt) const {
     if (!hex || variant == 1) return nullptr;
     const HexTiles* best = nullptr;
@@ -447,7 +467,8 @@ struct fem_mesh {
         need = (size_t)t.nloc_max * (3 * rpad * elem_bytes + 4);
         budget = elem_bytes == 4 ? 100 * 1024 : 200 * 1024;
       }
-      if (need <= budget || (hpt && need <= 220 * 1024)) best = &t;
+      if (need > budget && !(hpt && need <= 220 * 1024)) continue;
+      if (!best || t.n_tiles >= sm_count()) best = &t;
     }
     return best;
   }
@@ -466,7 +487,7 @@ struct fem_mesh {
 };
 
 // EBE product q = (aM M + aK K) p on the mesh: the tiled hex kernel when the mesh has hex patches and a
-// tiling fits, else the generic element kernel (q masked on Dirichlet DOFs by the consumers).
+// tiling fits, else the generic element kernel.  Dirichlet rows of q are zero.
 template <typename T>
 static cudaError_t ebe_elem_product(const fem_mesh* m, int rpad, const T* p, T* q, double aM, double aK,
                                     const Reducer* red, CgCase* sc, double* ptq, const int* gate, cudaStream_t s,
@@ -2259,11 +2280,9 @@ fem_status fem_ebe_apply(fem_mesh* m, int precision, const void* p_dev, void* q_
   if (precision == FEM_FP64) {
     CU(ebe_product<double>(m, n_rhs, (const double*)p_dev, (double*)q_dev, alpha_M, alpha_K,
                            ptq_dev ? &red : nullptr, nullptr, ptq_dev, nullptr, s));
-    CU(launch_mask<double>(m->N, n_rhs, m->fm, (double*)q_dev, s));
   } else if (precision == FEM_FP32_INNER) {
     CU(ebe_product<float>(m, n_rhs, (const float*)p_dev, (float*)q_dev, alpha_M, alpha_K,
                           ptq_dev ? &red : nullptr, nullptr, ptq_dev, nullptr, s));
-    CU(launch_mask<float>(m->N, n_rhs, m->fm, (float*)q_dev, s));
   } else {
     return fail(FEM_ERR_ARG, "unknown precision");
   }

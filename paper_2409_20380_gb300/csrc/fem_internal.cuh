@@ -176,7 +176,7 @@ cudaError_t launch_binv(int64_t N, const double* D, const uint8_t* freemask, dou
                         int* err_flag, cudaStream_t s);
 
 // q = (aM M + aK K) pm  (+ aK K pk - aK K pm when pk != nullptr: M acts on pm, K on pk).  q is zeroed
-// first; Dirichlet DOFs of q are NOT masked (consumers mask).  If red != nullptr the per-case p^T q
+// first; Dirichlet DOFs of q stay zero.  If red != nullptr the per-case p^T q
 // (element-wise p_e^T A_e p_e) is reduced into red->out[c] / ptq_out[c] and, if sc != nullptr, the CG
 // step length alpha = rho / p^T A p is set.  gate: skip when *gate == 0.
 template <typename T>

@@ -5,11 +5,12 @@
 // multi-RHS form.  Element apply in factorised form:
 //   G = sum_b p_b g_b^T,  sigma = lambda tr(G) I + mu (G + G^T),  (K_e p)_a = V sigma g_a,
 //   (M_e p)_a = rho V / 20 (p_a + sum_b p_b).
-// This generic kernel scatters with global atomics; fixed DOFs are left to the consumer to mask.
+// This generic kernel scatters with global atomics into a zeroed q, skipping Dirichlet DOFs (rows stay zero).
 #include <cuda_fp16.h>
 
 #include "fem_internal.cuh"
 
+#include <algorithm>
 #include <mutex>
 #include <unordered_map>
 
@@ -48,75 +49,152 @@ static int log2i(int r) {
   return s;
 }
 
-template <typename T, bool TWO, bool DOT>
-__global__ void __launch_bounds__(kBlock) k_ebe_atomic(MeshView m, int rpad, int rshift, const T* __restrict__ pm,
+// Paired FP32 operations (one instruction, two cases).
+__device__ __forceinline__ float2 bc2(float v) { return make_float2(v, v); }
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
+
+// The values a thread of the generic kernel works on: one case (float, double), or two adjacent cases of a node in
+// paired FP32 operations.
+template <typename T, int NC> struct ElemVal;
+template <typename T> struct ElemVal<T, 1> {
+  T v;
+  __device__ __forceinline__ static ElemVal load(const T* p) { return {*p}; }
+  __device__ __forceinline__ static ElemVal zero() { return {(T)0}; }
+  __device__ __forceinline__ void add_to(T* q) const { atomicAdd(q, v); }
+};
+template <> struct ElemVal<float, 2> {
+  float2 v;
+  __device__ __forceinline__ static ElemVal load(const float* p) { return {*reinterpret_cast<const float2*>(p)}; }
+  __device__ __forceinline__ static ElemVal zero() { return {make_float2(0.f, 0.f)}; }
+  __device__ __forceinline__ void add_to(float* q) const { atomicAdd(reinterpret_cast<float2*>(q), v); }
+};
+template <typename T> __device__ __forceinline__ ElemVal<T, 1> ev_add(ElemVal<T, 1> a, ElemVal<T, 1> b) { return {a.v + b.v}; }
+template <typename T> __device__ __forceinline__ ElemVal<T, 1> ev_sub(ElemVal<T, 1> a, ElemVal<T, 1> b) { return {a.v - b.v}; }
+template <typename T> __device__ __forceinline__ ElemVal<T, 1> ev_mul(ElemVal<T, 1> a, T b) { return {a.v * b}; }
+__device__ __forceinline__ ElemVal<float, 1> ev_fma(ElemVal<float, 1> a, float b, ElemVal<float, 1> c) { return {fmaf(a.v, b, c.v)}; }
+__device__ __forceinline__ ElemVal<double, 1> ev_fma(ElemVal<double, 1> a, double b, ElemVal<double, 1> c) { return {fma(a.v, b, c.v)}; }
+__device__ __forceinline__ ElemVal<float, 1> ev_fmv(ElemVal<float, 1> a, ElemVal<float, 1> b, ElemVal<float, 1> c) { return {fmaf(a.v, b.v, c.v)}; }
+__device__ __forceinline__ ElemVal<double, 1> ev_fmv(ElemVal<double, 1> a, ElemVal<double, 1> b, ElemVal<double, 1> c) { return {fma(a.v, b.v, c.v)}; }
+__device__ __forceinline__ ElemVal<float, 2> ev_add(ElemVal<float, 2> a, ElemVal<float, 2> b) { return {add2(a.v, b.v)}; }
+__device__ __forceinline__ ElemVal<float, 2> ev_sub(ElemVal<float, 2> a, ElemVal<float, 2> b) { return {sub2(a.v, b.v)}; }
+__device__ __forceinline__ ElemVal<float, 2> ev_mul(ElemVal<float, 2> a, float b) { return {mul2(a.v, bc2(b))}; }
+__device__ __forceinline__ ElemVal<float, 2> ev_fma(ElemVal<float, 2> a, float b, ElemVal<float, 2> c) { return {fma2(a.v, bc2(b), c.v)}; }
+__device__ __forceinline__ ElemVal<float, 2> ev_fmv(ElemVal<float, 2> a, ElemVal<float, 2> b, ElemVal<float, 2> c) { return {fma2(a.v, b.v, c.v)}; }
+
+// One thread per (element, NC adjacent cases).  TWO: M acts on pm, K on pk.  I: index type of the vector offsets.
+// The global FP32 atomics bound it (0.6e12 scalar adds a second): a pair of cases adds its two sums as one
+// 8-byte atomic.  386,370 tets, FP32, 8 cases: 63.6 -> 57.8 us with pairs and without the separate Dirichlet pass
+// (four cases a thread with 16-byte atomics: no faster than one).
+template <typename T, int NC, bool TWO, bool DOT, typename I>
+__global__ void __launch_bounds__(kBlock) k_ebe_atomic(MeshView m, int rpad, int gshift, const T* __restrict__ pm,
                                                        const T* __restrict__ pk, T* __restrict__ q, T aM, T aK,
                                                        Reducer red, CgCase* sc, double* ptq_out,
                                                        const int* gate_active) {
   if (gate_active && *gate_active == 0) return;
+  using E = ElemVal<T, NC>;
   const T* __restrict__ rec = rec_of<T>(m);
-  T dot = 0;
-  const int64_t total = m.E << rshift;
+  E dot = E::zero();
+  const int64_t total = m.E << gshift;      // gshift: log2 of the case groups of a node, rpad / NC
+  const int c = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) & ((1 << gshift) - 1)) * NC;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t e = i >> rshift;
-    const int c = (int)(i & (rpad - 1));
+    const int64_t e = i >> gshift;
     const int4 cn = __ldg(m.conn + e);
-    const int64_t nd[4] = {cn.x, cn.y, cn.z, cn.w};
+    const int nd[4] = {cn.x, cn.y, cn.z, cn.w};
+    I off[4];
+    E P[4][3], PK[4][3];
+    int fr[4];
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+      off[a] = (I)nd[a] * (I)(3 * rpad) + (I)c;
+      fr[a] = m.freemask[nd[a]];
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        P[a][k] = E::load(pm + off[a] + (I)(k * rpad));
+        PK[a][k] = TWO ? E::load(pk + off[a] + (I)(k * rpad)) : P[a][k];
+      }
+    }
     const T* re = rec + e * kRec;
     T g[9];
 #pragma unroll
     for (int j = 0; j < 9; ++j) g[j] = re[j];
     const T lam = aK * re[9], mu = aK * re[10], ms = aM * re[11];
-    T P[4][3], PK[4][3];
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        P[a][k] = pm[(nd[a] * 3 + k) * rpad + c];
-        PK[a][k] = TWO ? pk[(nd[a] * 3 + k) * rpad + c] : P[a][k];
-      }
     // displacement gradient G_ij = sum_{b=1..3} (p_b - p_0)_i g_b,j
-    T G[3][3];
+    E G[3][3];
 #pragma unroll
     for (int i2 = 0; i2 < 3; ++i2) {
-      const T d1 = PK[1][i2] - PK[0][i2], d2 = PK[2][i2] - PK[0][i2], d3 = PK[3][i2] - PK[0][i2];
+      const E d1 = ev_sub(PK[1][i2], PK[0][i2]), d2 = ev_sub(PK[2][i2], PK[0][i2]), d3 = ev_sub(PK[3][i2], PK[0][i2]);
 #pragma unroll
-      for (int j = 0; j < 3; ++j) G[i2][j] = d1 * g[j] + d2 * g[3 + j] + d3 * g[6 + j];
+      for (int j = 0; j < 3; ++j) G[i2][j] = ev_fma(d3, g[6 + j], ev_fma(d2, g[3 + j], ev_mul(d1, g[j])));
     }
-    const T tr = G[0][0] + G[1][1] + G[2][2];
-    T S[3][3];
+    const E ltr = ev_mul(ev_add(ev_add(G[0][0], G[1][1]), G[2][2]), lam);
+    E S[3][3];
     const T mu2 = mu + mu;
 #pragma unroll
-    for (int i2 = 0; i2 < 3; ++i2) S[i2][i2] = lam * tr + mu2 * G[i2][i2];
-    S[0][1] = S[1][0] = mu * (G[0][1] + G[1][0]);
-    S[0][2] = S[2][0] = mu * (G[0][2] + G[2][0]);
-    S[1][2] = S[2][1] = mu * (G[1][2] + G[2][1]);
-    T Q[4][3];
+    for (int i2 = 0; i2 < 3; ++i2) S[i2][i2] = ev_fma(G[i2][i2], mu2, ltr);
+    S[0][1] = S[1][0] = ev_mul(ev_add(G[0][1], G[1][0]), mu);
+    S[0][2] = S[2][0] = ev_mul(ev_add(G[0][2], G[2][0]), mu);
+    S[1][2] = S[2][1] = ev_mul(ev_add(G[1][2], G[2][1]), mu);
+    E Q[4][3];
 #pragma unroll
     for (int b = 1; b < 4; ++b)
 #pragma unroll
       for (int i2 = 0; i2 < 3; ++i2)
-        Q[b][i2] = S[i2][0] * g[(b - 1) * 3 + 0] + S[i2][1] * g[(b - 1) * 3 + 1] + S[i2][2] * g[(b - 1) * 3 + 2];
-#pragma unroll
-    for (int i2 = 0; i2 < 3; ++i2) Q[0][i2] = -(Q[1][i2] + Q[2][i2] + Q[3][i2]);
+        Q[b][i2] = ev_fma(S[i2][2], g[(b - 1) * 3 + 2], ev_fma(S[i2][1], g[(b - 1) * 3 + 1], ev_mul(S[i2][0], g[(b - 1) * 3])));
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-      const T sum = P[0][k] + P[1][k] + P[2][k] + P[3][k];
+      const E fs = ev_add(ev_add(Q[1][k], Q[2][k]), Q[3][k]);
+      const E sum = ev_add(ev_add(P[0][k], P[1][k]), ev_add(P[2][k], P[3][k]));
+      Q[0][k] = ev_sub(ev_mul(ev_add(P[0][k], sum), ms), fs);
 #pragma unroll
-      for (int a = 0; a < 4; ++a) Q[a][k] += ms * (P[a][k] + sum);
+      for (int a = 1; a < 4; ++a) Q[a][k] = ev_fma(ev_add(P[a][k], sum), ms, Q[a][k]);
     }
 #pragma unroll
     for (int a = 0; a < 4; ++a)
 #pragma unroll
       for (int k = 0; k < 3; ++k) {
-        if (DOT) dot += P[a][k] * Q[a][k];
-        atomicAdd(q + (nd[a] * 3 + k) * rpad + c, Q[a][k]);
+        if (DOT) dot = ev_fmv(P[a][k], Q[a][k], dot);
+        if (dof_free((uint8_t)fr[a], k)) Q[a][k].add_to(q + off[a] + (I)(k * rpad));
       }
   }
-  if (DOT) {
-    double v[1] = {(double)dot};
+  if constexpr (DOT) {
+    static_assert(NC == 1, "a thread's sum belongs to one case");
+    double v[1] = {(double)dot.v};
     if (block_reduce_last<1>(v, rpad, red)) ebe_tail(red, sc, ptq_out, rpad);
   }
+}
+
+template <typename T, int NC>
+static cudaError_t ebe_atomic_nc(const MeshView& m, int rpad, const T* pm, const T* pk, T* q, T aM, T aK,
+                                 const Reducer* red, CgCase* sc, double* ptq_out, const int* gate, cudaStream_t s) {
+  const int gs = log2i(rpad / NC);
+  // Small meshes: blocks small enough that the items cover the SMs twice (3072 tets, one case: 96 blocks of a
+  // warp instead of 12 of 256 threads; FP64 product 12.5 us), but of at least 8 rpad threads, so that the last
+  // block of the p^T q reduction has eight threads a case.
+  const int64_t items = m.E << gs;
+  int block = kBlock;
+  while (block > 32 && block > 8 * rpad && items < (int64_t)block * 2 * sm_count()) block >>= 1;
+  const int cap = red ? vec_grid_cap() * (kBlock / block) : red_grid_cap();
+  int64_t grid = (items + block - 1) / block;
+  if (grid > std::min(cap, kMaxRedBlocks)) grid = std::min(cap, kMaxRedBlocks);
+  const Reducer rd = red ? *red : Reducer{nullptr, nullptr, nullptr};
+  const bool i32 = m.N * 3 * rpad < ((int64_t)1 << 31);
+  auto run = [&](auto kfn) {
+    kfn<<<(int)grid, block, 0, s>>>(m, rpad, gs, pm, pk ? pk : pm, q, aM, aK, rd, red ? sc : nullptr,
+                                    red ? ptq_out : nullptr, gate);
+    return cudaGetLastError();
+  };
+  if (pk) {
+    if constexpr (NC == 1) return i32 ? run(k_ebe_atomic<T, 1, true, false, int32_t>) : run(k_ebe_atomic<T, 1, true, false, int64_t>);
+    return cudaErrorInvalidValue;
+  }
+  if (red) {
+    if constexpr (NC == 1) return i32 ? run(k_ebe_atomic<T, 1, false, true, int32_t>) : run(k_ebe_atomic<T, 1, false, true, int64_t>);
+    return cudaErrorInvalidValue;
+  }
+  return i32 ? run(k_ebe_atomic<T, NC, false, false, int32_t>) : run(k_ebe_atomic<T, NC, false, false, int64_t>);
 }
 
 template <typename T>
@@ -124,17 +202,13 @@ cudaError_t launch_ebe_gated(const MeshView& m, int rpad, const T* pm, const T* 
                              const Reducer* red, CgCase* sc, double* ptq_out, const int* gate, cudaStream_t s) {
   cudaError_t err = cudaMemsetAsync(q, 0, sizeof(T) * (size_t)m.N * 3 * rpad, s);
   if (err != cudaSuccess) return err;
-  const int rs = log2i(rpad);
-  const int grid = grid_for(m.E << rs, red ? vec_grid_cap() : red_grid_cap());
-  Reducer rd = red ? *red : Reducer{nullptr, nullptr, nullptr};
-  if (pk) {
-    k_ebe_atomic<T, true, false><<<grid, kBlock, 0, s>>>(m, rpad, rs, pm, pk, q, (T)aM, (T)aK, rd, nullptr, nullptr, gate);
-  } else if (red) {
-    k_ebe_atomic<T, false, true><<<grid, kBlock, 0, s>>>(m, rpad, rs, pm, pm, q, (T)aM, (T)aK, rd, sc, ptq_out, gate);
-  } else {
-    k_ebe_atomic<T, false, false><<<grid, kBlock, 0, s>>>(m, rpad, rs, pm, pm, q, (T)aM, (T)aK, rd, nullptr, nullptr, gate);
+  if constexpr (sizeof(T) == 4) {
+    // Pairs of cases where two are adjacent and their 8-byte accesses aligned.  Not with p^T q, whose FP32 sum of a
+    // thread runs over all its elements: one case a thread keeps the same elements in each sum, in the same order.
+    if (!pk && !red && rpad >= 2 && ((reinterpret_cast<uintptr_t>(pm) | reinterpret_cast<uintptr_t>(q)) & 7) == 0)
+      return ebe_atomic_nc<T, 2>(m, rpad, pm, pk, q, (T)aM, (T)aK, red, sc, ptq_out, gate, s);
   }
-  return cudaGetLastError();
+  return ebe_atomic_nc<T, 1>(m, rpad, pm, pk, q, (T)aM, (T)aK, red, sc, ptq_out, gate, s);
 }
 
 template <typename T>
@@ -485,16 +559,19 @@ cudaError_t launch_ebe_hex(const HexTiles& ht, const MeshView& m, int rpad, cons
   const int nsm = sm_count();
   int per_sm = 1;
   auto kfn = red ? (m.seg ? k_ebe_hex<T, true, true> : k_ebe_hex<T, true, false>) : k_ebe_hex<T, false, false>;
+  // one thread an item (hex, case) of a tile, at most kBlock: small tiles of one or two cases take small blocks
+  int block = kBlock;
+  while (block > 32 && block / 2 >= ht.hex_per_tile * rpad) block >>= 1;
   err = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (err == cudaSuccess) err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kfn, kBlock, smem);
+  if (err == cudaSuccess) err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kfn, block, smem);
   if (err != cudaSuccess) return err;
   if (per_sm < 1) per_sm = 1;
   int grid = nsm * per_sm;
   if (grid > ht.n_tiles) grid = ht.n_tiles;
   if (grid > red_grid_cap()) grid = red_grid_cap();
   Reducer rd = red ? *red : Reducer{nullptr, nullptr, nullptr};
-  kfn<<<grid, kBlock, smem, s>>>(ht, m, rpad, rs, p, q, (T)aM, (T)aK, rd, red ? sc : nullptr, red ? ptq_out : nullptr,
-                                 gate);
+  kfn<<<grid, block, smem, s>>>(ht, m, rpad, rs, p, q, (T)aM, (T)aK, rd, red ? sc : nullptr, red ? ptq_out : nullptr,
+                                gate);
   return cudaGetLastError();
 }
 template cudaError_t launch_ebe_hex<double>(const HexTiles&, const MeshView&, int, const double*, double*, double,
@@ -527,12 +604,6 @@ template <> struct SVec4<double> {
 // Two cases per thread on Blackwell's paired FP32 pipe operations (one instruction, two lanes of values):
 // the cases of a node are adjacent in memory, so a pair loads as one float2 and every operation of the
 // element arithmetic is the same for both; the element records are shared and broadcast to both halves.
-__device__ __forceinline__ float2 bc2(float v) { return make_float2(v, v); }
-__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
-
 // The tet_acc arithmetic for a pair of cases.
 template <int A0, int A1, int A2, int A3>
 __device__ __forceinline__ void tet_acc_p(const float* re, float aM, float aK, const float2 (&P)[8][3],

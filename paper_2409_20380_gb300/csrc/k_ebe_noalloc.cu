@@ -91,11 +91,9 @@ extern "C" fem_status fem_ebe_apply_noalloc(fem_mesh* m, int precision, const vo
   } else if (precision == FEM_FP64) {
     e = launch_ebe<double>(mv, n_rhs, (const double*)p_dev, nullptr, (double*)q_dev, alpha_M, alpha_K,
                            ptq_dev ? &red : nullptr, nullptr, ptq_dev, s);
-    if (e == cudaSuccess) e = launch_mask<double>(mv.N, n_rhs, mv.freemask, (double*)q_dev, s);
   } else {
     e = launch_ebe<float>(mv, n_rhs, (const float*)p_dev, nullptr, (float*)q_dev, alpha_M, alpha_K,
                           ptq_dev ? &red : nullptr, nullptr, ptq_dev, s);
-    if (e == cudaSuccess) e = launch_mask<float>(mv.N, n_rhs, mv.freemask, (float*)q_dev, s);
   }
   if (e != cudaSuccess) return set_error(FEM_ERR_CUDA, std::string("fem_ebe_apply_noalloc: ") + cudaGetErrorString(e));
   return FEM_OK;
