@@ -39,235 +39,316 @@ __device__ __forceinline__ float gelu_grad_f(float z) {
 }
 
 // ------------------------------------------------------------------------------------------------------
-// C = A B^T on the tensor cores.  A [M][K] and B [N][K] are BF16 with K contiguous; FP32 accumulation.
-// M % 64 == 0, N % 32 == 0, K % 32 == 0, lda/ldb % 8 == 0 (16-byte rows of the staged tiles).  A CTA of
-// 4 warps computes a 64 x 32 tile; warp w owns rows 16w..16w+15 and all 32 columns (4 m16n8 tiles).
-// With gridDim.z > 1 (split contraction, plain epilogue only) CTA z sums its share of K and adds it into C,
-// which the caller has zeroed.
+// The network on the tensor cores (BF16 mma.sync m16n8k16, FP32 accumulation).  Everything but the weight
+// gradients is local to a sample, so one kernel takes a block of kRows samples through the forward pass, the
+// loss and the backward pass with the activations in shared memory and the GELU derivatives in registers (a
+// thread owns the same entries of a layer on the way forward and back), and a second kernel forms the three
+// weight gradients.  What bounds both is latency (2.2 GFLOP a training pass at 4096 samples, ~2 us of tensor
+// time), so passes and launches are what is saved: 4096 samples took 246 us in 13 launches (three column sums of
+// 60 us on 1 to 8 blocks among them), and take 47 us in 2 launches now (66,560 samples: 3332 -> 331 us; forward
+// alone at 4096: 37 -> 10 us).  32 samples a block (128 blocks at 4096) leave the
+// tensor cores mostly idle either way; tcgen05's smallest tile (128 rows) would leave 120 of 152 SMs without work.
+// Weights come straight from L2 in the order of the MMA's B fragments (k_pack): 16 bytes a lane cover 32 of K
+// for 8 output columns, so no shared-memory staging and no barrier between K steps.
 // ------------------------------------------------------------------------------------------------------
-enum { EPI_BIAS = 0, EPI_GELU = 1, EPI_GELU_BWD = 2, EPI_PLAIN = 3 };
+constexpr int kRows = 32;                      // samples a block (two m16 tiles)
+constexpr int kMlpBlock = 256;                 // 8 warps: 32 of a layer's 256 columns each
+constexpr int kSX = kL0 + 8, kSA = kL1 + 8, kSD = kL3 + 8;   // padded rows (16 bytes mod 128: conflict-free ldmatrix)
 
-struct GemmArgs {
-  int M, N, K;
-  const bf16* A;
-  int lda;
-  const bf16* B;
-  int ldb;
-  float* C;            // optional FP32 output C[m * c_rs + n * c_cs]
-  int64_t c_rs, c_cs;
-  const float* bias;   // [N] (EPI_BIAS, EPI_GELU)
-  const float* zin;    // pre-activation zin[m * ldz + n] (EPI_GELU_BWD)
-  int ldz;
-  bf16* act;           // optional BF16 output act[m * ld_act + n]
-  int ld_act;
-  bf16* actT;          // optional BF16 output actT[n * ld_actT + m]
-  int ld_actT;
-  int m_valid;         // EPI_GELU_BWD: rows >= m_valid are written as zero
-};
-
-__device__ __forceinline__ void mma_bf16_16816(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
-                                               uint32_t b0, uint32_t b1) {
+__device__ __forceinline__ void mma_bf16_16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
   asm volatile(
       "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
       "{%0,%1,%2,%3};\n"
       : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], const bf16* p) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"((uint32_t)__cvta_generic_to_shared(p)));
+}
+__device__ __forceinline__ void ldsm4t(uint32_t (&r)[4], const bf16* p) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"((uint32_t)__cvta_generic_to_shared(p)));
 }
 
-template <int EPI>
-__global__ void __launch_bounds__(128) k_gemm_tn(GemmArgs g) {
-  __shared__ __align__(16) bf16 As[64][40];   // 80-byte rows: 16-byte aligned, conflict-free fragment reads
-  __shared__ __align__(16) bf16 Bs[32][40];
-  const int m0 = blockIdx.x * 64, n0 = blockIdx.y * 32;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, gq = lane >> 2, tq = lane & 3;
-  float acc[4][4];
+// acc[mt][j] = rows 16 mt .. +15 of A (shared, row stride ld) times 8 columns nt0 + j of the packed weights P.
+template <int K, int MT, int NT>
+__device__ __forceinline__ void layer_mma(const bf16* A, int ld, const uint4* __restrict__ P, int nt0,
+                                          float (&acc)[MT][NT][4]) {
+  const int lane = threadIdx.x & 31;
+  const bf16* a0 = A + (lane & 15) * ld + (lane >> 4) * 8;
 #pragma unroll
-  for (int j = 0; j < 4; ++j)
+  for (int m = 0; m < MT; ++m)
 #pragma unroll
-    for (int e = 0; e < 4; ++e) acc[j][e] = 0.0f;
-  const int kper = g.K / (int)gridDim.z, kbeg = (int)blockIdx.z * kper;
-  for (int k0 = kbeg; k0 < kbeg + kper; k0 += 32) {
+    for (int j = 0; j < NT; ++j)
 #pragma unroll
-    for (int v = tid; v < 256; v += 128) {
-      const int r = v >> 2, cv = (v & 3) * 8;
-      *reinterpret_cast<uint4*>(&As[r][cv]) =
-          *reinterpret_cast<const uint4*>(g.A + (int64_t)(m0 + r) * g.lda + k0 + cv);
-    }
-    {
-      const int r = tid >> 2, cv = (tid & 3) * 8;
-      *reinterpret_cast<uint4*>(&Bs[r][cv]) =
-          *reinterpret_cast<const uint4*>(g.B + (int64_t)(n0 + r) * g.ldb + k0 + cv);
-    }
-    __syncthreads();
+      for (int e = 0; e < 4; ++e) acc[m][j][e] = 0.0f;
 #pragma unroll
-    for (int kk = 0; kk < 32; kk += 16) {
-      const int ar = warp * 16 + gq;
-      const uint32_t a0 = *reinterpret_cast<const uint32_t*>(&As[ar][kk + tq * 2]);
-      const uint32_t a1 = *reinterpret_cast<const uint32_t*>(&As[ar + 8][kk + tq * 2]);
-      const uint32_t a2 = *reinterpret_cast<const uint32_t*>(&As[ar][kk + 8 + tq * 2]);
-      const uint32_t a3 = *reinterpret_cast<const uint32_t*>(&As[ar + 8][kk + 8 + tq * 2]);
+  for (int kp = 0; kp < K / 32; ++kp) {
+    uint4 b[NT];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const uint32_t b0 = *reinterpret_cast<const uint32_t*>(&Bs[j * 8 + gq][kk + tq * 2]);
-        const uint32_t b1 = *reinterpret_cast<const uint32_t*>(&Bs[j * 8 + gq][kk + 8 + tq * 2]);
-        mma_bf16_16816(acc[j], a0, a1, a2, a3, b0, b1);
+    for (int j = 0; j < NT; ++j) b[j] = __ldg(P + ((nt0 + j) * (K / 32) + kp) * 32 + lane);
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int m = 0; m < MT; ++m) {
+        uint32_t a[4];
+        ldsm4(a, a0 + m * 16 * ld + kp * 32 + h * 16);
+#pragma unroll
+        for (int j = 0; j < NT; ++j) mma_bf16_16816(acc[m][j], a, h ? b[j].z : b[j].x, h ? b[j].w : b[j].y);
       }
-    }
-    __syncthreads();
   }
-  // accumulator (j, e): row gq + 8 (e >> 1) of the warp's 16, column 8 j + 2 tq + (e & 1)
+}
+
+struct MlpPass {
+  const float* x;          // [n_src][64]
+  const int32_t* idx;      // rows of the batch (null: row r is sample r)
+  int64_t n_src, B, Mpad;  // samples, rows of the batch, rows of the workspace (multiple of kRows)
+  const uint4 *P1, *P2, *P3, *P3T, *P2T;   // packed weights
+  const float* th;         // FP32 parameters (biases)
+  int* bad;                // set where a sample index is out of range (the row is zero)
+  float* out;              // forward only: [B][32]
+  const float* t;          // training: [n_src][32] targets, or residual-space samples [n_src][kNRes]
+  bf16 *X0, *A1, *A2, *dZ1, *dZ2, *dZ3;    // training: row-major, for the weight gradients
+  float* grad;             // training: bias gradients are added here (the caller has zeroed it)
+  double* loss;
+};
+
+// entry (mt, j, e) of a thread's accumulators: row 16 mt + gq + 8 (e >> 1), column 32 warp + 8 j + 2 tq + (e & 1)
+template <int MODE>   // 0 forward only, 1 training (mean squared error), 2 training (residual space)
+__global__ void __launch_bounds__(kMlpBlock) k_mlp_pass(MlpPass g) {
+  __shared__ __align__(16) bf16 sX[kRows * kSX];
+  __shared__ __align__(16) bf16 sA[kRows * kSA];     // A1, then dZ1
+  __shared__ __align__(16) bf16 sB[kRows * kSA];     // A2, then dZ2
+  __shared__ __align__(16) bf16 sD[kRows * kSD];     // dZ3
+  __shared__ float sO[kRows][kL3 + 1];
+  __shared__ float sr[kMlpBlock / 32][kL3];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, gq = lane >> 2, tq = lane & 3;
+  const int64_t row0 = (int64_t)blockIdx.x * kRows;
+  auto sample = [&](int r) -> int64_t {   // source row of batch row row0 + r, -1: none
+    const int64_t b = row0 + r;
+    if (b >= g.B) return -1;
+    const int64_t sr_ = g.idx ? (int64_t)g.idx[b] : b;
+    return sr_ >= 0 && sr_ < g.n_src ? sr_ : -1;
+  };
 #pragma unroll
-  for (int j = 0; j < 4; ++j)
+  for (int u = 0; u < kRows * kL0 / kMlpBlock; ++u) {
+    const int i = tid + u * kMlpBlock, r = i / kL0, c = i % kL0;
+    const int64_t sr_ = sample(r);
+    sX[r * kSX + c] = __float2bfloat16_rn(sr_ >= 0 ? g.x[sr_ * kL0 + c] : 0.0f);
+    if (sr_ < 0 && c == 0 && row0 + r < g.B) atomicExch(g.bad, 1);
+  }
+  __syncthreads();
+  float acc[2][4][4], g1[2][4][4], g2[2][4][4];
+  // z + bias -> GELU into dst (BF16), its derivative into gd
+  auto act = [&](const float* bias, bf16* dst, float (&gd)[2][4][4]) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int c = 32 * warp + 8 * j + 2 * tq;
+      const float b0 = __ldg(bias + c), b1 = __ldg(bias + c + 1);
+#pragma unroll
+      for (int m = 0; m < 2; ++m)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const float z0 = acc[m][j][2 * h] + b0, z1 = acc[m][j][2 * h + 1] + b1;
+          if (MODE) gd[m][j][2 * h] = gelu_grad_f(z0), gd[m][j][2 * h + 1] = gelu_grad_f(z1);
+          *reinterpret_cast<__nv_bfloat162*>(dst + (16 * m + gq + 8 * h) * kSA + c) =
+              __floats2bfloat162_rn(gelu_f(z0), gelu_f(z1));
+        }
+    }
+  };
+  // a [kRows][W] tile of shared memory to rows row0 .. of a row-major matrix, 16 bytes a thread
+  auto put = [&](const bf16* src, int ld, int W, bf16* dst) {
+    for (int i = tid; i < kRows * W / 8; i += kMlpBlock) {
+      const int r = i / (W / 8), c = (i % (W / 8)) * 8;
+      *reinterpret_cast<uint4*>(dst + (row0 + r) * W + c) = *reinterpret_cast<const uint4*>(src + r * ld + c);
+    }
+  };
+  layer_mma<kL0, 2, 4>(sX, kSX, g.P1, 4 * warp, acc);
+  act(g.th + kOffB1, sA, g1);
+  if (MODE) put(sX, kSX, kL0, g.X0);
+  __syncthreads();
+  layer_mma<kL1, 2, 4>(sA, kSA, g.P2, 4 * warp, acc);
+  act(g.th + kOffB2, sB, g2);
+  if (MODE) put(sA, kSA, kL1, g.A1);
+  __syncthreads();
+  {   // layer 3: warp w takes rows 16 (w & 1) .. and columns 8 (w >> 1) ..
+    float o[1][1][4];
+    const int m = warp & 1, j = warp >> 1;
+    layer_mma<kL2, 1, 1>(sB + m * 16 * kSA, kSA, g.P3, j, o);
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
-      const int r = m0 + warp * 16 + gq + 8 * (e >> 1);
-      const int c = n0 + j * 8 + tq * 2 + (e & 1);
-      float v = acc[j][e];
-      float out = v, a = v;
-      if (EPI == EPI_BIAS || EPI == EPI_GELU) {
-        out = v + g.bias[c];
-        a = EPI == EPI_GELU ? gelu_f(out) : out;
-      } else if (EPI == EPI_GELU_BWD) {
-        out = r < g.m_valid ? v * gelu_grad_f(g.zin[(int64_t)r * g.ldz + c]) : 0.0f;
-        a = out;
-      }
-      if (g.C) {
-        float* dst = g.C + (int64_t)r * g.c_rs + (int64_t)c * g.c_cs;
-        if (gridDim.z > 1)
-          atomicAdd(dst, out);
-        else
-          *dst = out;
-      }
-      if (g.act) g.act[(int64_t)r * g.ld_act + c] = __float2bfloat16_rn(a);
-      if (g.actT) g.actT[(int64_t)c * g.ld_actT + r] = __float2bfloat16_rn(a);
-    }
-}
-
-template <int EPI>
-cudaError_t gemm(const GemmArgs& g, cudaStream_t s) {
-  if (g.M % 64 || g.N % 32 || g.K % 32 || g.lda % 8 || g.ldb % 8) return cudaErrorInvalidValue;
-  dim3 grid(g.M / 64, g.N / 32, 1);
-  // A contraction long against the output (the weight gradients: K = the batch) is split so that the grid
-  // covers the SMs twice, each share at least 8 of the 32-wide K steps; C (dense M x N) is zeroed first.
-  if (EPI == EPI_PLAIN && g.C && !g.act && !g.actT &&
-      ((g.c_rs == g.N && g.c_cs == 1) || (g.c_rs == 1 && g.c_cs == g.M))) {
-    const int steps = g.K / 32, tiles = (int)(grid.x * grid.y), want = 2 * sm_count();
-    int ks = 1;
-    for (int d = 2; d <= steps / 8 && tiles * ks < want; ++d)
-      if (steps % d == 0) ks = d;
-    if (ks > 1) {
-      cudaError_t e = cudaMemsetAsync(g.C, 0, sizeof(float) * (size_t)g.M * g.N, s);
-      if (e != cudaSuccess) return e;
-      grid.z = ks;
+      const int r = 16 * m + gq + 8 * (e >> 1), c = 8 * j + 2 * tq + (e & 1);
+      sO[r][c] = o[0][0][e] + __ldg(g.th + kOffB3 + c);
     }
   }
-  k_gemm_tn<EPI><<<grid, 128, 0, s>>>(g);
-  return cudaGetLastError();
-}
-
-GemmArgs gargs(int M, int N, int K, const bf16* A, int lda, const bf16* B, int ldb) {
-  GemmArgs g{};
-  g.M = M, g.N = N, g.K = K, g.A = A, g.lda = lda, g.B = B, g.ldb = ldb;
-  g.m_valid = M;
-  return g;
-}
-
-// x rows (optionally gathered through idx) -> BF16 [Mpad][64] and its transpose [64][Mpad]; pad rows zero.
-__global__ void k_stage(const float* __restrict__ x, const int32_t* __restrict__ idx, int64_t n_src, int64_t B,
-                        int64_t Mpad, bf16* __restrict__ X0, bf16* __restrict__ X0T, int* __restrict__ bad) {
-  const int64_t total = Mpad * kL0;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t r = i / kL0;
-    const int c = (int)(i % kL0);
-    float v = 0.0f;
-    if (r < B) {
-      const int64_t sr = idx ? (int64_t)idx[r] : r;
-      if (sr >= 0 && sr < n_src)
-        v = x[sr * kL0 + c];
-      else if (c == 0)
-        atomicExch(bad, 1);     // sample index outside [0, n_src): the row is zero, the call reports it
+  if (MODE) put(sB, kSA, kL2, g.A2);
+  __syncthreads();
+  if (MODE == 0) {
+    for (int i = tid; i < kRows * kL3; i += kMlpBlock) {
+      const int r = i / kL3, c = i % kL3;
+      if (row0 + r < g.B) g.out[(row0 + r) * kL3 + c] = sO[r][c];
     }
-    const bf16 b = __float2bfloat16_rn(v);
-    X0[i] = b;
-    if (X0T) X0T[(int64_t)c * Mpad + r] = b;
+    return;
   }
-}
-
-// dL/dout of the mean squared error, in FP32 and BF16 (row-major and transposed); pad rows zero.
-__global__ void k_loss(const float* __restrict__ out, const float* __restrict__ t, const int32_t* __restrict__ idx,
-                       int64_t n_src, int64_t B, int64_t Mpad, float* __restrict__ dzf, bf16* __restrict__ dzb,
-                       bf16* __restrict__ dzT, double* __restrict__ loss_acc) {
-  const float scale = 2.0f / ((float)B * kL3);
+  // loss and dL/dout: a warp takes four rows, a lane one output; sO becomes dL/dout in FP32
   double sq = 0.0;
-  const int64_t total = Mpad * kL3;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t r = i / kL3;
-    const int j = (int)(i % kL3);
+#pragma unroll
+  for (int u = 0; u < kRows / 8; ++u) {
+    const int r = warp * (kRows / 8) + u;
+    const int64_t sr_ = sample(r);
     float d = 0.0f;
-    const int64_t sr = r < B ? (idx ? (int64_t)idx[r] : r) : -1;
-    if (sr >= 0 && sr < n_src) {
-      const float diff = out[i] - t[sr * kL3 + j];
-      d = scale * diff;
-      sq += (double)diff * diff;
-    }
-    dzf[i] = d;
-    dzb[i] = __float2bfloat16_rn(d);
-    dzT[(int64_t)j * Mpad + r] = __float2bfloat16_rn(d);
-  }
-  for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
-  if ((threadIdx.x & 31) == 0 && sq != 0.0) atomicAdd(loss_acc, sq);
-}
-
-// dL/dout of the residual-space loss, one warp per row: with the row's sample (W upper triangular, w),
-// r = W d - w, loss += ||r||^2, dL/dd = 2 W^T r / B; FP32 and BF16 (row-major and transposed); pad rows zero.
-__global__ void __launch_bounds__(256) k_loss_res(const float* __restrict__ out, const float* __restrict__ smp,
-                                                  const int32_t* __restrict__ idx, int64_t n_src, int64_t B,
-                                                  int64_t Mpad, float* __restrict__ dzf, bf16* __restrict__ dzb,
-                                                  bf16* __restrict__ dzT, double* __restrict__ loss_acc) {
-  __shared__ float sd[8][kL3], sr[8][kL3];
-  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-  const float scale = 2.0f / (float)B;
-  for (int64_t r = (int64_t)blockIdx.x * 8 + wp; r < Mpad; r += (int64_t)gridDim.x * 8) {
-    const int64_t sr_ = r < B ? (idx ? (int64_t)idx[r] : r) : -1;
-    const bool valid = sr_ >= 0 && sr_ < n_src;
-    float g = 0.0f;
-    if (valid) {
-      const float* S = smp + sr_ * kNRes;
-      sd[wp][lane] = out[r * kL3 + lane];
-      __syncwarp();
-      // r_i = sum_{j >= i} W_ij d_j - w_i  (lane i; row i of the packed triangle starts at 32 i - i (i - 1) / 2)
+    if (MODE == 1) {
+      if (sr_ >= 0) {
+        const float scale = 2.0f / ((float)g.B * kL3);
+        const float diff = sO[r][lane] - g.t[sr_ * kL3 + lane];
+        d = scale * diff;
+        sq += (double)diff * diff;
+      }
+    } else if (sr_ >= 0) {
+      // residual space: with the row's sample (W upper triangular, w), r = W d - w, loss += ||r||^2,
+      // dL/dd = 2 W^T r / B (row i of the packed triangle starts at 32 i - i (i - 1) / 2)
+      const float* S = g.t + sr_ * kNRes;
       const int off = lane * kL3 - lane * (lane - 1) / 2;
       float ri = -S[kNTri + lane];
-      for (int j = lane; j < kL3; ++j) ri = fmaf(S[off + j - lane], sd[wp][j], ri);
-      sr[wp][lane] = ri;
-      double sq = (double)ri * ri;
-      for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
-      if (lane == 0) atomicAdd(loss_acc, sq);
+      for (int j = lane; j < kL3; ++j) ri = fmaf(S[off + j - lane], sO[r][j], ri);
       __syncwarp();
-      // g_j = scale sum_{i <= j} W_ij r_i  (lane j)
-      for (int i = 0; i <= lane; ++i) g = fmaf(S[i * kL3 - i * (i - 1) / 2 + lane - i], sr[wp][i], g);
-      g *= scale;
+      sr[warp][lane] = ri;
+      sq += (double)ri * ri;
+      __syncwarp();
+      for (int i = 0; i <= lane; ++i) d = fmaf(S[i * kL3 - i * (i - 1) / 2 + lane - i], sr[warp][i], d);
+      d *= 2.0f / (float)g.B;
       __syncwarp();
     }
-    dzf[r * kL3 + lane] = g;
-    dzb[r * kL3 + lane] = __float2bfloat16_rn(g);
-    dzT[(int64_t)lane * Mpad + r] = __float2bfloat16_rn(g);
+    sO[r][lane] = d;
+    sD[r * kSD + lane] = __float2bfloat16_rn(d);
   }
+  for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+  if (lane == 0 && sq != 0.0) atomicAdd(g.loss, sq);
+  __syncthreads();
+  if (warp == 0) {
+    float c = 0.0f;
+#pragma unroll 8
+    for (int r = 0; r < kRows; ++r) c += sO[r][lane];
+    atomicAdd(g.grad + kOffB3 + lane, c);
+  }
+  put(sD, kSD, kL3, g.dZ3);
+  // dZ = (dZ_next W) * GELU'(Z): BF16 into dst, the FP32 column sums (bias gradient) into gb
+  auto back = [&](const float (&gd)[2][4][4], bf16* dst, float* gb) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int c = 32 * warp + 8 * j + 2 * tq;
+      float s0 = 0.0f, s1 = 0.0f;
+#pragma unroll
+      for (int m = 0; m < 2; ++m)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const float v0 = acc[m][j][2 * h] * gd[m][j][2 * h], v1 = acc[m][j][2 * h + 1] * gd[m][j][2 * h + 1];
+          s0 += v0, s1 += v1;
+          *reinterpret_cast<__nv_bfloat162*>(dst + (16 * m + gq + 8 * h) * kSA + c) = __floats2bfloat162_rn(v0, v1);
+        }
+#pragma unroll
+      for (int o = 4; o < 32; o <<= 1) {
+        s0 += __shfl_xor_sync(0xffffffffu, s0, o);
+        s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+      }
+      if (gq == 0) {
+        atomicAdd(gb + c, s0);
+        atomicAdd(gb + c + 1, s1);
+      }
+    }
+  };
+  layer_mma<kL3, 2, 4>(sD, kSD, g.P3T, 4 * warp, acc);
+  back(g2, sB, g.grad + kOffB2);      // (rows past the batch have dL/dout = 0, so their dZ is zero)
+  __syncthreads();
+  put(sB, kSA, kL2, g.dZ2);
+  layer_mma<kL2, 2, 4>(sB, kSA, g.P2T, 4 * warp, acc);
+  back(g1, sA, g.grad + kOffB1);
+  __syncthreads();
+  put(sA, kSA, kL1, g.dZ1);
 }
 
-// Bias gradient: column sums of dz [Mpad][N] (fixed order: deterministic).
-__global__ void k_colsum(const float* __restrict__ dz, int64_t Mpad, int N, float* __restrict__ out) {
-  __shared__ float part[8][33];
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  const int c = blockIdx.x * 32 + tx;
-  float s = 0.0f;
-  for (int64_t r = ty; r < Mpad; r += 8) s += dz[r * N + c];
-  part[ty][tx] = s;
-  __syncthreads();
-  if (ty == 0) {
-    float t = 0.0f;
-    for (int k = 0; k < 8; ++k) t += part[k][tx];
-    out[c] = t;
+// Weight gradients: C[m][n] += sum_b P[b][m] Q[b][n] over the batch rows b, 64 x 64 tiles of the three outputs
+// (dW2 = dZ2^T A1: 16 tiles; dW1 = dZ1^T X0: 4; dW3 = dZ3^T A2, as its transpose A2^T dZ3 with 32 columns: 4),
+// each with its batch split over gridDim.y blocks that add into the zeroed gradient (so that the grid covers the
+// SMs twice).  Both operands lie row-major by sample: ldmatrix.trans turns them.  A block stages 32 samples at a
+// time, double-buffered by cp.async.
+constexpr int kWgStride = 72;                  // BF16 values a staged row of 64 (144 bytes: conflict-free)
+struct MlpWgrad {
+  const bf16 *X0, *A1, *A2, *dZ1, *dZ2, *dZ3;
+  float* grad;
+  int steps;                                   // batch rows / 32
+};
+__global__ void __launch_bounds__(128) k_mlp_wgrad(MlpWgrad g) {
+  __shared__ __align__(16) bf16 sP[2][32 * kWgStride], sQ[2][32 * kWgStride];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, gq = lane >> 2, tq = lane & 3;
+  const int tile = blockIdx.x;
+  const bf16 *P, *Q;
+  float* C;
+  int ldp, ldq, nq = 64, rs, cs;               // C[m * rs + n * cs]
+  if (tile < 16) {
+    P = g.dZ2 + (tile >> 2) * 64, Q = g.A1 + (tile & 3) * 64, ldp = kL2, ldq = kL1, rs = kL1, cs = 1;
+    C = g.grad + kOffW2 + (tile >> 2) * 64 * kL1 + (tile & 3) * 64;
+  } else if (tile < 20) {
+    P = g.dZ1 + (tile - 16) * 64, Q = g.X0, ldp = kL1, ldq = kL0, rs = kL0, cs = 1;
+    C = g.grad + kOffW1 + (tile - 16) * 64 * kL0;
+  } else {
+    P = g.A2 + (tile - 20) * 64, Q = g.dZ3, ldp = kL2, ldq = kL3, nq = 32, rs = 1, cs = kL2;
+    C = g.grad + kOffW3 + (tile - 20) * 64;
+  }
+  const int k0 = (int)((int64_t)g.steps * blockIdx.y / gridDim.y), k1 = (int)((int64_t)g.steps * (blockIdx.y + 1) / gridDim.y);
+  auto cp16 = [](bf16* dst, const bf16* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+  };
+  auto stage = [&](int k, int b) {
+    const int64_t r0 = (int64_t)k * 32;
+    for (int i = tid; i < 32 * 8; i += 128) {
+      const int r = i >> 3, c = (i & 7) * 8;
+      cp16(sP[b] + r * kWgStride + c, P + (r0 + r) * ldp + c);
+      if (c < nq) cp16(sQ[b] + r * kWgStride + c, Q + (r0 + r) * ldq + c);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  float acc[8][4];
+#pragma unroll
+  for (int j = 0; j < 8; ++j)
+#pragma unroll
+    for (int e = 0; e < 4; ++e) acc[j][e] = 0.0f;
+  if (k0 < k1) stage(k0, 0);
+  const int mi = lane >> 3, lr = lane & 7;
+  for (int k = k0; k < k1; ++k) {
+    const int b = (k - k0) & 1;
+    if (k + 1 < k1) {
+      stage(k + 1, b ^ 1);
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+    } else {
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+    }
+    __syncthreads();
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      uint32_t a[4];
+      ldsm4t(a, sP[b] + (16 * h + lr + (mi >> 1) * 8) * kWgStride + 16 * warp + (mi & 1) * 8);
+#pragma unroll
+      for (int jj = 0; jj < 4; ++jj) {
+        if (16 * jj >= nq) break;
+        uint32_t q[4];
+        ldsm4t(q, sQ[b] + (16 * h + lr + (mi & 1) * 8) * kWgStride + 16 * jj + (mi >> 1) * 8);
+        mma_bf16_16816(acc[2 * jj], a, q[0], q[1]);
+        mma_bf16_16816(acc[2 * jj + 1], a, q[2], q[3]);
+      }
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    if (8 * j >= nq) break;
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      atomicAdd(C + (16 * warp + gq + 8 * (e >> 1)) * rs + (8 * j + 2 * tq + (e & 1)) * cs, acc[j][e]);
   }
 }
 
@@ -284,25 +365,28 @@ __global__ void k_adam(float* __restrict__ th, float* __restrict__ m, float* __r
   }
 }
 
-// BF16 copies of the weight matrices used by the products: W_l [N][K] and, for the backward products,
-// W_l^T [K][N] (layers 2 and 3).
-__global__ void k_pack(const float* __restrict__ th, bf16* W1, bf16* W2, bf16* W2T, bf16* W3, bf16* W3T) {
-  const int64_t n1 = (int64_t)kL1 * kL0, n2 = (int64_t)kL2 * kL1, n3 = (int64_t)kL3 * kL2;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n1 + n2 + n3;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    if (i < n1) {
-      W1[i] = __float2bfloat16_rn(th[kOffW1 + i]);
-    } else if (i < n1 + n2) {
-      const int64_t j = i - n1, n = j / kL1, k = j % kL1;
-      const bf16 b = __float2bfloat16_rn(th[kOffW2 + j]);
-      W2[j] = b;
-      W2T[k * kL2 + n] = b;
-    } else {
-      const int64_t j = i - n1 - n2, n = j / kL2, k = j % kL2;
-      const bf16 b = __float2bfloat16_rn(th[kOffW3 + j]);
-      W3[j] = b;
-      W3T[k * kL3 + n] = b;
-    }
+// The weights in BF16 in the order of the MMA's B fragments: for output columns 8 nt .. +7 and 32 of K (kp), lane
+// (gq = lane / 4, tq = lane % 4) holds at P[(nt * K / 32 + kp) * 32 + lane] the values W[8 nt + gq][32 kp + 8 i +
+// 2 tq + {0, 1}], i = 0 .. 3.  W1, W2, W3 for the forward pass; W3^T, W2^T for the backward one.
+__global__ void k_pack(const float* __restrict__ th, bf16* P1, bf16* P2, bf16* P3, bf16* P3T, bf16* P2T) {
+  constexpr int n1 = kL1 * kL0, n2 = kL2 * kL1, n3 = kL3 * kL2;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n1 + 2 * n2 + 2 * n3; i += gridDim.x * blockDim.x) {
+    int o = i, K = kL0, n = 0, k = 0;
+    bf16* P = P1;
+    int which = 0;
+    if (o >= n1) o -= n1, which = 1, P = P2, K = kL1;
+    if (which == 1 && o >= n2) o -= n2, which = 2, P = P3, K = kL2;
+    if (which == 2 && o >= n3) o -= n3, which = 3, P = P3T, K = kL3;
+    if (which == 3 && o >= n3) o -= n3, which = 4, P = P2T, K = kL2;
+    const int v = o & 7, lane = (o >> 3) & 31, blk = o >> 8;       // 8 values a lane, 32 lanes a block
+    n = (blk / (K / 32)) * 8 + (lane >> 2);
+    k = (blk % (K / 32)) * 32 + (v >> 1) * 8 + (lane & 3) * 2 + (v & 1);
+    const int64_t src = which == 0   ? kOffW1 + n * kL0 + k
+                        : which == 1 ? kOffW2 + n * kL1 + k
+                        : which == 2 ? kOffW3 + n * kL2 + k
+                        : which == 3 ? kOffW3 + k * kL2 + n      // W3^T[n][k] = W3[k][n]
+                                     : kOffW2 + k * kL1 + n;     // W2^T[n][k] = W2[k][n]
+    P[o] = __float2bfloat16_rn(th[src]);
   }
 }
 
@@ -321,28 +405,25 @@ struct fem_mlp {
   cudaStream_t s = nullptr;
   float *th = nullptr, *m = nullptr, *v = nullptr, *grad = nullptr;
   int64_t t = 0;                       // Adam steps taken
-  bf16 *W1 = nullptr, *W2 = nullptr, *W2T = nullptr, *W3 = nullptr, *W3T = nullptr;
-  int64_t cap = 0;                     // rows of the activation workspace (multiple of 64)
-  bf16 *X0 = nullptr, *X0T = nullptr, *A1 = nullptr, *A1T = nullptr, *A2 = nullptr, *A2T = nullptr;
-  bf16 *dZ3b = nullptr, *dZ3T = nullptr, *dZ2b = nullptr, *dZ2T = nullptr, *dZ1T = nullptr;
-  float *Z1 = nullptr, *Z2 = nullptr, *OUT = nullptr, *dZ3f = nullptr, *dZ2f = nullptr, *dZ1f = nullptr;
+  bf16 *P1 = nullptr, *P2 = nullptr, *P3 = nullptr, *P3T = nullptr, *P2T = nullptr;   // packed weights (k_pack)
+  int64_t cap = 0;                     // rows of the training workspace (multiple of kRows)
+  bf16 *X0 = nullptr, *A1 = nullptr, *A2 = nullptr, *dZ1 = nullptr, *dZ2 = nullptr, *dZ3 = nullptr;
+  int64_t out_cap = 0;                 // rows of OUT
+  float* OUT = nullptr;
   double* loss_acc = nullptr;
   int* bad = nullptr;                  // set by a kernel that met a sample index out of range
   std::mutex mu;
 
   void free_ws() {
-    for (void* p : {(void*)X0, (void*)X0T, (void*)A1, (void*)A1T, (void*)A2, (void*)A2T, (void*)dZ3b, (void*)dZ3T,
-                    (void*)dZ2b, (void*)dZ2T, (void*)dZ1T, (void*)Z1, (void*)Z2, (void*)OUT, (void*)dZ3f,
-                    (void*)dZ2f, (void*)dZ1f})
+    for (void* p : {(void*)X0, (void*)A1, (void*)A2, (void*)dZ1, (void*)dZ2, (void*)dZ3})
       if (p) cudaFree(p);
-    X0 = X0T = A1 = A1T = A2 = A2T = dZ3b = dZ3T = dZ2b = dZ2T = dZ1T = nullptr;
-    Z1 = Z2 = OUT = dZ3f = dZ2f = dZ1f = nullptr;
+    X0 = A1 = A2 = dZ1 = dZ2 = dZ3 = nullptr;
     cap = 0;
   }
   ~fem_mlp() {
     free_ws();
-    for (void* p : {(void*)th, (void*)m, (void*)v, (void*)grad, (void*)W1, (void*)W2, (void*)W2T, (void*)W3,
-                    (void*)W3T, (void*)loss_acc, (void*)bad})
+    for (void* p : {(void*)th, (void*)m, (void*)v, (void*)grad, (void*)P1, (void*)P2, (void*)P3, (void*)P3T,
+                    (void*)P2T, (void*)OUT, (void*)loss_acc, (void*)bad})
       if (p) cudaFree(p);
   }
 };
@@ -360,9 +441,9 @@ cudaError_t alloc_n(T** p, int64_t n) {
   return cudaMalloc((void**)p, sizeof(T) * (size_t)(n > 0 ? n : 1));
 }
 
+// Training workspace of `rows` rows (a multiple of kRows).
 cudaError_t ensure_cap(fem_mlp* n, int64_t rows) {
-  const int64_t need = ((rows + 63) / 64) * 64;
-  if (need <= n->cap) return cudaSuccess;
+  if (rows <= n->cap) return cudaSuccess;
   // the old workspace may still be read by work queued on another stream
   CE(cudaDeviceSynchronize());
   n->free_ws();
@@ -370,95 +451,59 @@ cudaError_t ensure_cap(fem_mlp* n, int64_t rows) {
   auto A = [&](auto** p, int64_t k) {
     if (e == cudaSuccess) e = alloc_n(p, k);
   };
-  A(&n->X0, need * kL0); A(&n->X0T, need * kL0);
-  A(&n->A1, need * kL1); A(&n->A1T, need * kL1); A(&n->A2, need * kL2); A(&n->A2T, need * kL2);
-  A(&n->dZ3b, need * kL3); A(&n->dZ3T, need * kL3); A(&n->dZ2b, need * kL2); A(&n->dZ2T, need * kL2);
-  A(&n->dZ1T, need * kL1);
-  A(&n->Z1, need * kL1); A(&n->Z2, need * kL2); A(&n->OUT, need * kL3);
-  A(&n->dZ3f, need * kL3); A(&n->dZ2f, need * kL2); A(&n->dZ1f, need * kL1);
+  A(&n->X0, rows * kL0); A(&n->A1, rows * kL1); A(&n->A2, rows * kL2);
+  A(&n->dZ1, rows * kL1); A(&n->dZ2, rows * kL2); A(&n->dZ3, rows * kL3);
   if (e != cudaSuccess) {
     cudaGetLastError();
     n->free_ws();
     return e;
   }
-  n->cap = need;
+  n->cap = rows;
   return cudaSuccess;
 }
 
 cudaError_t pack_weights(fem_mlp* n, cudaStream_t s) {
-  k_pack<<<grid_of(90112), 256, 0, s>>>(n->th, n->W1, n->W2, n->W2T, n->W3, n->W3T);
+  k_pack<<<grid_of(kNParams + kL2 * kL1), 256, 0, s>>>(n->th, n->P1, n->P2, n->P3, n->P3T, n->P2T);
   return cudaGetLastError();
 }
 
-
-// Forward over B rows of x (gathered through idx if given).  training: keep pre-activations and the
-// transposed activations for the backward pass.  The output stays in n->OUT [Mpad][32].
-cudaError_t forward(fem_mlp* n, const float* x, const int32_t* idx, int64_t n_src, int64_t B, bool training,
-                    cudaStream_t s) {
-  CE(ensure_cap(n, B));
-  const int64_t Mp = ((B + 63) / 64) * 64;
-  const int M = (int)Mp;
-  k_stage<<<grid_of(Mp * kL0), 256, 0, s>>>(x, idx, n_src, B, Mp, n->X0, training ? n->X0T : nullptr, n->bad);
-  CE(cudaGetLastError());
-  GemmArgs g1 = gargs(M, kL1, kL0, n->X0, kL0, n->W1, kL0);
-  g1.bias = n->th + kOffB1;
-  g1.C = training ? n->Z1 : nullptr, g1.c_rs = kL1, g1.c_cs = 1;
-  g1.act = n->A1, g1.ld_act = kL1;
-  g1.actT = training ? n->A1T : nullptr, g1.ld_actT = M;
-  CE(gemm<EPI_GELU>(g1, s));
-  GemmArgs g2 = gargs(M, kL2, kL1, n->A1, kL1, n->W2, kL1);
-  g2.bias = n->th + kOffB2;
-  g2.C = training ? n->Z2 : nullptr, g2.c_rs = kL2, g2.c_cs = 1;
-  g2.act = n->A2, g2.ld_act = kL2;
-  g2.actT = training ? n->A2T : nullptr, g2.ld_actT = M;
-  CE(gemm<EPI_GELU>(g2, s));
-  GemmArgs g3 = gargs(M, kL3, kL2, n->A2, kL2, n->W3, kL2);
-  g3.bias = n->th + kOffB3;
-  g3.C = n->OUT, g3.c_rs = kL3, g3.c_cs = 1;
-  CE(gemm<EPI_BIAS>(g3, s));
-  return cudaSuccess;
+MlpPass pass_args(const fem_mlp* n, const float* x, const int32_t* idx, int64_t n_src, int64_t B) {
+  MlpPass g{};
+  g.x = x, g.idx = idx, g.n_src = n_src, g.B = B, g.Mpad = ((B + kRows - 1) / kRows) * kRows;
+  g.P1 = (const uint4*)n->P1, g.P2 = (const uint4*)n->P2, g.P3 = (const uint4*)n->P3;
+  g.P3T = (const uint4*)n->P3T, g.P2T = (const uint4*)n->P2T;
+  g.th = n->th, g.bad = n->bad;
+  return g;
 }
 
-// Backward of the mean squared error against t (rows gathered through idx) after forward(training):
-// gradient into n->grad, sum of squared errors added to n->loss_acc.
-cudaError_t backward(fem_mlp* n, const float* t, const int32_t* idx, int64_t n_src, int64_t B, cudaStream_t s,
-                     bool residual = false) {
-  const int64_t Mp = ((B + 63) / 64) * 64;
-  const int M = (int)Mp;
+// out [B][32] = network of the B rows of x.
+cudaError_t forward(fem_mlp* n, const float* x, int64_t B, float* out, cudaStream_t s) {
+  MlpPass g = pass_args(n, x, nullptr, B, B);
+  g.out = out;
+  k_mlp_pass<0><<<(unsigned)(g.Mpad / kRows), kMlpBlock, 0, s>>>(g);
+  return cudaGetLastError();
+}
+
+// Loss (added to n->loss_acc) and its gradient into grad, over B rows (gathered through idx if given) of x and
+// the targets t (residual: residual-space samples).
+cudaError_t loss_grad(fem_mlp* n, const float* x, const float* t, const int32_t* idx, int64_t n_src, int64_t B,
+                      float* grad, cudaStream_t s, bool residual) {
+  MlpPass g = pass_args(n, x, idx, n_src, B);
+  CE(ensure_cap(n, g.Mpad));
+  CE(cudaMemsetAsync(grad, 0, sizeof(float) * kNParams, s));
+  g.t = t, g.grad = grad, g.loss = n->loss_acc;
+  g.X0 = n->X0, g.A1 = n->A1, g.A2 = n->A2, g.dZ1 = n->dZ1, g.dZ2 = n->dZ2, g.dZ3 = n->dZ3;
+  const unsigned blocks = (unsigned)(g.Mpad / kRows);
   if (residual)
-    k_loss_res<<<(int)std::min<int64_t>((Mp + 7) / 8, 4096), 256, 0, s>>>(n->OUT, t, idx, n_src, B, Mp, n->dZ3f,
-                                                                          n->dZ3b, n->dZ3T, n->loss_acc);
+    k_mlp_pass<2><<<blocks, kMlpBlock, 0, s>>>(g);
   else
-    k_loss<<<grid_of(Mp * kL3), 256, 0, s>>>(n->OUT, t, idx, n_src, B, Mp, n->dZ3f, n->dZ3b, n->dZ3T, n->loss_acc);
+    k_mlp_pass<1><<<blocks, kMlpBlock, 0, s>>>(g);
   CE(cudaGetLastError());
-  // dW3 [32][256] = dZ3^T A2, computed as its transpose (256 x 32, contraction over the batch)
-  GemmArgs w3 = gargs(kL2, kL3, M, n->A2T, M, n->dZ3T, M);
-  w3.C = n->grad + kOffW3, w3.c_rs = 1, w3.c_cs = kL2;
-  CE(gemm<EPI_PLAIN>(w3, s));
-  k_colsum<<<kL3 / 32, 256, 0, s>>>(n->dZ3f, Mp, kL3, n->grad + kOffB3);
-  CE(cudaGetLastError());
-  // dZ2 = (dZ3 W3) * GELU'(Z2)
-  GemmArgs d2 = gargs(M, kL2, kL3, n->dZ3b, kL3, n->W3T, kL3);
-  d2.zin = n->Z2, d2.ldz = kL2, d2.m_valid = (int)B;
-  d2.C = n->dZ2f, d2.c_rs = kL2, d2.c_cs = 1;
-  d2.act = n->dZ2b, d2.ld_act = kL2;
-  d2.actT = n->dZ2T, d2.ld_actT = M;
-  CE(gemm<EPI_GELU_BWD>(d2, s));
-  GemmArgs w2 = gargs(kL2, kL1, M, n->dZ2T, M, n->A1T, M);
-  w2.C = n->grad + kOffW2, w2.c_rs = kL1, w2.c_cs = 1;
-  CE(gemm<EPI_PLAIN>(w2, s));
-  k_colsum<<<kL2 / 32, 256, 0, s>>>(n->dZ2f, Mp, kL2, n->grad + kOffB2);
-  CE(cudaGetLastError());
-  // dZ1 = (dZ2 W2) * GELU'(Z1)
-  GemmArgs d1 = gargs(M, kL1, kL2, n->dZ2b, kL2, n->W2T, kL2);
-  d1.zin = n->Z1, d1.ldz = kL1, d1.m_valid = (int)B;
-  d1.C = n->dZ1f, d1.c_rs = kL1, d1.c_cs = 1;
-  d1.actT = n->dZ1T, d1.ld_actT = M;
-  CE(gemm<EPI_GELU_BWD>(d1, s));
-  GemmArgs w1 = gargs(kL1, kL0, M, n->dZ1T, M, n->X0T, M);
-  w1.C = n->grad + kOffW1, w1.c_rs = kL0, w1.c_cs = 1;
-  CE(gemm<EPI_PLAIN>(w1, s));
-  k_colsum<<<kL1 / 32, 256, 0, s>>>(n->dZ1f, Mp, kL1, n->grad + kOffB1);
+  // 24 tiles; the batch split so that the grid covers the SMs twice, at least 4 of the 32-row steps a block
+  MlpWgrad w{n->X0, n->A1, n->A2, n->dZ1, n->dZ2, n->dZ3, grad, (int)(g.Mpad / 32)};
+  int split = (2 * sm_count() + 23) / 24;
+  if (split > w.steps / 4) split = w.steps / 4;
+  k_mlp_wgrad<<<dim3(24, split < 1 ? 1 : split), 128, 0, s>>>(w);
   return cudaGetLastError();
 }
 
@@ -715,7 +760,14 @@ cudaError_t mlp_features(const PredView& p, int n_pairs, const float4* case_src,
 
 cudaError_t mlp_propose(fem_mlp* net, const float* F, int64_t rows, int n_pairs, double* dw, cudaStream_t s) {
   std::lock_guard<std::mutex> lk(net->mu);
-  CE(forward(net, F, nullptr, rows, rows, false, s));
+  if (rows > net->out_cap) {
+    CE(cudaDeviceSynchronize());      // (the old buffer may still be read by work queued on another stream)
+    if (net->OUT) cudaFree(net->OUT);
+    net->OUT = nullptr, net->out_cap = 0;
+    CE(alloc_n(&net->OUT, rows * kL3));
+    net->out_cap = rows;
+  }
+  CE(forward(net, F, rows, net->OUT, s));
   k_coef_delta<<<grid_of(rows * kMaxSlots), 256, 0, s>>>(rows, n_pairs, net->OUT, dw);
   return cudaGetLastError();
 }
@@ -790,8 +842,8 @@ fem_status fem_mlp_create(const float* params, void* stream, fem_mlp** out) {
     if (e == cudaSuccess) e = alloc_n(p, k);
   };
   A(&n->th, kNParams); A(&n->m, kNParams); A(&n->v, kNParams); A(&n->grad, kNParams);
-  A(&n->W1, (int64_t)kL1 * kL0); A(&n->W2, (int64_t)kL2 * kL1); A(&n->W2T, (int64_t)kL2 * kL1);
-  A(&n->W3, (int64_t)kL3 * kL2); A(&n->W3T, (int64_t)kL3 * kL2); A(&n->loss_acc, 1); A(&n->bad, 1);
+  A(&n->P1, (int64_t)kL1 * kL0); A(&n->P2, (int64_t)kL2 * kL1); A(&n->P2T, (int64_t)kL2 * kL1);
+  A(&n->P3, (int64_t)kL3 * kL2); A(&n->P3T, (int64_t)kL3 * kL2); A(&n->loss_acc, 1); A(&n->bad, 1);
   if (e != cudaSuccess) {
     cudaGetLastError();
     delete n;
@@ -830,8 +882,7 @@ fem_status fem_mlp_forward(fem_mlp* n, const float* x_dev, int64_t B, float* out
   if (!n || (B > 0 && (!x_dev || !out_dev)) || B < 0) return set_error(FEM_ERR_ARG, "fem_mlp_forward: bad argument");
   if (B == 0) return FEM_OK;
   std::lock_guard<std::mutex> lk(n->mu);
-  MCU(forward(n, x_dev, nullptr, B, B, false, n->s));
-  MCU(cudaMemcpyAsync(out_dev, n->OUT, sizeof(float) * kL3 * B, cudaMemcpyDeviceToDevice, n->s));
+  MCU(forward(n, x_dev, B, out_dev, n->s));
   return FEM_OK;
 }
 
@@ -842,9 +893,7 @@ static fem_status mlp_loss_grad_any(fem_mlp* n, const float* x_dev, const float*
   if (!n || !x_dev || !t_dev || B <= 0) return set_error(FEM_ERR_ARG, "fem_mlp_loss_grad: bad argument");
   std::lock_guard<std::mutex> lk(n->mu);
   MCU(cudaMemsetAsync(n->loss_acc, 0, sizeof(double), n->s));
-  MCU(forward(n, x_dev, nullptr, B, B, true, n->s));
-  MCU(backward(n, t_dev, nullptr, B, B, n->s, residual));
-  if (grad_dev) MCU(cudaMemcpyAsync(grad_dev, n->grad, sizeof(float) * kNParams, cudaMemcpyDeviceToDevice, n->s));
+  MCU(loss_grad(n, x_dev, t_dev, nullptr, B, B, grad_dev ? grad_dev : n->grad, n->s, residual));
   double acc = 0.0;
   MCU(cudaMemcpyAsync(&acc, n->loss_acc, sizeof(double), cudaMemcpyDeviceToHost, n->s));
   MCU(cudaStreamSynchronize(n->s));
@@ -863,8 +912,7 @@ static fem_status mlp_train_any(fem_mlp* n, const float* x_dev, const float* t_d
   for (int u = 0; u < n_updates; ++u) {
     const int32_t* idx = order_dev + (int64_t)u * batch;
     if (loss_out) MCU(cudaMemsetAsync(n->loss_acc, 0, sizeof(double), n->s));
-    MCU(forward(n, x_dev, idx, n_samples, batch, true, n->s));
-    MCU(backward(n, t_dev, idx, n_samples, batch, n->s, residual));
+    MCU(loss_grad(n, x_dev, t_dev, idx, n_samples, batch, n->grad, n->s, residual));
     if (loss_out) {
       double acc = 0.0;
       MCU(cudaMemcpyAsync(&acc, n->loss_acc, sizeof(double), cudaMemcpyDeviceToHost, n->s));

@@ -452,3 +452,40 @@ def test_learned_proposal_gain_on_held_out_cases(torch_dev):
         assert it_ml.sum() <= it_dd.sum() * 1.02 + 8
     finally:
         fem.fem_mlp_destroy(net)
+
+
+@pytest.mark.parametrize("B", [1, 31, 32, 33, 127, 500])
+@pytest.mark.parametrize("residual", [False, True])
+def test_batch_edges(torch_dev, B, residual):
+    """Batches around the kernels' block of 32 samples: a row's output does not depend on the batch it is in (same
+    operations: equal), and the gradient of a batch is the mean of its halves' (FP32 sums of at most 500 samples
+    in another order: 1e-5 of the largest entry, times the BF16 rounding of dL/dout, scaled by 1/B: 2^-8)."""
+    torch = torch_dev
+    rng = np.random.default_rng(B)
+    x = rng.standard_normal((B, 64)).astype(np.float32)
+    x[:, 36:] = 0.0
+    X = torch.tensor(x, device="cuda")
+    T = torch.tensor(rng.standard_normal((B, fem.FEM_MLP_RES if residual else 32)).astype(np.float32), device="cuda")
+    net = fem.fem_mlp_create(wl.mlp_init_weights(3).astype(np.float32))
+    f = fem.fem_mlp_loss_grad_residual if residual else fem.fem_mlp_loss_grad
+    try:
+        out = torch.full((B, 32), float("nan"), device="cuda")
+        fem.fem_mlp_forward(net, X, out)
+        one = torch.empty((1, 32), device="cuda")
+        for r in {0, B // 2, B - 1}:
+            fem.fem_mlp_forward(net, X[r:r + 1].contiguous(), one)
+            assert torch.equal(one[0], out[r])
+
+        def grad(a, b):
+            g = torch.full((fem.FEM_MLP_N_PARAMS,), float("nan"), device="cuda")
+            return f(net, X[a:b].contiguous(), T[a:b].contiguous(), g), g
+
+        loss, g = grad(0, B)
+        if B > 1:
+            h = B // 2
+            (l1, g1), (l2, g2) = grad(0, h), grad(h, B)
+            assert abs(loss - (l1 * h + l2 * (B - h)) / B) <= 1e-9 * abs(loss)
+            ref = (g1.double() * h + g2.double() * (B - h)) / B
+            assert float((g.double() - ref).abs().max()) <= 2.0 ** -8 * float(ref.abs().max())
+    finally:
+        fem.fem_mlp_destroy(net)
