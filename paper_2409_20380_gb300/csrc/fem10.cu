@@ -3,21 +3,20 @@
 // gradients g_a are constant on a tet, so the element record is the tet4 one of its corners (g_1..g_3,
 // lambda V, mu V, rho V / 20) and the quadratic shape-function gradients are formed on the fly,
 //   corner a:    grad N_a  = (4 L_a - 1) g_a,       edge (a, b): grad N_ab = 4 (L_a g_b + L_b g_a),
-// at the four points of the degree-2 Gauss rule (exact for the stiffness, whose integrand is quadratic):
-//   (K p)_i = sum_q V/4 sigma(G_q) grad N_i(L_q),  G_q = sum_j p_j (x) grad N_j(L_q),
-//   sigma(G) = lambda tr(G) I + mu (G + G^T),
-// both sums taken through the four corner gradients (about 180 operations a point instead of 450).
+// whose linear strain is taken at the four corners (elem10: the stiffness integrand is quadratic, so the corner
+// form integrates it exactly, as the degree-2 Gauss rule of the preconditioner's and the assembled blocks does).
 // The consistent mass (M p)_i = rho V sum_j m_ij p_j with m_ij = int N_i N_j dV / V: generated on the host
 // from int L_0^a L_1^b L_2^c L_3^d dV = 6 V a! b! c! d! / (a + b + c + d + 3)! for the preconditioner's
 // diagonal, applied in the product through the seven distinct values of 420 m_ij.
 // Local order: corners 0-3, edges (0,1), (1,2), (0,2), (0,3), (1,3), (2,3).  One thread per (element,
-// case); sums scatter with global atomics (Dirichlet rows masked afterwards).
+// case); sums scatter with global atomics into a zeroed q, Dirichlet DOFs skipped (the FP32 products of four cases
+// and more go through the tiles of k_elem_tile.cu).
 #include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <vector>
 
-#include "fem_internal.cuh"
+#include "elem_ops.cuh"
 
 namespace fem {
 
@@ -26,8 +25,6 @@ namespace {
 // edge s joins corners edge_a(s) and edge_b(s)
 __host__ __device__ constexpr int edge_a(int s) { return s == 0 ? 0 : s == 1 ? 1 : s == 2 ? 0 : s == 3 ? 0 : s == 4 ? 1 : 2; }
 __host__ __device__ constexpr int edge_b(int s) { return s == 0 ? 1 : s == 1 ? 2 : s == 2 ? 2 : s == 3 ? 3 : s == 4 ? 3 : 3; }
-// the edge sharing no corner with edge s
-__host__ __device__ constexpr int edge_opp(int s) { return s == 0 ? 5 : s == 1 ? 3 : s == 2 ? 4 : s == 3 ? 1 : s == 4 ? 2 : 0; }
 
 struct Mass10 {
   double m64[55];   // upper triangle of m_ij, row-major
@@ -91,123 +88,40 @@ template <> struct Rec10<double> {
 template <typename T, bool DOT, typename I>
 __global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? 2 : 1) k_ebe10(int64_t E, int rpad, int rshift, const int32_t* __restrict__ conn,
                                                    const float* __restrict__ rec32, const double* __restrict__ rec64,
-                                                   const T* __restrict__ p, T* __restrict__ q, T aM, T aK,
+                                                   const uint8_t* __restrict__ fm, const T* __restrict__ p,
+                                                   T* __restrict__ q, T aM, T aK,
                                                    Reducer red, double* ptq_out, CgCase* sc,
                                                    const int* gate) {
   if (gate && *gate == 0) return;
   const T* __restrict__ recs = Rec10<T>::get(rec32, rec64);
-  // barycentric coordinates of the four Gauss points: (A, B, B, B) and its permutations
-  const T GA = (T)0.5854101966249685, GB = (T)0.1381966011250105;
   double dot = 0.0;
   const int64_t total = E << rshift;
   for (int64_t it = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; it < total; it += (int64_t)gridDim.x * blockDim.x) {
     const int64_t e = it >> rshift;
     const int c = (int)(it & (rpad - 1));
     I off[10];   // offset of node i's first value of case c
+    int fr[10];
 #pragma unroll
-    for (int i = 0; i < 10; ++i) off[i] = (I)__ldg(conn + e * 10 + i) * (I)(3 * rpad) + (I)c;
-    T P[10][3], Q[10][3];
-#pragma unroll
-    for (int i = 0; i < 10; ++i)
-#pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        P[i][k] = __ldg(p + off[i] + (I)(k * rpad));
-        Q[i][k] = (T)0;
-      }
-    const T* r = recs + e * kRec;
-    T g[4][3];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      g[1][k] = r[k], g[2][k] = r[3 + k], g[3][k] = r[6 + k];
-      g[0][k] = -(g[1][k] + g[2][k] + g[3][k]);
+    for (int i = 0; i < 10; ++i) {
+      const int nd = __ldg(conn + e * 10 + i);
+      off[i] = (I)nd * (I)(3 * rpad) + (I)c;
+      fr[i] = fm[nd];
     }
-    const T lam = aK * r[9] * (T)0.25, mu = aK * r[10] * (T)0.25, rv = aM * r[11] * (T)20;   // V/4 weights
-    // At a Gauss point grad N_i = sum_a c_ia g_a (c linear in L), so both contractions run through the four
-    // corners: G = sum_a W_a (x) g_a with W_a = sum_i c_ia p_i, and the forces sum_a c_ia (sigma g_a):
-    //   W_a = (4 L_a - 1) p_a + 4 sum_{edges (a, b)} L_b p_ab,
-    //   f_a += (4 L_a - 1) T_a,   f_ab += 4 (L_a T_b + L_b T_a),   T_a = sigma g_a.
-#pragma unroll
-    for (int qp = 0; qp < 4; ++qp) {   // (unrolled: the points' coefficients are constants)
-      T L[4];
-#pragma unroll
-      for (int a = 0; a < 4; ++a) L[a] = a == qp ? GA : GB;
-      T W[4][3];
-#pragma unroll
-      for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int k = 0; k < 3; ++k) W[a][k] = ((T)4 * L[a] - (T)1) * P[a][k];
-#pragma unroll
-      for (int e = 0; e < 6; ++e) {
-        const int a = edge_a(e), b = edge_b(e);
-        const T lb4 = (T)4 * L[b], la4 = (T)4 * L[a];
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-          W[a][k] += lb4 * P[4 + e][k];
-          W[b][k] += la4 * P[4 + e][k];
-        }
-      }
-      T G[3][3];
-#pragma unroll
-      for (int k = 0; k < 3; ++k)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) G[k][j] = W[0][k] * g[0][j] + W[1][k] * g[1][j] + W[2][k] * g[2][j] + W[3][k] * g[3][j];
-      const T ltr = lam * (G[0][0] + G[1][1] + G[2][2]);
-      T S[3][3];
-#pragma unroll
-      for (int k = 0; k < 3; ++k)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) S[k][j] = mu * (G[k][j] + G[j][k]) + (k == j ? ltr : (T)0);
-      T Tg[4][3];
-#pragma unroll
-      for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int k = 0; k < 3; ++k) Tg[a][k] = S[k][0] * g[a][0] + S[k][1] * g[a][1] + S[k][2] * g[a][2];
-#pragma unroll
-      for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int k = 0; k < 3; ++k) Q[a][k] += ((T)4 * L[a] - (T)1) * Tg[a][k];
-#pragma unroll
-      for (int e = 0; e < 6; ++e) {
-        const int a = edge_a(e), b = edge_b(e);
-        const T la4 = (T)4 * L[a], lb4 = (T)4 * L[b];
-#pragma unroll
-        for (int k = 0; k < 3; ++k) Q[4 + e][k] += la4 * Tg[b][k] + lb4 * Tg[a][k];
-      }
-    }
-    // consistent mass through its structure: 420 m_ij = 6 / 1 (corner diagonal / other corner), -4 / -6
-    // (corner and an edge through it / the others), 32 / 16 / 8 (edge diagonal / an edge sharing a corner /
-    // the opposite edge), so with the corner and edge sums Sc, Se:
-    //   corner a:      5 p_a + Sc - 6 Se + 2 (sum of a's three edges)
-    //   edge (a, b):  -6 Sc + 2 (p_a + p_b) + 16 Se + 16 p_ab - 8 p_opposite
-    const T rv420 = rv * (T)(1.0 / 420.0);
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      const T Sc = (P[0][k] + P[1][k]) + (P[2][k] + P[3][k]);
-      const T Se = (P[4][k] + P[5][k]) + (P[6][k] + P[7][k]) + (P[8][k] + P[9][k]);
-      const T base_c = Sc - (T)6 * Se, base_e = (T)16 * Se - (T)6 * Sc;
-#pragma unroll
-      for (int a = 0; a < 4; ++a) {
-        T Ea = (T)0;
-#pragma unroll
-        for (int e = 0; e < 6; ++e)
-          if (edge_a(e) == a || edge_b(e) == a) Ea += P[4 + e][k];
-        Q[a][k] += rv420 * ((T)5 * P[a][k] + base_c + (T)2 * Ea);
-      }
-#pragma unroll
-      for (int e = 0; e < 6; ++e) {
-        const int a = edge_a(e), b = edge_b(e), o = edge_opp(e);
-        Q[4 + e][k] += rv420 * (base_e + (T)2 * (P[a][k] + P[b][k]) + (T)16 * P[4 + e][k] - (T)8 * P[4 + o][k]);
-      }
-    }
+    T r[12];
+    load_rec(recs + e * kRec, r);
     T hd = (T)0;   // (the element's p^T q in the product's precision, one conversion an element: FP64
                    // conversions and adds run on GB300's narrow FP64 pipe)
+    elem10<DOT, T, T>(
+        [&](int i, T (&P)[3]) {
 #pragma unroll
-    for (int i = 0; i < 10; ++i)
+          for (int k = 0; k < 3; ++k) P[k] = __ldg(p + off[i] + (I)(k * rpad));
+        },
+        [&](int i, const T (&Q)[3]) {
 #pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        if (DOT) hd += P[i][k] * Q[i][k];
-        atomicAdd(q + off[i] + (I)(k * rpad), Q[i][k]);
-      }
+          for (int k = 0; k < 3; ++k)
+            if (dof_free((uint8_t)fr[i], k)) atomicAdd(q + off[i] + (I)(k * rpad), Q[k]);
+        },
+        r, aM, aK, hd);
     if (DOT) dot += (double)hd;
   }
   if (DOT) {
@@ -345,9 +259,13 @@ template <typename T>
 cudaError_t launch_ebe10_gated(int64_t E, int64_t N, int rpad, const int32_t* conn10, const float* rec32,
                                const double* rec64, const uint8_t* fm, const T* pm, const T* pk, T* q, double aM,
                                double aK, const Reducer* red, CgCase* sc, double* ptq, const int* gate,
-                               cudaStream_t s) {
+                               cudaStream_t s, const ElemTiles* et) {
   cudaError_t e = cudaMemsetAsync(q, 0, sizeof(T) * (size_t)N * 3 * rpad, s);
   if (e != cudaSuccess) return e;
+  if constexpr (sizeof(T) == 4) {
+    if (!pk && et && elem_tile_fits(10, *et, rpad, pm, q))
+      return launch_elem_tile(10, *et, E, rpad, rec32, pm, q, aM, aK, red, sc, ptq, gate, s);
+  }
   const int rs = lg2i(rpad);
   const bool i32 = N * 3 * rpad < ((int64_t)1 << 31);
   const Reducer none{nullptr, nullptr, nullptr};
@@ -355,7 +273,7 @@ cudaError_t launch_ebe10_gated(int64_t E, int64_t N, int rpad, const int32_t* co
     const int grid = grid_for(E << rs, dot ? red_grid_cap() : -1);
     auto fn = dot ? (i32 ? k_ebe10<T, true, int32_t> : k_ebe10<T, true, int64_t>)
                   : (i32 ? k_ebe10<T, false, int32_t> : k_ebe10<T, false, int64_t>);
-    fn<<<grid, kBlock, 0, s>>>(E, rpad, rs, conn10, rec32, rec64, p, q, a_m, a_k, dot ? *red : none,
+    fn<<<grid, kBlock, 0, s>>>(E, rpad, rs, conn10, rec32, rec64, fm, p, q, a_m, a_k, dot ? *red : none,
                                dot ? ptq : nullptr, dot ? sc : nullptr, gate);
     return cudaGetLastError();
   };
@@ -365,15 +283,14 @@ cudaError_t launch_ebe10_gated(int64_t E, int64_t N, int rpad, const int32_t* co
   } else {
     e = run(pm, (T)aM, (T)aK, red != nullptr);
   }
-  if (e == cudaSuccess) e = launch_mask<T>(N, rpad, fm, q, s);
   return e;
 }
 template cudaError_t launch_ebe10_gated<float>(int64_t, int64_t, int, const int32_t*, const float*, const double*,
                                                const uint8_t*, const float*, const float*, float*, double, double,
-                                               const Reducer*, CgCase*, double*, const int*, cudaStream_t);
+                                               const Reducer*, CgCase*, double*, const int*, cudaStream_t, const ElemTiles*);
 template cudaError_t launch_ebe10_gated<double>(int64_t, int64_t, int, const int32_t*, const float*, const double*,
                                                 const uint8_t*, const double*, const double*, double*, double, double,
-                                                const Reducer*, CgCase*, double*, const int*, cudaStream_t);
+                                                const Reducer*, CgCase*, double*, const int*, cudaStream_t, const ElemTiles*);
 
 cudaError_t launch_diag10(int64_t E, const int32_t* conn10, const double* rec64, double aM, double aK, double* D,
                           cudaStream_t s) {
@@ -409,7 +326,9 @@ struct fem_mesh10 {
   unsigned* counter = nullptr;
   double* out = nullptr;
   Mass10 mc{};
+  ElemTiles et;               // tiles of the FP32 products
   ~fem_mesh10() {
+    free_elem_tiles(&et);
     cudaFree(conn); cudaFree(rec32); cudaFree(rec64); cudaFree(fm); cudaFree(partial); cudaFree(counter); cudaFree(out);
   }
 };
@@ -476,6 +395,12 @@ fem_status fem_mesh10_create(int64_t n_nodes, const double* xyz, int64_t n_elems
     if (e != cudaSuccess) return set_error(FEM_ERR_CUDA, std::string("tet10 mesh: ") + cudaGetErrorString(e));
     return set_error(FEM_ERR_ARG, h_err & 2 ? "degenerate or inverted corner tet" : "bad material id");
   }
+  e = build_elem_tiles(10, n_elems, n_nodes, m->conn, m->fm, m->rec32, &m->et, s);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    delete m;
+    return set_error(FEM_ERR_CUDA, std::string("tet10 tiles: ") + cudaGetErrorString(e));
+  }
   double mm[10][10];
   mass10_host(mm);
   for (int i = 0; i < 10; ++i)
@@ -497,31 +422,14 @@ fem_status fem_ebe10_apply(fem_mesh10* m, int precision, const void* p_dev, void
   if (n_rhs < 1 || n_rhs > kMaxRpad || (n_rhs & (n_rhs - 1))) return set_error(FEM_ERR_ARG, "n_rhs must be 1, 2, 4, 8, 16 or 32");
   if (precision != FEM_FP64 && precision != FEM_FP32_INNER) return set_error(FEM_ERR_ARG, "unknown precision");
   cudaStream_t s = (cudaStream_t)stream;
-  const int rs = lg2i(n_rhs);
-  const int64_t items = m->E << rs;
-  int grid = grid_for(items, red_grid_cap());
   const Reducer red{m->partial, m->counter, m->out};
-  const bool dot = ptq_dev != nullptr;
-  const size_t bytes = (precision == FEM_FP64 ? 8 : 4) * (size_t)m->N * 3 * n_rhs;
-  cudaError_t e = cudaMemsetAsync(q_dev, 0, bytes, s);
-  if (e == cudaSuccess) {
-    const bool i32 = m->N * 3 * n_rhs < ((int64_t)1 << 31);
-    if (precision == FEM_FP64) {
-      auto fn = dot ? (i32 ? k_ebe10<double, true, int32_t> : k_ebe10<double, true, int64_t>)
-                    : (i32 ? k_ebe10<double, false, int32_t> : k_ebe10<double, false, int64_t>);
-      fn<<<grid, kBlock, 0, s>>>(m->E, n_rhs, rs, m->conn, m->rec32, m->rec64, (const double*)p_dev, (double*)q_dev,
-                                 alpha_M, alpha_K, red, ptq_dev, nullptr, nullptr);
-    } else {
-      auto fn = dot ? (i32 ? k_ebe10<float, true, int32_t> : k_ebe10<float, true, int64_t>)
-                    : (i32 ? k_ebe10<float, false, int32_t> : k_ebe10<float, false, int64_t>);
-      fn<<<grid, kBlock, 0, s>>>(m->E, n_rhs, rs, m->conn, m->rec32, m->rec64, (const float*)p_dev, (float*)q_dev,
-                                 (float)alpha_M, (float)alpha_K, red, ptq_dev, nullptr, nullptr);
-    }
-    e = cudaGetLastError();
-  }
-  if (e == cudaSuccess)
-    e = precision == FEM_FP64 ? launch_mask<double>(m->N, n_rhs, m->fm, (double*)q_dev, s)
-                              : launch_mask<float>(m->N, n_rhs, m->fm, (float*)q_dev, s);
+  const Reducer* rd = ptq_dev ? &red : nullptr;
+  const cudaError_t e =
+      precision == FEM_FP64
+          ? launch_ebe10_gated<double>(m->E, m->N, n_rhs, m->conn, m->rec32, m->rec64, m->fm, (const double*)p_dev,
+                                       nullptr, (double*)q_dev, alpha_M, alpha_K, rd, nullptr, ptq_dev, nullptr, s)
+          : launch_ebe10_gated<float>(m->E, m->N, n_rhs, m->conn, m->rec32, m->rec64, m->fm, (const float*)p_dev, nullptr,
+                                      (float*)q_dev, alpha_M, alpha_K, rd, nullptr, ptq_dev, nullptr, s, &m->et);
   if (e != cudaSuccess) return set_error(FEM_ERR_CUDA, std::string("tet10 product: ") + cudaGetErrorString(e));
   return FEM_OK;
 }
@@ -535,7 +443,7 @@ fem_status pcg10_solve(fem_mesh10* m, int precision, const double* b_dev, double
   if (n_rhs < 1 || n_rhs > kMaxRpad || (n_rhs & (n_rhs - 1))) return set_error(FEM_ERR_ARG, "n_rhs must be 1, 2, 4, 8, 16 or 32");
   if (!(tol > 0.0) || maxit < 1) return set_error(FEM_ERR_ARG, "tol must be > 0 and maxit >= 1");
   cudaStream_t s = (cudaStream_t)stream;
-  const int rpad = n_rhs, rs = lg2i(n_rhs);
+  const int rpad = n_rhs;
   const size_t n = (size_t)m->N * 3 * rpad;
   double *D = nullptr, *b64 = nullptr, *r = nullptr, *z = nullptr, *p = nullptr, *q = nullptr;
   float* b32 = nullptr;
@@ -563,27 +471,16 @@ fem_status pcg10_solve(fem_mesh10* m, int precision, const double* b_dev, double
   }
   MeshView mv{m->N, m->E, nullptr, m->rec64, m->rec32, b64, b32, m->fm, nullptr, 0};
   const Reducer red{m->partial, m->counter, m->out};
-  const int grid = grid_for(m->E << rs, red_grid_cap());
   auto product32 = [&](const float* in, float* out) {   // FP32 product with p^T q and the step length
-    if (e == cudaSuccess) e = cudaMemsetAsync(out, 0, sizeof(float) * n, s);
-    if (e != cudaSuccess) return;
-    k_ebe10<float, true, int64_t><<<grid, kBlock, 0, s>>>(m->E, rpad, rs, m->conn, m->rec32, m->rec64, in, out,
-                                                          (float)alpha_M, (float)alpha_K, red, nullptr, sc,
-                                                          n_active);
-    e = cudaGetLastError();
-    if (e == cudaSuccess) e = launch_mask<float>(m->N, rpad, m->fm, out, s);
+    if (e == cudaSuccess)
+      e = launch_ebe10_gated<float>(m->E, m->N, rpad, m->conn, m->rec32, m->rec64, m->fm, in, nullptr, out, alpha_M,
+                                    alpha_K, &red, sc, nullptr, n_active, s, &m->et);
   };
   auto product = [&](const double* in, double* out, bool dot) {
-    if (e == cudaSuccess) e = cudaMemsetAsync(out, 0, sizeof(double) * n, s);
-    if (e != cudaSuccess) return;
-    if (dot)
-      k_ebe10<double, true, int64_t><<<grid, kBlock, 0, s>>>(m->E, rpad, rs, m->conn, m->rec32, m->rec64, in, out,
-                                                             alpha_M, alpha_K, red, nullptr, sc, n_active);
-    else
-      k_ebe10<double, false, int64_t><<<grid, kBlock, 0, s>>>(m->E, rpad, rs, m->conn, m->rec32, m->rec64, in, out,
-                                                              alpha_M, alpha_K, red, nullptr, nullptr, nullptr);
-    e = cudaGetLastError();
-    if (e == cudaSuccess) e = launch_mask<double>(m->N, rpad, m->fm, out, s);
+    if (e == cudaSuccess)
+      e = launch_ebe10_gated<double>(m->E, m->N, rpad, m->conn, m->rec32, m->rec64, m->fm, in, nullptr, out, alpha_M,
+                                     alpha_K, dot ? &red : nullptr, dot ? sc : nullptr, nullptr,
+                                     dot ? n_active : nullptr, s);
   };
   if (e == cudaSuccess) e = cudaMemsetAsync(D, 0, sizeof(double) * 6 * m->N, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(err, 0, sizeof(int), s);

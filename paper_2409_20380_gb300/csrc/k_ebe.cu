@@ -8,7 +8,7 @@
 // This generic kernel scatters with global atomics into a zeroed q, skipping Dirichlet DOFs (rows stay zero).
 #include <cuda_fp16.h>
 
-#include "fem_internal.cuh"
+#include "elem_ops.cuh"
 
 #include <algorithm>
 #include <mutex>
@@ -49,40 +49,8 @@ static int log2i(int r) {
   return s;
 }
 
-// Paired FP32 operations (one instruction, two cases).
-__device__ __forceinline__ float2 bc2(float v) { return make_float2(v, v); }
-__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
-
-// The values a thread of the generic kernel works on: one case (float, double), or two adjacent cases of a node in
-// paired FP32 operations.
-template <typename T, int NC> struct ElemVal;
-template <typename T> struct ElemVal<T, 1> {
-  T v;
-  __device__ __forceinline__ static ElemVal load(const T* p) { return {*p}; }
-  __device__ __forceinline__ static ElemVal zero() { return {(T)0}; }
-  __device__ __forceinline__ void add_to(T* q) const { atomicAdd(q, v); }
-};
-template <> struct ElemVal<float, 2> {
-  float2 v;
-  __device__ __forceinline__ static ElemVal load(const float* p) { return {*reinterpret_cast<const float2*>(p)}; }
-  __device__ __forceinline__ static ElemVal zero() { return {make_float2(0.f, 0.f)}; }
-  __device__ __forceinline__ void add_to(float* q) const { atomicAdd(reinterpret_cast<float2*>(q), v); }
-};
-template <typename T> __device__ __forceinline__ ElemVal<T, 1> ev_add(ElemVal<T, 1> a, ElemVal<T, 1> b) { return {a.v + b.v}; }
-template <typename T> __device__ __forceinline__ ElemVal<T, 1> ev_sub(ElemVal<T, 1> a, ElemVal<T, 1> b) { return {a.v - b.v}; }
-template <typename T> __device__ __forceinline__ ElemVal<T, 1> ev_mul(ElemVal<T, 1> a, T b) { return {a.v * b}; }
-__device__ __forceinline__ ElemVal<float, 1> ev_fma(ElemVal<float, 1> a, float b, ElemVal<float, 1> c) { return {fmaf(a.v, b, c.v)}; }
-__device__ __forceinline__ ElemVal<double, 1> ev_fma(ElemVal<double, 1> a, double b, ElemVal<double, 1> c) { return {fma(a.v, b, c.v)}; }
-__device__ __forceinline__ ElemVal<float, 1> ev_fmv(ElemVal<float, 1> a, ElemVal<float, 1> b, ElemVal<float, 1> c) { return {fmaf(a.v, b.v, c.v)}; }
-__device__ __forceinline__ ElemVal<double, 1> ev_fmv(ElemVal<double, 1> a, ElemVal<double, 1> b, ElemVal<double, 1> c) { return {fma(a.v, b.v, c.v)}; }
-__device__ __forceinline__ ElemVal<float, 2> ev_add(ElemVal<float, 2> a, ElemVal<float, 2> b) { return {add2(a.v, b.v)}; }
-__device__ __forceinline__ ElemVal<float, 2> ev_sub(ElemVal<float, 2> a, ElemVal<float, 2> b) { return {sub2(a.v, b.v)}; }
-__device__ __forceinline__ ElemVal<float, 2> ev_mul(ElemVal<float, 2> a, float b) { return {mul2(a.v, bc2(b))}; }
-__device__ __forceinline__ ElemVal<float, 2> ev_fma(ElemVal<float, 2> a, float b, ElemVal<float, 2> c) { return {fma2(a.v, bc2(b), c.v)}; }
-__device__ __forceinline__ ElemVal<float, 2> ev_fmv(ElemVal<float, 2> a, ElemVal<float, 2> b, ElemVal<float, 2> c) { return {fma2(a.v, b.v, c.v)}; }
+template <typename T, int NC> struct CaseVal { using type = T; };
+template <> struct CaseVal<float, 2> { using type = float2; };
 
 // One thread per (element, NC adjacent cases).  TWO: M acts on pm, K on pk.  I: index type of the vector offsets.
 // The global FP32 atomics bound it (0.6e12 scalar adds a second): a pair of cases adds its two sums as one
@@ -94,9 +62,9 @@ __global__ void __launch_bounds__(kBlock) k_ebe_atomic(MeshView m, int rpad, int
                                                        Reducer red, CgCase* sc, double* ptq_out,
                                                        const int* gate_active) {
   if (gate_active && *gate_active == 0) return;
-  using E = ElemVal<T, NC>;
+  using V = typename CaseVal<T, NC>::type;
   const T* __restrict__ rec = rec_of<T>(m);
-  E dot = E::zero();
+  V dot = vzero<V>();
   const int64_t total = m.E << gshift;      // gshift: log2 of the case groups of a node, rpad / NC
   const int c = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) & ((1 << gshift) - 1)) * NC;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
@@ -104,64 +72,29 @@ __global__ void __launch_bounds__(kBlock) k_ebe_atomic(MeshView m, int rpad, int
     const int4 cn = __ldg(m.conn + e);
     const int nd[4] = {cn.x, cn.y, cn.z, cn.w};
     I off[4];
-    E P[4][3], PK[4][3];
     int fr[4];
 #pragma unroll
     for (int a = 0; a < 4; ++a) {
       off[a] = (I)nd[a] * (I)(3 * rpad) + (I)c;
       fr[a] = m.freemask[nd[a]];
-#pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        P[a][k] = E::load(pm + off[a] + (I)(k * rpad));
-        PK[a][k] = TWO ? E::load(pk + off[a] + (I)(k * rpad)) : P[a][k];
-      }
     }
-    const T* re = rec + e * kRec;
-    T g[9];
+    T r[12];
+    load_rec(rec + e * kRec, r);
+    auto ld = [&](const T* src, int a, V (&P)[3]) {
 #pragma unroll
-    for (int j = 0; j < 9; ++j) g[j] = re[j];
-    const T lam = aK * re[9], mu = aK * re[10], ms = aM * re[11];
-    // displacement gradient G_ij = sum_{b=1..3} (p_b - p_0)_i g_b,j
-    E G[3][3];
+      for (int k = 0; k < 3; ++k) P[k] = *reinterpret_cast<const V*>(src + off[a] + (I)(k * rpad));
+    };
+    auto fl = [&](int a, const V (&Q)[3]) {
 #pragma unroll
-    for (int i2 = 0; i2 < 3; ++i2) {
-      const E d1 = ev_sub(PK[1][i2], PK[0][i2]), d2 = ev_sub(PK[2][i2], PK[0][i2]), d3 = ev_sub(PK[3][i2], PK[0][i2]);
-#pragma unroll
-      for (int j = 0; j < 3; ++j) G[i2][j] = ev_fma(d3, g[6 + j], ev_fma(d2, g[3 + j], ev_mul(d1, g[j])));
-    }
-    const E ltr = ev_mul(ev_add(ev_add(G[0][0], G[1][1]), G[2][2]), lam);
-    E S[3][3];
-    const T mu2 = mu + mu;
-#pragma unroll
-    for (int i2 = 0; i2 < 3; ++i2) S[i2][i2] = ev_fma(G[i2][i2], mu2, ltr);
-    S[0][1] = S[1][0] = ev_mul(ev_add(G[0][1], G[1][0]), mu);
-    S[0][2] = S[2][0] = ev_mul(ev_add(G[0][2], G[2][0]), mu);
-    S[1][2] = S[2][1] = ev_mul(ev_add(G[1][2], G[2][1]), mu);
-    E Q[4][3];
-#pragma unroll
-    for (int b = 1; b < 4; ++b)
-#pragma unroll
-      for (int i2 = 0; i2 < 3; ++i2)
-        Q[b][i2] = ev_fma(S[i2][2], g[(b - 1) * 3 + 2], ev_fma(S[i2][1], g[(b - 1) * 3 + 1], ev_mul(S[i2][0], g[(b - 1) * 3])));
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      const E fs = ev_add(ev_add(Q[1][k], Q[2][k]), Q[3][k]);
-      const E sum = ev_add(ev_add(P[0][k], P[1][k]), ev_add(P[2][k], P[3][k]));
-      Q[0][k] = ev_sub(ev_mul(ev_add(P[0][k], sum), ms), fs);
-#pragma unroll
-      for (int a = 1; a < 4; ++a) Q[a][k] = ev_fma(ev_add(P[a][k], sum), ms, Q[a][k]);
-    }
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        if (DOT) dot = ev_fmv(P[a][k], Q[a][k], dot);
-        if (dof_free((uint8_t)fr[a], k)) Q[a][k].add_to(q + off[a] + (I)(k * rpad));
-      }
+      for (int k = 0; k < 3; ++k)
+        if (dof_free((uint8_t)fr[a], k)) atomicAdd(reinterpret_cast<V*>(q + off[a] + (I)(k * rpad)), Q[k]);
+    };
+    elem4<DOT, TWO, V, T>([&](int a, V (&P)[3]) { ld(pm, a, P); }, [&](int a, V (&P)[3]) { ld(pk, a, P); }, fl, r, aM,
+                          aK, dot);
   }
   if constexpr (DOT) {
     static_assert(NC == 1, "a thread's sum belongs to one case");
-    double v[1] = {(double)dot.v};
+    double v[1] = {(double)dot};
     if (block_reduce_last<1>(v, rpad, red)) ebe_tail(red, sc, ptq_out, rpad);
   }
 }
