@@ -12,6 +12,7 @@
 
 #include <algorithm>
 #include <mutex>
+#include <type_traits>
 #include <unordered_map>
 
 namespace fem {
@@ -582,14 +583,14 @@ __device__ __forceinline__ void tet_acc_p(const float* re, float aM, float aK, c
 // values are loaded just before its first tet and its sums leave for the tile accumulator right after its
 // second; corner 2, which closes the cycle, leaves after the first tet and is loaded again for the last,
 // so at most four corners are live at once (instead of all eight held through the hex).
-template <bool DOT>
-__device__ __forceinline__ void hex_acc_p(const float* ps, int* qs, const int (&o)[8], int rpad, const float* re,
-                                          float aM, float aK, float2 sinv, float2& hd) {
+template <bool DOT, int R>
+__device__ __forceinline__ void hex_acc_p(const float* ps, int* qs, const int (&o)[8], const float* re, float aM,
+                                          float aK, float2 sinv, float2& hd) {
   float2 P[8][3], Q[8][3];
   auto ld = [&](int sl) {
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-      P[sl][k] = *reinterpret_cast<const float2*>(ps + o[sl] + k * rpad);
+      P[sl][k] = *reinterpret_cast<const float2*>(ps + o[sl] + k * R);
       Q[sl][k] = make_float2(0.f, 0.f);
     }
   };
@@ -600,7 +601,7 @@ __device__ __forceinline__ void hex_acc_p(const float* ps, int* qs, const int (&
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
       if (DOT) hd = fma2(P[sl][k], Q[sl][k], hd);
-      int* d = qs + o[sl] + k * rpad;
+      int* d = qs + o[sl] + k * R;
       const float2 v = mul2(Q[sl][k], sinv);
       atomicAdd(d, __float2int_rn(v.x));
       atomicAdd(d + 1, __float2int_rn(v.y));
@@ -701,8 +702,8 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int tri
   return false;
 }
 
-template <typename T, bool DOT, bool SEG, int PK>
-__global__ void __launch_bounds__(kBlock, (sizeof(T) == 4 && PK != 2) ? 2 : 1) k_ebe_hex_staged(
+template <typename T, bool DOT, bool SEG>
+__global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? 2 : 1) k_ebe_hex_staged(
     HexTiles ht, MeshView m, int rpad, int rshift, const T* __restrict__ p, T* __restrict__ q, T aM, T aK, Reducer red,
     CgCase* sc, double* ptq_out, const int* gate) {
   if (gate && *gate == 0) return;
@@ -760,8 +761,7 @@ __global__ void __launch_bounds__(kBlock, (sizeof(T) == 4 && PK != 2) ? 2 : 1) k
       }
     }
   };
-  double dot = 0.0, dot1 = 0.0;   // (packed: dot1 is the second case of the thread's pair)
-  constexpr bool pk = PK != 0;
+  double dot = 0.0;
   int nd_next[2], nd_after[2];
   const int t0 = blockIdx.x;
   {
@@ -770,53 +770,16 @@ __global__ void __launch_bounds__(kBlock, (sizeof(T) == 4 && PK != 2) ? 2 : 1) k
     load_nodes(t0 + gridDim.x, nd_next);
     if (t0 < ht.n_tiles) issue(t0, 0, nd0);
   }
-  // packed: fixed-point tile sums.  Per tile and case c the scale is 2^(30 - E_c) with 2^E_c >= bound_c =
-  // (|aM| abs_m + |aK| abs_k) max |p_c| over the tile's nodes, which bounds every partial sum of element
-  // contributions to a tile node's row: the integer sums stay below 2^30, and the rounding of the sums is
-  // below 2^-31 bound_c per contribution.  spm[2][32]: the per-case maxima (|p| bit patterns, ordered as
-  // integers), one buffer per tile parity; sfwd[32]: 2^(E_c - 30), the factors back to floating point.
-  int* spm = reinterpret_cast<int*>(smem_raw + 32);
-  float* sfwd = reinterpret_cast<float*>(smem_raw + 288);
-  const float bco = fabsf((float)aM) * ht.abs_m + fabsf((float)aK) * ht.abs_k;
-  if constexpr (pk) {   // the tile accumulator starts zeroed; each flush zeroes what it reads
-    for (int i = threadIdx.x; i < (ht.nloc_max * per_node) >> 2; i += blockDim.x)
-      reinterpret_cast<float4*>(qs)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-    if ((int)threadIdx.x < 2 * 32) spm[threadIdx.x] = 0;
-  }
-  // packed: the case pairs with an active case (inner iterations; all pairs otherwise), nap of them, laid
-  // on napw >= nap item slots (a power of two, so a thread's slot, and pair, is fixed); a converged pair's
-  // product is not needed (its step length is zero)
-  uint32_t pmask = 0;
-  int nap = 0, napw = 1, lgw = 0, mypair = -1;
-  if constexpr (pk) {
-    const int npair = rpad >> 1;
-    if (DOT && sc) {
-      for (int pr = 0; pr < npair; ++pr)
-        if (sc[2 * pr].active || sc[2 * pr + 1].active) pmask |= 1u << pr;
-    } else {
-      pmask = npair >= 32 ? 0xffffffffu : ((1u << npair) - 1u);
-    }
-    nap = __popc(pmask);
-    while (napw < nap) napw <<= 1, ++lgw;
-    const int slot = threadIdx.x & (napw - 1);
-    if (slot < nap) {   // the slot-th active pair
-      uint32_t m = pmask;
-      for (int q = 0; q < slot; ++q) m &= m - 1;
-      mypair = __ffs(m) - 1;
-    }
-  }
   for (int k = 0;; ++k) {
     const int t = t0 + k * gridDim.x;
     if (t >= ht.n_tiles) break;
     const int b = k & 1;
     const int tn = t + gridDim.x;
     if (tn < ht.n_tiles) issue(tn, b ^ 1, nd_next);
-    if constexpr (!PK) load_nodes(tn + gridDim.x, nd_after);
+    load_nodes(tn + gridDim.x, nd_after);
     const int n0 = ht.tile_node_off[t], nl = ht.tile_node_off[t + 1] - n0;
     const int h0 = ht.tile_hex_off[t], nh = ht.tile_hex_off[t + 1] - h0;
-    if constexpr (!pk) {   // (the packed flush leaves the accumulator zeroed behind it)
-      for (int i = threadIdx.x; i < nl * per_node; i += blockDim.x) qs[i] = (T)0;
-    }
+    for (int i = threadIdx.x; i < nl * per_node; i += blockDim.x) qs[i] = (T)0;
     const uint32_t bar = smem_u32(mbar + b);
     if (!mbar_wait(bar, (uint32_t)((k >> 1) & 1), g_wait_budget)) {
       atomicExch(&g_tma_timeout, 1);
@@ -826,47 +789,6 @@ __global__ void __launch_bounds__(kBlock, (sizeof(T) == 4 && PK != 2) ? 2 : 1) k
     const T* ps = psb(b);
     const T* sr = srb(b);
     const int* snode = snb(b);
-    float2 sinv = make_float2(1.f, 1.f);
-    if constexpr (pk) {
-      // per-case largest |p| of the staged tile (a thread's values all belong to case threadIdx.x mod rpad)
-      const float* pf = reinterpret_cast<const float*>(ps);
-      float mx = 0.f;
-      for (int i = threadIdx.x; i < nl * per_node; i += blockDim.x) mx = fmaxf(mx, fabsf(pf[i]));
-      for (int off = 16; off >= rpad; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-      int* spm_b = spm + (b << 5);
-      if ((int)(threadIdx.x & 31) < rpad) atomicMax(spm_b + (threadIdx.x & 31), __float_as_int(mx));
-      if ((int)threadIdx.x < rpad) spm[((b ^ 1) << 5) + threadIdx.x] = 0;   // the next tile's buffer
-      __syncthreads();
-      // E_c: the exponent field of bound_c gives bound_c < 2^(field - 126)
-      auto expo = [&](int c) {
-        const uint32_t f = (__float_as_uint(bco * __int_as_float(spm_b[c])) >> 23) & 0xffu;
-        return f == 0u ? -126 : (int)f - 126;
-      };
-      auto pow2 = [](int e) { return __uint_as_float((uint32_t)min(max(e + 127, 1), 254) << 23); };
-      if (mypair >= 0) sinv = make_float2(pow2(30 - expo(2 * mypair)), pow2(30 - expo(2 * mypair + 1)));
-      if ((int)threadIdx.x < rpad) sfwd[threadIdx.x] = pow2(expo(threadIdx.x) - 30);
-    }
-    if constexpr (pk) {
-      // items (hex, active-pair slot); a thread's slot and pair are fixed (blockDim.x is a multiple of napw)
-      const int items = mypair >= 0 ? nh << lgw : 0;
-      const int c0 = mypair << 1;
-      float2 tdot2 = make_float2(0.f, 0.f);
-      uint4 lw_next = (int)threadIdx.x < items ? __ldg(ht.hex_local + h0 + (threadIdx.x >> lgw)) : make_uint4(0, 0, 0, 0);
-      for (int it = threadIdx.x; it < items; it += blockDim.x) {
-        const int hl = it >> lgw;
-        const uint4 lw = lw_next;
-        if (it + (int)blockDim.x < items) lw_next = __ldg(ht.hex_local + h0 + ((it + blockDim.x) >> lgw));
-        const int o[8] = {(int)(lw.x & 0xffff) * per_node + c0, (int)(lw.x >> 16) * per_node + c0,
-                          (int)(lw.y & 0xffff) * per_node + c0, (int)(lw.y >> 16) * per_node + c0,
-                          (int)(lw.z & 0xffff) * per_node + c0, (int)(lw.z >> 16) * per_node + c0,
-                          (int)(lw.w & 0xffff) * per_node + c0, (int)(lw.w >> 16) * per_node + c0};
-        hex_acc_p<DOT>(reinterpret_cast<const float*>(ps), reinterpret_cast<int*>(qs), o, rpad,
-                       reinterpret_cast<const float*>(sr) + hl * 6 * kRec, (float)aM, (float)aK, sinv, tdot2);
-      }
-      dot += (double)tdot2.x;
-      dot1 += (double)tdot2.y;
-      load_nodes(tn + gridDim.x, nd_after);   // (after the items: fewer registers live through them)
-    } else {
     T tdot = 0;
     const int items = nh << rshift;
     const int rounds_end = seg ? ((items + blockDim.x - 1) / blockDim.x) * blockDim.x : items;
@@ -903,30 +825,7 @@ __global__ void __launch_bounds__(kBlock, (sizeof(T) == 4 && PK != 2) ? 2 : 1) k
       }
     }
     dot += (double)tdot;
-    }
     __syncthreads();
-    if constexpr (pk) {
-      // float4 pieces of the tile accumulator (four cases of one component of one node)
-      const int sh4 = rshift - 2;
-      const int f4 = per_node >> 2;
-      for (int i = threadIdx.x; i < nl * f4; i += blockDim.x) {
-        const int l = (i >> sh4) / 3, kk = (i - l * f4) >> sh4;
-        const int raw = snode[l];
-        const int64_t g = raw & 0x0fffffff;
-        const bool fixed = !dof_free((uint8_t)((raw >> 28) & 7), kk);
-        float4* dst = reinterpret_cast<float4*>(q + g * per_node) + (i - l * f4);
-        const int4 vi = reinterpret_cast<const int4*>(qs)[i];
-        const int c4 = (i << 2) & (rpad - 1);   // the four cases of this piece: c4 .. c4 + 3
-        const float4 v = make_float4((float)vi.x * sfwd[c4], (float)vi.y * sfwd[c4 + 1], (float)vi.z * sfwd[c4 + 2],
-                                     (float)vi.w * sfwd[c4 + 3]);
-        reinterpret_cast<int4*>(qs)[i] = make_int4(0, 0, 0, 0);
-        if (raw < 0) {
-          if (!fixed) atomicAdd(dst, v);
-        } else {
-          *dst = fixed ? make_float4(0.f, 0.f, 0.f, 0.f) : v;
-        }
-      }
-    } else
     for (int i = threadIdx.x; i < nl * per_node; i += blockDim.x) {
       const int l = (i >> rshift) / 3, rem = i - l * per_node;
       const int kk = rem >> rshift;
@@ -947,36 +846,228 @@ __global__ void __launch_bounds__(kBlock, (sizeof(T) == 4 && PK != 2) ? 2 : 1) k
   if (DOT) {
     if (seg) {
       if (block_reduce_last_seg<1>(sacc, m.nseg, red)) ebe_tail_seg(red, sc, ptq_out, m.nseg);
-    } else if constexpr (pk) {
-      // slot sums over the warp's hexes, then over the warps (through the idle record buffer), then thread
-      // c < rpad takes case c (the layout of the block reduction); converged pairs give 0
-      const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-      double d0 = dot, d1 = dot1;
-      for (int off = napw; off < 32; off <<= 1) {
-        d0 += __shfl_xor_sync(0xffffffffu, d0, off);
-        d1 += __shfl_xor_sync(0xffffffffu, d1, off);
-      }
-      double* spair = reinterpret_cast<double*>(smem_raw + L.rec0);   // [warp][16 slots][2]
-      __syncthreads();
-      if (lane < napw) {
-        spair[(warp * 16 + lane) * 2] = d0;
-        spair[(warp * 16 + lane) * 2 + 1] = d1;
-      }
-      __syncthreads();
-      double vc = 0.0;
-      if ((int)threadIdx.x < rpad) {
-        const int pr = threadIdx.x >> 1;
-        if ((pmask >> pr) & 1u) {
-          const int sl = __popc(pmask & ((1u << pr) - 1u));
-          for (int w = 0; w < nw; ++w) vc += spair[(w * 16 + sl) * 2 + (threadIdx.x & 1)];
-        }
-      }
-      double v[1] = {vc};
-      if (block_reduce_last<1>(v, rpad, red)) ebe_tail(red, sc, ptq_out, rpad);
     } else {
       double v[1] = {dot};
       if (block_reduce_last<1>(v, rpad, red)) ebe_tail(red, sc, ptq_out, rpad);
     }
+  }
+}
+
+// ------------------------------------------------------------------------------------------------------
+// The packed form (FP32, R >= 4 cases, not fused groups): the same double-buffered tiles, each thread applying its
+// hex to a pair of cases.
+//
+// Fixed-point tile sums: per tile and case c the scale is 2^(30 - E_c) with 2^E_c >= bound_c = (|aM| abs_m + |aK|
+// abs_k) max |p_c| over the tile's nodes, which bounds every partial sum of element contributions to a tile node's
+// row: the integer sums stay below 2^30, and the rounding of the sums is below 2^-31 bound_c per contribution.
+//
+// What bounds it is latency (two FP32 pipe cycles an instruction, 16 warps an SM by registers, phases of a tile
+// that wait), so a tile has two block barriers (maxima -> items, items -> flush; the copies of the next tile are
+// issued after the first, when every thread has left the last flush), nothing on its critical path comes from
+// global memory (the next tile's node count and first corner table are loaded during this one), and R is a constant,
+// so the offsets of a node's values are immediates.  With four barriers, those loads at each tile's start and R at
+// run time: 16 cases on 786,432 tets 100.6 -> 93.2 us, 8 cases on 6,291,456 tets 404 -> 368 us.  Blocks of 128 threads
+// (four an SM by registers, two by the shared memory of 64-hex tiles) took 112 and 499 us, on 32-hex tiles 106 and 411.
+// ------------------------------------------------------------------------------------------------------
+template <int R, bool DOT, int MINB>
+__global__ void __launch_bounds__(kBlock, MINB) k_ebe_hex_packed(HexTiles ht, MeshView m, const float* __restrict__ p,
+                                                             float* __restrict__ q, float aM, float aK, Reducer red,
+                                                             CgCase* sc, double* ptq_out, const int* gate) {
+  if (gate && *gate == 0) return;
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  constexpr int per_node = 3 * R, F4 = per_node / 4;
+  constexpr uint32_t node_bytes = per_node * sizeof(float);
+  const StagedLayout L = staged_layout<float>(ht.nloc_max, R, ht.hex_per_tile, 0);
+  uint64_t* mbar = reinterpret_cast<uint64_t*>(smem_raw + L.bar);
+  int* qs = reinterpret_cast<int*>(smem_raw + L.qs);
+  auto psb = [&](int b) { return reinterpret_cast<float*>(smem_raw + (b ? L.ps1 : L.ps0)); };
+  auto srb = [&](int b) { return reinterpret_cast<float*>(smem_raw + (b ? L.rec1 : L.rec0)); };
+  auto snb = [&](int b) { return reinterpret_cast<int*>(smem_raw + (b ? L.node1 : L.node0)); };
+  // spm[2][32]: the per-case maxima (|p| bit patterns, ordered as integers), one buffer per tile parity;
+  // sfwd[32]: 2^(E_c - 30), the factors back to floating point
+  int* spm = reinterpret_cast<int*>(smem_raw + 32);
+  float* sfwd = reinterpret_cast<float*>(smem_raw + 288);
+  const float bco = fabsf(aM) * ht.abs_m + fabsf(aK) * ht.abs_k;
+  const int n_hex = (int)(m.E / 6);
+  if (threadIdx.x == 0) {
+    mbar_init(smem_u32(&mbar[0]), 1);
+    mbar_init(smem_u32(&mbar[1]), 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (threadIdx.x < 64) spm[threadIdx.x] = 0;
+  // the tile accumulator starts zeroed; each flush zeroes what it reads
+  for (int i = threadIdx.x; i < ht.nloc_max * F4; i += kBlock) reinterpret_cast<int4*>(qs)[i] = make_int4(0, 0, 0, 0);
+  __syncthreads();
+  // tile t: its node range, and the node entries this thread copies (tile nodes threadIdx.x and threadIdx.x + kBlock)
+  struct Nodes {
+    int nl, nd[2];
+  };
+  auto load_nodes = [&](int t, Nodes& n) {
+    n.nl = 0;
+    if (t < ht.n_tiles) {
+      const int n0 = ht.tile_node_off[t];
+      n.nl = ht.tile_node_off[t + 1] - n0;
+#pragma unroll
+      for (int j = 0; j < 2; ++j)
+        if ((int)threadIdx.x + j * kBlock < n.nl) n.nd[j] = ht.tile_nodes[n0 + threadIdx.x + j * kBlock];
+    }
+  };
+  auto hexes = [&](int t) { return min(ht.hex_per_tile, n_hex - t * ht.hex_per_tile); };
+  // bulk copies of tile t into buffer b (the buffer's previous readers have passed a block barrier)
+  auto issue = [&](int t, int b, const Nodes& n) {
+    const uint32_t bar = smem_u32(mbar + b);
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    if (threadIdx.x == 0) {
+      const uint32_t rbytes = (uint32_t)(hexes(t) * 6 * kRec * sizeof(float));
+      mbar_expect_tx(bar, rbytes + (uint32_t)n.nl * node_bytes);
+      bulk_g2s(smem_u32(srb(b)), m.rec32 + (int64_t)t * ht.hex_per_tile * 6 * kRec, rbytes, bar);
+    }
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const int l = threadIdx.x + j * kBlock;
+      if (l < n.nl) {
+        snb(b)[l] = n.nd[j];
+        bulk_g2s(smem_u32(psb(b) + l * per_node), p + (int64_t)(n.nd[j] & 0x0fffffff) * per_node, node_bytes, bar);
+      }
+    }
+  };
+  // the case pairs with an active case (inner iterations; all pairs otherwise), nap of them, laid on napw >= nap
+  // item slots (a power of two, so a thread's slot, and pair, is fixed); a converged pair's product is not needed
+  // (its step length is zero)
+  uint32_t pmask = 0;
+  int napw = 1, lgw = 0, mypair = -1;
+  {
+    constexpr int npair = R >> 1;
+    if (DOT && sc) {
+      for (int pr = 0; pr < npair; ++pr)
+        if (sc[2 * pr].active || sc[2 * pr + 1].active) pmask |= 1u << pr;
+    } else {
+      pmask = (1u << npair) - 1u;
+    }
+    const int nap = __popc(pmask);
+    while (napw < nap) napw <<= 1, ++lgw;
+    const int slot = threadIdx.x & (napw - 1);
+    if (slot < nap) {   // the slot-th active pair
+      uint32_t mm = pmask;
+      for (int u = 0; u < slot; ++u) mm &= mm - 1;
+      mypair = __ffs(mm) - 1;
+    }
+  }
+  const int c0 = mypair << 1;
+  auto expo = [&](int mx) {   // the exponent field of bound_c gives bound_c < 2^(field - 126)
+    const uint32_t f = (__float_as_uint(bco * __int_as_float(mx)) >> 23) & 0xffu;
+    return f == 0u ? -126 : (int)f - 126;
+  };
+  auto pow2 = [](int e) { return __uint_as_float((uint32_t)min(max(e + 127, 1), 254) << 23); };
+  auto first_corners = [&](int t) {
+    return t < ht.n_tiles && mypair >= 0 && (int)(threadIdx.x >> lgw) < hexes(t)
+               ? __ldg(ht.hex_local + (int64_t)t * ht.hex_per_tile + (threadIdx.x >> lgw))
+               : make_uint4(0, 0, 0, 0);
+  };
+  const int t0 = blockIdx.x;
+  Nodes nx{};       // nodes of the next tile to copy
+  int nl = 0;
+  {
+    Nodes n0{};
+    load_nodes(t0, n0);
+    load_nodes(t0 + gridDim.x, nx);
+    nl = n0.nl;
+    if (t0 < ht.n_tiles) issue(t0, 0, n0);
+  }
+  uint4 lw_next = first_corners(t0);
+  double dot0 = 0.0, dot1 = 0.0;
+  for (int k = 0;; ++k) {
+    const int t = t0 + k * gridDim.x;
+    if (t >= ht.n_tiles) break;
+    const int b = k & 1, tn = t + gridDim.x;
+    const uint32_t bar = smem_u32(mbar + b);
+    if (!mbar_wait(bar, (uint32_t)((k >> 1) & 1), g_wait_budget)) {
+      atomicExch(&g_tma_timeout, 1);
+      mbar_wait(bar, (uint32_t)((k >> 1) & 1));   // second bounded wait for the copies still in flight
+    }
+    const float* ps = psb(b);
+    const int* snode = snb(b);
+    {
+      // per-case largest |p| of the staged tile (a thread's values all belong to case threadIdx.x mod R)
+      float mx = 0.f;
+      for (int i = threadIdx.x; i < nl * per_node; i += kBlock) mx = fmaxf(mx, fabsf(ps[i]));
+      for (int off = 16; off >= R; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+      if ((int)(threadIdx.x & 31) < R) atomicMax(spm + (b << 5) + (threadIdx.x & 31), __float_as_int(mx));
+    }
+    __syncthreads();
+    const int nl_next = nx.nl;
+    if (tn < ht.n_tiles) issue(tn, b ^ 1, nx);
+    float2 sinv = make_float2(1.f, 1.f);
+    if (mypair >= 0) sinv = make_float2(pow2(30 - expo(spm[(b << 5) + c0])), pow2(30 - expo(spm[(b << 5) + c0 + 1])));
+    if ((int)threadIdx.x < R) {
+      sfwd[threadIdx.x] = pow2(expo(spm[(b << 5) + threadIdx.x]) - 30);
+      spm[((b ^ 1) << 5) + threadIdx.x] = 0;   // the next tile's buffer (last read before the previous flush)
+    }
+    {
+      // items (hex, active-pair slot); a thread's slot and pair are fixed (kBlock is a multiple of napw)
+      const int items = mypair >= 0 ? hexes(t) << lgw : 0;
+      float2 tdot2 = make_float2(0.f, 0.f);
+      for (int it = threadIdx.x; it < items; it += kBlock) {
+        const int hl = it >> lgw;
+        const uint4 lw = lw_next;
+        if (it + kBlock < items) lw_next = __ldg(ht.hex_local + (int64_t)t * ht.hex_per_tile + ((it + kBlock) >> lgw));
+        const int o[8] = {(int)(lw.x & 0xffff) * per_node + c0, (int)(lw.x >> 16) * per_node + c0,
+                          (int)(lw.y & 0xffff) * per_node + c0, (int)(lw.y >> 16) * per_node + c0,
+                          (int)(lw.z & 0xffff) * per_node + c0, (int)(lw.z >> 16) * per_node + c0,
+                          (int)(lw.w & 0xffff) * per_node + c0, (int)(lw.w >> 16) * per_node + c0};
+        hex_acc_p<DOT, R>(ps, qs, o, srb(b) + hl * 6 * kRec, aM, aK, sinv, tdot2);
+      }
+      dot0 += (double)tdot2.x;
+      dot1 += (double)tdot2.y;
+    }
+    // (after the items: fewer registers live through them)
+    load_nodes(tn + gridDim.x, nx);
+    lw_next = first_corners(tn);
+    __syncthreads();
+    // float4 pieces of the tile accumulator (four cases of one component of one node)
+    for (int i = threadIdx.x; i < nl * F4; i += kBlock) {
+      const int l = i / F4, j = i - l * F4, kk = 4 * j / R, c4 = (i << 2) & (R - 1);
+      const int raw = snode[l];
+      const bool fixed = !dof_free((uint8_t)((raw >> 28) & 7), kk);
+      float4* dst = reinterpret_cast<float4*>(q + (int64_t)(raw & 0x0fffffff) * per_node) + j;
+      const int4 vi = reinterpret_cast<const int4*>(qs)[i];
+      const float4 v = make_float4((float)vi.x * sfwd[c4], (float)vi.y * sfwd[c4 + 1], (float)vi.z * sfwd[c4 + 2],
+                                   (float)vi.w * sfwd[c4 + 3]);
+      reinterpret_cast<int4*>(qs)[i] = make_int4(0, 0, 0, 0);
+      if (raw < 0) {
+        if (!fixed) atomicAdd(dst, v);
+      } else {
+        *dst = fixed ? make_float4(0.f, 0.f, 0.f, 0.f) : v;
+      }
+    }
+    nl = nl_next;
+  }
+  if (DOT) {
+    // slot sums over the warp's hexes, then over the warps (through the idle record buffer), then thread
+    // c < R takes case c (the layout of the block reduction); converged pairs give 0
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    double d0 = dot0, d1 = dot1;
+    for (int off = napw; off < 32; off <<= 1) {
+      d0 += __shfl_xor_sync(0xffffffffu, d0, off);
+      d1 += __shfl_xor_sync(0xffffffffu, d1, off);
+    }
+    double* spair = reinterpret_cast<double*>(smem_raw + L.rec0);   // [warp][16 slots][2]
+    __syncthreads();
+    if (lane < napw) {
+      spair[(warp * 16 + lane) * 2] = d0;
+      spair[(warp * 16 + lane) * 2 + 1] = d1;
+    }
+    __syncthreads();
+    double vc = 0.0;
+    if ((int)threadIdx.x < R) {
+      const int pr = threadIdx.x >> 1;
+      if ((pmask >> pr) & 1u) {
+        const int sl = __popc(pmask & ((1u << pr) - 1u));
+        for (int w = 0; w < kBlock / 32; ++w) vc += spair[(w * 16 + sl) * 2 + (threadIdx.x & 1)];
+      }
+    }
+    double v[1] = {vc};
+    if (block_reduce_last<1>(v, R, red)) ebe_tail(red, sc, ptq_out, R);
   }
 }
 
@@ -1172,27 +1263,45 @@ cudaError_t launch_ebe_hex_staged(const HexTiles& ht, const MeshView& m, int rpa
   if (err != cudaSuccess) return err;
   const int rs = log2i(rpad);
   const int nsm = sm_count();
-  int per_sm = 1;
-  // packed pairs: FP32 only, one case per lane of the node row (not fused groups), a 16-byte aligned output
-  // (the tile flush writes float4 pieces); 1: registers capped for two blocks per SM, 2: one block per SM
-  const int pk = (sizeof(T) == 4 && !m.seg && rpad >= 4 && (reinterpret_cast<uintptr_t>(q) & 15) == 0) ? packed : 0;
-  auto kfn = red ? (m.seg ? k_ebe_hex_staged<T, true, true, 0> : k_ebe_hex_staged<T, true, false, 0>)
-                 : k_ebe_hex_staged<T, false, false, 0>;
-  if constexpr (sizeof(T) == 4) {
-    if (pk == 1) kfn = red ? k_ebe_hex_staged<T, true, false, 1> : k_ebe_hex_staged<T, false, false, 1>;
-    if (pk == 2) kfn = red ? k_ebe_hex_staged<T, true, false, 2> : k_ebe_hex_staged<T, false, false, 2>;
-  }
-  err = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (err == cudaSuccess) err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kfn, kBlock, smem);
-  if (err != cudaSuccess) return err;
-  if (per_sm < 1) per_sm = 1;
-  int grid = nsm * per_sm;
-  if (grid > ht.n_tiles) grid = ht.n_tiles;
-  if (grid > red_grid_cap()) grid = red_grid_cap();
   Reducer rd = red ? *red : Reducer{nullptr, nullptr, nullptr};
-  kfn<<<grid, kBlock, smem, s>>>(ht, m, rpad, rs, p, q, (T)aM, (T)aK, rd, red ? sc : nullptr, red ? ptq_out : nullptr,
-                                 gate);
-  return cudaGetLastError();
+  CgCase* csc = red ? sc : nullptr;
+  double* cptq = red ? ptq_out : nullptr;
+  auto run = [&](auto kfn, int block, auto launch) {
+    int per_sm = 1;
+    cudaError_t e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kfn, block, smem);
+    if (e != cudaSuccess) return e;
+    if (per_sm < 1) per_sm = 1;
+    int grid = nsm * per_sm;
+    if (grid > ht.n_tiles) grid = ht.n_tiles;
+    if (grid > red_grid_cap()) grid = red_grid_cap();
+    launch(kfn, grid, block);
+    return cudaGetLastError();
+  };
+  // packed pairs: FP32 only, one case per lane of the node row (not fused groups), a 16-byte aligned output
+  // (the tile flush writes float4 pieces); 1: registers capped for 16 warps an SM, 2: one block per SM
+  if constexpr (sizeof(T) == 4) {
+    if (packed && !m.seg && rpad >= 4 && (reinterpret_cast<uintptr_t>(q) & 15) == 0) {
+      auto go = [&](auto kfn, int grid, int block) {
+        kfn<<<grid, block, smem, s>>>(ht, m, p, q, (float)aM, (float)aK, rd, csc, cptq, gate);
+      };
+      auto by = [&](auto r) {
+        constexpr int R = decltype(r)::value;
+        if (packed == 2) return red ? run(k_ebe_hex_packed<R, true, 1>, kBlock, go) : run(k_ebe_hex_packed<R, false, 1>, kBlock, go);
+        return red ? run(k_ebe_hex_packed<R, true, 2>, kBlock, go) : run(k_ebe_hex_packed<R, false, 2>, kBlock, go);
+      };
+      switch (rpad) {
+        case 4: return by(std::integral_constant<int, 4>{});
+        case 8: return by(std::integral_constant<int, 8>{});
+        case 16: return by(std::integral_constant<int, 16>{});
+        default: return by(std::integral_constant<int, 32>{});
+      }
+    }
+  }
+  return run(red ? (m.seg ? k_ebe_hex_staged<T, true, true> : k_ebe_hex_staged<T, true, false>) : k_ebe_hex_staged<T, false, false>,
+             kBlock, [&](auto kfn, int grid, int block) {
+               kfn<<<grid, block, smem, s>>>(ht, m, rpad, rs, p, q, (T)aM, (T)aK, rd, csc, cptq, gate);
+             });
 }
 template cudaError_t launch_ebe_hex_staged<double>(const HexTiles&, const MeshView&, int, const double*, double*,
                                                    double, double, const Reducer*, CgCase*, double*, const int*,
