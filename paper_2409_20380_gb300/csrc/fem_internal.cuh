@@ -189,6 +189,11 @@ cudaError_t launch_elem_tile(int npe, const ElemTiles& et, int64_t E, int rpad, 
 // Grid of grid-stride kernel `fn` (blocks of `block` threads, no dynamic shared memory): at most one wave of
 // the blocks that fit on the GPU at once, so no partial second wave.
 int grid_resident(const void* fn, int block, int64_t items);
+// Block of the reducing vector kernels: kVecBlock, halved while that spreads few items over at most 64 blocks (more
+// blocks cost the last one more partial sums than they save) of at least 64 threads and 4 rpad (the reductions'
+// slices).  The FP64 forms run at two lanes a clock and SM: ten FP64 steps of the 729-node box, whose k_update<double>
+// ran 2 blocks of 512 threads, 3.71 -> 3.45 ms.
+int vec_block(int64_t items, int rpad);
 
 cudaError_t launch_elem_setup(int64_t E, int64_t N, const double* xyz, const int4* conn, const int32_t* mat,
                               int n_mat, const double* lmr, double* rec64, float* rec32, int* err_flag,

@@ -13,8 +13,8 @@ template <typename T> __device__ __forceinline__ const T* binv_of(const MeshView
 template <> __device__ __forceinline__ const double* binv_of<double>(const MeshView& m) { return m.binv64; }
 template <> __device__ __forceinline__ const float* binv_of<float>(const MeshView& m) { return m.binv32; }
 
-static int vec_grid(int64_t items) {
-  int64_t g = (items + kVecBlock - 1) / kVecBlock;
+static int vec_grid(int64_t items, int block) {
+  int64_t g = (items + block - 1) / block;
   if (g < 1) g = 1;
   if (g > vec_grid_cap()) g = vec_grid_cap();
   return (int)g;
@@ -444,7 +444,8 @@ template <typename T>
 cudaError_t launch_norm_b_gated(const MeshView& m, int rpad, const T* b, Reducer red, CgCase* sc,
                                 const CgCase* gate, double tol, cudaStream_t s) {
   const int rs = log2i(rpad);
-  k_norm_b<T><<<vec_grid(m.N << rs), kVecBlock, 0, s>>>(m, rpad, rs, b, red, sc, gate, tol);
+  const int vb = vec_block(m.N << rs, rpad);
+  k_norm_b<T><<<vec_grid(m.N << rs, vb), vb, 0, s>>>(m, rpad, rs, b, red, sc, gate, tol);
   return cudaGetLastError();
 }
 
@@ -452,7 +453,8 @@ template <typename T>
 cudaError_t launch_resid(const MeshView& m, int rpad, const T* b, const T* q, T* x, T* r, T* z, int first,
                          Reducer red, CgCase* sc, int* n_active, double tol, int maxit, cudaStream_t s) {
   const int rs = log2i(rpad);
-  k_resid<T><<<vec_grid(m.N << rs), kVecBlock, 0, s>>>(m, rpad, rs, b, q, x, r, z, first, red, sc, n_active, tol, maxit);
+  const int vb = vec_block(m.N << rs, rpad);
+  k_resid<T><<<vec_grid(m.N << rs, vb), vb, 0, s>>>(m, rpad, rs, b, q, x, r, z, first, red, sc, n_active, tol, maxit);
   return cudaGetLastError();
 }
 
@@ -468,7 +470,8 @@ template <typename T>
 cudaError_t launch_update(const MeshView& m, int rpad, const T* p, const T* q, T* x, T* r, T* z, Reducer red,
                           CgCase* sc, int* n_active, double tol, int maxit, cudaStream_t s) {
   const int rs = log2i(rpad);
-  k_update<T><<<vec_grid(m.N << rs), kVecBlock, 0, s>>>(m, rpad, rs, p, q, x, r, z, red, sc, n_active, tol, maxit);
+  const int vb = vec_block(m.N << rs, rpad);
+  k_update<T><<<vec_grid(m.N << rs, vb), vb, 0, s>>>(m, rpad, rs, p, q, x, r, z, red, sc, n_active, tol, maxit);
   return cudaGetLastError();
 }
 
@@ -476,7 +479,8 @@ template <typename T>
 cudaError_t launch_dir_defer(const MeshView& m, int rpad, const T* r, T* p, T* x, const CgCase* sc,
                              const int* n_active, cudaStream_t s) {
   const int rs = log2i(rpad);
-  k_dir_defer<T><<<vec_grid(m.N << rs), kVecBlock, 0, s>>>(m, rpad, rs, r, p, x, sc, n_active);
+  const int vb = vec_block(m.N << rs, rpad);
+  k_dir_defer<T><<<vec_grid(m.N << rs, vb), vb, 0, s>>>(m, rpad, rs, r, p, x, sc, n_active);
   return cudaGetLastError();
 }
 
@@ -484,7 +488,9 @@ template <typename T>
 cudaError_t launch_update_defer(const MeshView& m, int rpad, const T* q, T* r, Reducer red, CgCase* sc,
                                 int* n_active, int maxit, cudaStream_t s) {
   const int rs = log2i(rpad);
-  k_update_defer<T><<<grid_resident((const void*)k_update_defer<T>, kVecBlock, m.N << rs), kVecBlock, 0, s>>>(m, rpad, rs, q, r, red, sc, n_active, maxit);
+  const int vb = vec_block(m.N << rs, rpad);
+  const int grid = vb == kVecBlock ? grid_resident((const void*)k_update_defer<T>, kVecBlock, m.N << rs) : vec_grid(m.N << rs, vb);
+  k_update_defer<T><<<grid, vb, 0, s>>>(m, rpad, rs, q, r, red, sc, n_active, maxit);
   return cudaGetLastError();
 }
 template cudaError_t launch_dir_defer<float>(const MeshView&, int, const float*, float*, float*, const CgCase*,
@@ -503,7 +509,8 @@ cudaError_t launch_outer_resid(const MeshView& m, int rpad, const double* b, con
                                Reducer red, CgCase* outer, int* n_active, double tol, double inner_max, double aim,
                                cudaStream_t s) {
   const int rs = log2i(rpad);
-  k_outer_resid<<<vec_grid(m.N << rs), kVecBlock, 0, s>>>(m, rpad, rs, b, q, r32, red, outer, n_active, tol, inner_max,
+  const int vb = vec_block(m.N << rs, rpad);
+  k_outer_resid<<<vec_grid(m.N << rs, vb), vb, 0, s>>>(m, rpad, rs, b, q, r32, red, outer, n_active, tol, inner_max,
                                                           aim);
   return cudaGetLastError();
 }

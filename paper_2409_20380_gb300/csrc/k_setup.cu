@@ -56,6 +56,12 @@ int vec_grid_cap() { return std::min(3 * sm_count(), kMaxRedBlocks); }
 int red_grid_cap() { return std::min(8 * sm_count(), kMaxRedBlocks); }
 int wide_grid_cap() { return 16 * sm_count(); }
 
+int vec_block(int64_t items, int rpad) {
+  int b = kVecBlock;
+  while (b > 64 && b / 2 >= 4 * rpad && items <= (int64_t)(b / 2) * 64) b >>= 1;
+  return b;
+}
+
 int grid_for(int64_t items, int cap) {
   if (cap < 0) cap = red_grid_cap();
   int64_t g = (items + kBlock - 1) / kBlock;

@@ -86,11 +86,9 @@ template <typename E> __device__ __forceinline__ const E* snap_slot(const E* rin
 }
 
 
-static int vec_grid(int64_t items) {
-  int64_t g = (items + kVecBlock - 1) / kVecBlock;
-  if (g < 1) g = 1;
-  if (g > vec_grid_cap()) g = vec_grid_cap();
-  return (int)g;
+// Grid of a reducing vector kernel with blocks of `block` threads (vec_block).
+static int vec_grid(const void* fn, int64_t items, int block) {
+  return block == kVecBlock ? grid_resident(fn, kVecBlock, items) : (int)((items + block - 1) / block);
 }
 
 static int log2i(int r) {
@@ -1119,13 +1117,13 @@ cudaError_t launch_r0(const MeshView& m, int rpad, double dt, const double* b, c
                       const double* Av2, const double* Av1, const float* qy, float* r32, Reducer red, CgCase* outer,
                       int* n_active, double tol, double inner_max, double aim, cudaStream_t s, Ring4 avr,
                       const StepCtl* ctl, CgCase* inner, bool guard, int* fallbacks) {
-  const int rs = log2i(rpad);
+  const int rs = log2i(rpad), vb = vec_block(m.N << rs, rpad);
   if (guard && qy) {
-    k_r0<true><<<grid_resident((const void*)k_r0<true>, kVecBlock, m.N << rs), kVecBlock, 0, s>>>(
+    k_r0<true><<<vec_grid((const void*)k_r0<true>, m.N << rs, vb), vb, 0, s>>>(
         m, rpad, rs, dt / 24.0, b, Av4, Av3, Av2, Av1, qy, r32, red, outer, n_active, tol, inner_max, aim, avr, ctl,
         inner, fallbacks);
   } else {
-    k_r0<false><<<grid_resident((const void*)k_r0<false>, kVecBlock, m.N << rs), kVecBlock, 0, s>>>(
+    k_r0<false><<<vec_grid((const void*)k_r0<false>, m.N << rs, vb), vb, 0, s>>>(
         m, rpad, rs, dt / 24.0, b, Av4, Av3, Av2, Av1, qy, r32, red, outer, n_active, tol, inner_max, aim, avr, ctl,
         inner, nullptr);
   }
@@ -1143,7 +1141,8 @@ cudaError_t launch_cert(const MeshView& m, int rpad, double cM, double cK, const
                         const double* qK, float* r32, Reducer red, CgCase* outer, int* n_active, double tol,
                         double inner_max, double aim, cudaStream_t s, CgCase* inner) {
   const int rs = log2i(rpad);
-  k_cert<<<grid_resident((const void*)k_cert, kVecBlock, m.N << rs), kVecBlock, 0, s>>>(m, rpad, rs, cM, cK, b, qM, qK, r32, red, outer, n_active, tol,
+  const int vb = vec_block(m.N << rs, rpad);
+  k_cert<<<vec_grid((const void*)k_cert, m.N << rs, vb), vb, 0, s>>>(m, rpad, rs, cM, cK, b, qM, qK, r32, red, outer, n_active, tol,
                                                 inner_max, aim, inner);
   return cudaGetLastError();
 }
