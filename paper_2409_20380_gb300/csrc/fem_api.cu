@@ -422,19 +422,18 @@ struct fem_mesh {
       if (t.variant) *variant = t.variant, *hpt = t.hpt;
     }
     if (*variant == 0 && *hpt == 0 && hex && !seg) {
-      // Automatic choice on hex patches by the work H x r (hexes x cases), both sides measured alone:
+      // Automatic choice on hex patches by the hexes H and the cases r, both sides measured alone:
       //   FP32: packed staged tiles (5), with 1 or 2 cases (no 16-byte node rows) unstaged tiles, but the element
       //   kernel for those up to H r = 8192 (H = 512, r = 1: 8.4 us against 12.2; 4096: 10.8 against 12.8; 15,283:
       //   17.8 against 14.7), where the tiles would leave most SMs idle.
-      //   FP64 (bound by the FP64 pipe): tiles of at most 128 hexes from H r = 500,000 on (131,072 hexes, 4
-      //   cases: 711 us against 728 staged, 761 element kernel), the element kernel below, whose threads spread
-      //   over all SMs (512 hexes, 1 case: 12.5 us against 33.5 for 64-hex tiles and 103 for one 512-hex tile;
-      //   15,283 hexes, 16 cases: 359 against 401).
-      const int64_t work = (E / 6) * rpad;
+      //   FP64 (bound by the FP64 pipe): tiles of at most 128 hexes from 50,000 hexes on, three tiles an SM
+      //   (110,593 hexes, 4 cases: 586 us against 620 staged, 638 element kernel; 1 case 153 against 204, 178), the
+      //   element kernel below, whose threads spread over all SMs (512 hexes, 1 case: 12.5 us against 33.5 for 64-hex
+      //   tiles and 103 for one 512-hex tile; 15,283 hexes, 16 cases: 354 against 403).
       if (elem_bytes == 4) {
-        if (rpad <= 2 && work <= 8192) *variant = 1;
+        if (rpad <= 2 && (E / 6) * rpad <= 8192) *variant = 1;
       } else {
-        *variant = work < 500000 ? 1 : 2;
+        *variant = E / 6 < 50000 ? 1 : 2;
         *hpt = *variant == 2 ? 128 : 0;
         if (*variant == 2 && !tiles_for(elem_bytes, rpad, 2, 128)) *hpt = 0;
       }
