@@ -275,9 +275,10 @@ cudaError_t launch_r0_seg(const MeshView& m, double dt, const double* b, const d
 cudaError_t launch_cert_seg(const MeshView& m, double cM, double cK, const double* b, const double* qM, const double* qK,
                             float* r32, Reducer red, CgCase* outer, int* n_active, double tol, double inner_floor,
                             double aim, cudaStream_t s);
-// x = 0 on Dirichlet DOFs and for cases with ||b|| = 0.
+// x = 0 on Dirichlet DOFs and for cases with ||b|| = 0; *nonzero (nullable) = 1 when a value other than zero is left.
 template <typename T>
-cudaError_t launch_zero_b0_t(const MeshView& m, int rpad, T* x, const CgCase* sc, cudaStream_t s);
+cudaError_t launch_zero_b0_t(const MeshView& m, int rpad, T* x, const CgCase* sc, cudaStream_t s,
+                             int* nonzero = nullptr);
 cudaError_t launch_extract_case(int64_t N, int rpad, int c, const double* src, double* dst, cudaStream_t s);
 
 // Time stepping (FP64 [N][3][rpad]).

@@ -416,29 +416,40 @@ __global__ void k_refine_pending(int64_t n_items, int rpad, int ncase, double* _
   }
 }
 
-// x = 0 on Dirichlet DOFs and for cases whose right-hand side is zero (||b|| = 0 gives x = 0).
+// x = 0 on Dirichlet DOFs and for cases whose right-hand side is zero (||b|| = 0 gives x = 0).  nonzero (nullable, 0
+// on entry): set when a value other than zero (a NaN too) is left.
 template <typename T>
-__global__ void k_zero_b0(MeshView m, int rpad, int rshift, T* __restrict__ x, const CgCase* __restrict__ sc) {
+__global__ void k_zero_b0(MeshView m, int rpad, int rshift, T* __restrict__ x, const CgCase* __restrict__ sc,
+                          int* __restrict__ nonzero) {
   const int64_t total = m.N << rshift;
+  bool nz = false;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
     const int64_t n = i >> rshift;
     const int c = (int)(i & (rpad - 1));
     const uint8_t f = m.freemask[n];
     const bool z = sc[c].bb == 0.0;
-    for (int k = 0; k < 3; ++k)
-      if (z || !dof_free(f, k)) x[(n * 3 + k) * rpad + c] = (T)0;
+    for (int k = 0; k < 3; ++k) {
+      const int64_t id = (n * 3 + k) * rpad + c;
+      if (z || !dof_free(f, k)) x[id] = (T)0;
+      else if (nonzero) nz = nz || !(x[id] == (T)0);
+    }
   }
+  if (nonzero && __any_sync(0xffffffffu, nz) && (threadIdx.x & 31) == 0) atomicOr(nonzero, 1);
 }
 
 // ---- launchers ----
 template <typename T>
-cudaError_t launch_zero_b0_t(const MeshView& m, int rpad, T* x, const CgCase* sc, cudaStream_t s) {
+cudaError_t launch_zero_b0_t(const MeshView& m, int rpad, T* x, const CgCase* sc, cudaStream_t s, int* nonzero) {
   const int rs = log2i(rpad);
-  k_zero_b0<T><<<grid_for(m.N << rs), kBlock, 0, s>>>(m, rpad, rs, x, sc);
+  if (nonzero) {
+    const cudaError_t e = cudaMemsetAsync(nonzero, 0, sizeof(int), s);
+    if (e != cudaSuccess) return e;
+  }
+  k_zero_b0<T><<<grid_for(m.N << rs), kBlock, 0, s>>>(m, rpad, rs, x, sc, nonzero);
   return cudaGetLastError();
 }
-template cudaError_t launch_zero_b0_t<double>(const MeshView&, int, double*, const CgCase*, cudaStream_t);
-template cudaError_t launch_zero_b0_t<float>(const MeshView&, int, float*, const CgCase*, cudaStream_t);
+template cudaError_t launch_zero_b0_t<double>(const MeshView&, int, double*, const CgCase*, cudaStream_t, int*);
+template cudaError_t launch_zero_b0_t<float>(const MeshView&, int, float*, const CgCase*, cudaStream_t, int*);
 
 template <typename T>
 cudaError_t launch_norm_b_gated(const MeshView& m, int rpad, const T* b, Reducer red, CgCase* sc,

@@ -113,3 +113,34 @@ def test_pcg_edge_cases(torch_dev):
             fem.pcg_solve(h, b, x, 4, fem.fem_opts_default(tol=-1.0))
     finally:
         fem.fem_mesh_destroy(h)
+
+
+@pytest.mark.parametrize("precision", [fem.FEM_FP64, fem.FEM_FP32_INNER])
+@pytest.mark.parametrize("variant", [0, 1, 8])
+@pytest.mark.parametrize("guess", ["zero", "one value", "nan"])
+def test_pcg_initial_guess(torch_dev, precision, variant, guess):
+    """The product of the initial guess is left out exactly when the guess is zero: one value in one case, far from
+    zero, still enters its residual (the solution is the same to the solve's tolerance, 1e-12 against 1e-9), and a NaN
+    is reported."""
+    torch = torch_dev
+    m, tp, sysm, A, bs = _setup((7, 5, 4), 4, seed=3)
+    h = fem.fem_mesh_create(m, tp)
+    try:
+        fem.fem_mesh_tune(h, variant, 0)
+        b = torch.tensor(from_cases(bs, m.n_nodes, 4), device="cuda")
+        x = torch.zeros_like(b)
+        opts = fem.fem_opts_default(precision=precision, tol=1e-12)
+        fem.pcg_solve(h, b, torch.ones_like(b), 4, opts)      # (leaves a product in the workspace)
+        if guess != "zero":
+            x[int(sysm.free[-1]) * 4 + 2] = 1e3 if guess == "one value" else float("nan")
+        if guess == "nan":
+            with pytest.raises(fem.FemError):
+                fem.pcg_solve(h, b, x, 4, opts)
+            return
+        fem.pcg_solve(h, b, x, 4, opts)
+        xs = to_cases(x.cpu().numpy(), m.n_nodes, 4)
+        for c in range(4):
+            ref = spla.spsolve(A.tocsc(), bs[c][sysm.free])
+            assert np.linalg.norm(xs[c][sysm.free] - ref) <= 1e-9 * np.linalg.norm(ref)
+    finally:
+        fem.fem_mesh_destroy(h)
