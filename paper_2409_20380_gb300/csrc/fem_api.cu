@@ -7,6 +7,7 @@
 #include <cstring>
 #include <string>
 #include <thread>
+#include <mutex>
 #include <vector>
 
 #include "fem_internal.cuh"
@@ -263,6 +264,9 @@ struct fem_mesh {
   int32_t* reg_gap = nullptr;
   int reg_lead = 0;
   std::vector<Workspace*> ws;
+  // stream-ordered scratch of fem_mesh_split_product (created on first use, given back with the mesh)
+  cudaMemPool_t pool = nullptr;
+  std::mutex pool_mu;
   // tiled hex-patch EBE (present when the elements come in Kuhn hex patches)
   bool hex = false;
   static constexpr int kNTile = 5;
@@ -408,6 +412,7 @@ struct fem_mesh {
     dfree(binv64); dfree(binv32); dfree(fm); dfree(reg_lo); dfree(reg_hi); dfree(reg_gap); dfree(seg); dfree(reg_cent);
     dfree(ab_node); dfree(ab_c64); dfree(ab_c32);
     for (auto* w : ws) delete w;
+    if (pool) cudaMemPoolDestroy(pool);
     for (void* b : tile_bufs) cudaFree(b);
     free_elem_tiles(&et);
   }
@@ -474,6 +479,29 @@ struct fem_mesh {
       if (!best || t.n_tiles >= sm_count()) best = &t;
     }
     return best;
+  }
+  // `bytes` of device memory for work on s alone, to be freed by cudaFreeAsync on s: calls on several threads and
+  // streams each have their own, and the pool keeps what they gave back for the next one.
+  fem_status scratch(void** out, size_t bytes, cudaStream_t s) {
+    std::lock_guard<std::mutex> lk(pool_mu);
+    if (!pool) {
+      cudaMemPoolProps props{};
+      props.allocType = cudaMemAllocationTypePinned;
+      props.location.type = cudaMemLocationTypeDevice;
+      props.location.id = device;
+      uint64_t keep = UINT64_MAX;
+      if (cudaMemPoolCreate(&pool, &props) != cudaSuccess) {
+        cudaGetLastError();
+        pool = nullptr;
+        return fail(FEM_ERR_OOM, "memory pool");
+      }
+      cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+    }
+    if (cudaMallocFromPoolAsync(out, bytes, pool, s) != cudaSuccess) {
+      cudaGetLastError();
+      return fail(FEM_ERR_OOM, "device allocation of " + std::to_string(bytes) + " bytes failed");
+    }
+    return FEM_OK;
   }
   fem_status workspace(int rpad, Workspace** out) {
     for (auto* w : ws)
@@ -2212,15 +2240,22 @@ fem_status fem_mesh_split_product(fem_mesh* m, int mode, const double* p_dev, do
   cudaStream_t s = (cudaStream_t)stream;
   float2* pdf = nullptr;
   if (mode >= 2) CHK(m->ensure_bcsr(s));
-  if (mode == 3) CHK(dalloc(&pdf, (size_t)m->N * 3 * n_rhs));
+  if (mode == 3) {
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
+      cudaGetLastError();
+      return fail(FEM_ERR_OOM, "fem_mesh_split_product: mode 3 allocates and cannot be captured");
+    }
+    CHK(m->scratch((void**)&pdf, sizeof(float2) * (size_t)m->N * 3 * n_rhs, s));
+  }
   cudaError_t e = split_product(m, mode, n_rhs, p_dev, pdf, qM_dev, qK_dev, s);
   if (e == cudaSuccess && mode < 2) {   // the element forms leave Dirichlet rows to their consumers
     e = launch_mask<double>(m->N, n_rhs, m->fm, qM_dev, s);
     if (e == cudaSuccess) e = launch_mask<double>(m->N, n_rhs, m->fm, qK_dev, s);
   }
   if (pdf) {
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    dfree(pdf);
+    const cudaError_t ef = cudaFreeAsync(pdf, s);
+    if (e == cudaSuccess) e = ef;
   }
   if (e != cudaSuccess) {
     cudaGetLastError();
