@@ -667,7 +667,7 @@ static fem_status pcg_core(fem_mesh* m, Workspace* w, const T* b, T* x, T* r, T*
     for (int k = 0; k < check_every; ++k) {
       int p0 = w->pbeg(P_VEC, s);
       if (defer) {
-        if constexpr (sizeof(T) == 4) CU(launch_dir_defer<float>(mv, rpad, r, p, x, sc, w->n_active, s));
+        if constexpr (sizeof(T) == 4) CU(launch_dir_defer(mv, rpad, r, p, x, sc, w->n_active, s));
       } else if (sg) {
         CU(launch_dir_seg<T>(mv, z, p, sc, w->n_active, s));
       } else {
@@ -679,7 +679,7 @@ static fem_status pcg_core(fem_mesh* m, Workspace* w, const T* b, T* x, T* r, T*
       w->pend(p1, s);
       int p2 = w->pbeg(P_VEC, s);
       if (defer) {
-        if constexpr (sizeof(T) == 4) CU(launch_update_defer<float>(mv, rpad, q, r, red, sc, w->n_active, maxit, s));
+        if constexpr (sizeof(T) == 4) CU(launch_update_defer(mv, rpad, q, r, red, sc, w->n_active, maxit, s));
       } else if (sg) {
         CU(launch_update_seg<T>(mv, p, q, x, r, z, red, sc, w->n_active, maxit, s));
       } else {
@@ -1547,7 +1547,7 @@ static cudaError_t capture_step(fem_batch* bt, Group* g) {
           if (sg) {
             GE(launch_dir_seg<float>(mv, w->z32, w->p32, w->sc, w->n_active, s4));
           } else {
-            GE(launch_dir_defer<float>(mv, rpad, w->r32, w->p32, w->x32, w->sc, w->n_active, s4));
+            GE(launch_dir_defer(mv, rpad, w->r32, w->p32, w->x32, w->sc, w->n_active, s4));
           }
           GE(ebe_product<float>(m, rpad, w->p32, w->q32, m->cM, m->cK, &red, w->sc, nullptr, w->n_active, s4, true,
                                 tc_loop));
@@ -1555,7 +1555,7 @@ static cudaError_t capture_step(fem_batch* bt, Group* g) {
             GE(launch_update_seg<float>(mv, w->p32, w->q32, w->x32, w->rr32, w->z32, red, w->sc, w->n_active,
                                         o.maxit, s4));
           } else {
-            GE(launch_update_defer<float>(mv, rpad, w->q32, w->r32, red, w->sc, w->n_active, o.maxit, s4));
+            GE(launch_update_defer(mv, rpad, w->q32, w->r32, red, w->sc, w->n_active, o.maxit, s4));
           }
         }
         GE(launch_inner_cond(w->n_active, ctl, h_in, ce, o.maxit + 64 * ce, n_inner, s4));

@@ -239,11 +239,9 @@ cudaError_t launch_update(const MeshView& m, int rpad, const T* p, const T* q, T
 // Deferred-update iteration of the FP32 inner solves (no true-residual test): the direction pass forms
 // z = B^{-1} r and applies the previous x += alpha p; the update pass only advances r.  x is complete
 // after launch_refine_pending, which adds each case's last alpha p.
-template <typename T>
-cudaError_t launch_dir_defer(const MeshView& m, int rpad, const T* r, T* p, T* x, const CgCase* sc,
+cudaError_t launch_dir_defer(const MeshView& m, int rpad, const float* r, float* p, float* x, const CgCase* sc,
                              const int* n_active, cudaStream_t s);
-template <typename T>
-cudaError_t launch_update_defer(const MeshView& m, int rpad, const T* q, T* r, Reducer red, CgCase* sc,
+cudaError_t launch_update_defer(const MeshView& m, int rpad, const float* q, float* r, Reducer red, CgCase* sc,
                                 int* n_active, int maxit, cudaStream_t s);
 cudaError_t launch_refine_pending(const MeshView& m, int rpad, int ncase, double* x, const float* d32,
                                   const float* p32, CgCase* outer, const CgCase* inner, cudaStream_t s);
