@@ -468,6 +468,10 @@ struct fem_mesh {
       } else if (variant == 3 || variant == 5 || variant == 6) {   // (6: one block per SM)
         need = elem_bytes == 4 ? ebe_hex_staged_smem<float>(t, view(), rpad) : ebe_hex_staged_smem<double>(t, view(), rpad);
         budget = variant == 6 ? 220 * 1024 : 110 * 1024;
+        if (variant == 5 && elem_bytes == 4 && need <= budget) {   // two blocks of the packed form still fit an SM
+          need += ebe_hex_packed_extra(t);
+          budget = 113 * 1024;
+        }
       } else if (variant == 4) {   // one block per SM
         need = elem_bytes == 4 ? ebe_hex_cm_smem<float>(t, view(), rpad) : ebe_hex_cm_smem<double>(t, view(), rpad);
         budget = 220 * 1024;

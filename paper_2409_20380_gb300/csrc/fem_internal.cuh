@@ -351,6 +351,7 @@ cudaError_t launch_ebe_hex_staged(const HexTiles& ht, const MeshView& m, int rpa
                                   cudaStream_t s, int packed = 0);
 template <typename T>
 size_t ebe_hex_staged_smem(const HexTiles& ht, const MeshView& m, int rpad);   // ~0 when not applicable
+size_t ebe_hex_packed_extra(const HexTiles& ht);   // more, for the packed form
 // Case-major staged variant: warps of 32 hexes of one case; converged cases (sc[c].active == 0) skipped.
 template <typename T>
 cudaError_t launch_ebe_hex_cm(const HexTiles& ht, const MeshView& m, int rpad, const T* p, T* q, double aM, double aK,
@@ -671,9 +672,10 @@ __device__ __forceinline__ void warp_case_sums(const double (*sh)[kVecBlock], in
   }
 }
 
+// The same with the caller's shared memory: sh[NQ][kVecBlock], 8-byte aligned, free when every thread arrives.
 template <int NQ>
-__device__ __forceinline__ bool block_reduce_last(double (&vals)[NQ], int rpad, const Reducer& red) {
-  __shared__ double sh[NQ][kVecBlock];
+__device__ __forceinline__ bool block_reduce_last_in(double (*sh)[kVecBlock], double (&vals)[NQ], int rpad,
+                                                     const Reducer& red) {
   __shared__ bool am_last;
   const int V = NQ * rpad;
 #pragma unroll
@@ -710,6 +712,11 @@ __device__ __forceinline__ bool block_reduce_last(double (&vals)[NQ], int rpad, 
   if (threadIdx.x == 0) *red.counter = 0u;
   __syncthreads();
   return true;
+}
+template <int NQ>
+__device__ __forceinline__ bool block_reduce_last(double (&vals)[NQ], int rpad, const Reducer& red) {
+  __shared__ double sh[NQ][kVecBlock];
+  return block_reduce_last_in<NQ>(sh, vals, rpad, red);
 }
 
 }  // namespace fem

@@ -589,9 +589,9 @@ __device__ __forceinline__ void tet_acc_p(const float* re, float aM, float aK, c
 // values are loaded just before its first tet and its sums leave for the tile accumulator right after its
 // second; corner 2, which closes the cycle, leaves after the first tet and is loaded again for the last,
 // so at most four corners are live at once (instead of all eight held through the hex).
-template <bool DOT, int R>
+template <int R>
 __device__ __forceinline__ void hex_acc_p(const float* ps, int* qs, const int (&o)[8], const float* re, float aM,
-                                          float aK, float2 sinv, float2& hd) {
+                                          float aK, float2 sinv) {
   float2 P[8][3], Q[8][3];
   auto ld = [&](int sl) {
 #pragma unroll
@@ -606,7 +606,6 @@ __device__ __forceinline__ void hex_acc_p(const float* ps, int* qs, const int (&
   auto fl = [&](int sl) {
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-      if (DOT) hd = fma2(P[sl][k], Q[sl][k], hd);
       int* d = qs + o[sl] + k * R;
       const float2 v = mul2(Q[sl][k], sinv);
       atomicAdd(d, __float2int_rn(v.x));
@@ -870,11 +869,18 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? 2 : 1) k_ebe_hex_stag
 // What bounds it is latency (two FP32 pipe cycles an instruction, 16 warps an SM by registers, phases of a tile
 // that wait), so a tile has two block barriers (maxima -> items, items -> flush; the copies of the next tile are
 // issued after the first, when every thread has left the last flush), nothing on its critical path comes from
-// global memory (the next tile's node count and first corner table are loaded during this one), and R is a constant,
-// so the offsets of a node's values are immediates.  With four barriers, those loads at each tile's start and R at
-// run time: 16 cases on 786,432 tets 100.6 -> 93.2 us, 8 cases on 6,291,456 tets 404 -> 368 us.  Blocks of 128 threads
+// global memory (the next tile's node list is loaded during this one, its corner table comes with its records), and R is
+// a constant, so the offsets of a node's values are immediates.  With four barriers, those loads at each tile's start and R at
+// run time: 16 cases on 786,432 tets 100.6 -> 93.2 us, 8 cases on 6,291,456 tets 404 -> 368 us (with p^T q).  No register
+// may be missing either: with corner tables in registers, the active pairs' slots kept live and p^T q in the items the
+// compiler spilled and loaded tables late, a fifth of the time; 98.8 -> 90.3 and 374 -> 338 us without.  Blocks of 128 threads
 // (four an SM by registers, two by the shared memory of 64-hex tiles) took 112 and 499 us, on 32-hex tiles 106 and 411.
 // ------------------------------------------------------------------------------------------------------
+// What it keeps in shared memory behind the staged layout: two buffers of corner tables, p^T q by thread, the
+// table of active pairs.
+__host__ __device__ inline size_t packed_extra(int hex_per_tile) {
+  return 2 * (size_t)hex_per_tile * sizeof(uint4) + kBlock * sizeof(double) + 80;
+}
 template <int R, bool DOT, int MINB>
 __global__ void __launch_bounds__(kBlock, MINB) k_ebe_hex_packed(HexTiles ht, MeshView m, const float* __restrict__ p,
                                                              float* __restrict__ q, float aM, float aK, Reducer red,
@@ -889,6 +895,8 @@ __global__ void __launch_bounds__(kBlock, MINB) k_ebe_hex_packed(HexTiles ht, Me
   auto psb = [&](int b) { return reinterpret_cast<float*>(smem_raw + (b ? L.ps1 : L.ps0)); };
   auto srb = [&](int b) { return reinterpret_cast<float*>(smem_raw + (b ? L.rec1 : L.rec0)); };
   auto snb = [&](int b) { return reinterpret_cast<int*>(smem_raw + (b ? L.node1 : L.node0)); };
+  auto slb = [&](int b) { return reinterpret_cast<uint4*>(smem_raw + L.total) + b * ht.hex_per_tile; };
+  double* sdot = reinterpret_cast<double*>(smem_raw + L.total + 2 * sizeof(uint4) * ht.hex_per_tile);
   // spm[2][32]: the per-case maxima (|p| bit patterns, ordered as integers), one buffer per tile parity;
   // sfwd[32]: 2^(E_c - 30), the factors back to floating point
   int* spm = reinterpret_cast<int*>(smem_raw + 32);
@@ -925,8 +933,10 @@ __global__ void __launch_bounds__(kBlock, MINB) k_ebe_hex_packed(HexTiles ht, Me
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     if (threadIdx.x == 0) {
       const uint32_t rbytes = (uint32_t)(hexes(t) * 6 * kRec * sizeof(float));
-      mbar_expect_tx(bar, rbytes + (uint32_t)n.nl * node_bytes);
+      const uint32_t lbytes = (uint32_t)(hexes(t) * sizeof(uint4));
+      mbar_expect_tx(bar, rbytes + lbytes + (uint32_t)n.nl * node_bytes);
       bulk_g2s(smem_u32(srb(b)), m.rec32 + (int64_t)t * ht.hex_per_tile * 6 * kRec, rbytes, bar);
+      bulk_g2s(smem_u32(slb(b)), ht.hex_local + (int64_t)t * ht.hex_per_tile, lbytes, bar);
     }
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
@@ -940,36 +950,31 @@ __global__ void __launch_bounds__(kBlock, MINB) k_ebe_hex_packed(HexTiles ht, Me
   // the case pairs with an active case (inner iterations; all pairs otherwise), nap of them, laid on napw >= nap
   // item slots (a power of two, so a thread's slot, and pair, is fixed); a converged pair's product is not needed
   // (its step length is zero)
-  uint32_t pmask = 0;
-  int napw = 1, lgw = 0, mypair = -1;
-  {
-    constexpr int npair = R >> 1;
-    if (DOT && sc) {
+  // (held in shared memory and read where they are needed)
+  constexpr int npair = R >> 1;
+  volatile int* slots = reinterpret_cast<volatile int*>(sdot + kBlock);   // log2 napw, then the pair of each slot
+  if (DOT) {
+    if (threadIdx.x == 0) {
+      int nap = 0, lg = 0;
       for (int pr = 0; pr < npair; ++pr)
-        if (sc[2 * pr].active || sc[2 * pr + 1].active) pmask |= 1u << pr;
-    } else {
-      pmask = (1u << npair) - 1u;
+        if (!sc || sc[2 * pr].active || sc[2 * pr + 1].active) slots[1 + nap++] = pr;
+      while ((1 << lg) < nap) ++lg;
+      for (; nap < npair; ++nap) slots[1 + nap] = -1;
+      slots[0] = lg;
     }
-    const int nap = __popc(pmask);
-    while (napw < nap) napw <<= 1, ++lgw;
-    const int slot = threadIdx.x & (napw - 1);
-    if (slot < nap) {   // the slot-th active pair
-      uint32_t mm = pmask;
-      for (int u = 0; u < slot; ++u) mm &= mm - 1;
-      mypair = __ffs(mm) - 1;
-    }
+    __syncthreads();
   }
-  const int c0 = mypair << 1;
+  constexpr int kLgPairs = R == 32 ? 4 : R == 16 ? 3 : R == 8 ? 2 : 1;
+  auto lg_slots = [&]() { return DOT ? slots[0] : kLgPairs; };
+  auto my_pair = [&]() {
+    const int slot = threadIdx.x & ((1 << lg_slots()) - 1);
+    return DOT ? slots[1 + slot] : slot;
+  };
   auto expo = [&](int mx) {   // the exponent field of bound_c gives bound_c < 2^(field - 126)
     const uint32_t f = (__float_as_uint(bco * __int_as_float(mx)) >> 23) & 0xffu;
     return f == 0u ? -126 : (int)f - 126;
   };
   auto pow2 = [](int e) { return __uint_as_float((uint32_t)min(max(e + 127, 1), 254) << 23); };
-  auto first_corners = [&](int t) {
-    return t < ht.n_tiles && mypair >= 0 && (int)(threadIdx.x >> lgw) < hexes(t)
-               ? __ldg(ht.hex_local + (int64_t)t * ht.hex_per_tile + (threadIdx.x >> lgw))
-               : make_uint4(0, 0, 0, 0);
-  };
   const int t0 = blockIdx.x;
   Nodes nx{};       // nodes of the next tile to copy
   int nl = 0;
@@ -980,8 +985,11 @@ __global__ void __launch_bounds__(kBlock, MINB) k_ebe_hex_packed(HexTiles ht, Me
     nl = n0.nl;
     if (t0 < ht.n_tiles) issue(t0, 0, n0);
   }
-  uint4 lw_next = first_corners(t0);
-  double dot0 = 0.0, dot1 = 0.0;
+  // p^T q is taken in the flush from the tile's sums and staged values (taken in the items it cost 19 us at 16 cases on
+  // 786,432 tets, here 11: the items run at the FP32 pipe's rate with no register to spare).  A thread's pieces belong
+  // to cases c4 .. c4 + 3; sums of them in FP32 over 4 lanes, each of which goes on with one of the cases in FP64
+  // (which runs at two lanes a clock and SM).
+  if (DOT) sdot[threadIdx.x] = 0.0;
   for (int k = 0;; ++k) {
     const int t = t0 + k * gridDim.x;
     if (t >= ht.n_tiles) break;
@@ -1003,77 +1011,66 @@ __global__ void __launch_bounds__(kBlock, MINB) k_ebe_hex_packed(HexTiles ht, Me
     __syncthreads();
     const int nl_next = nx.nl;
     if (tn < ht.n_tiles) issue(tn, b ^ 1, nx);
-    float2 sinv = make_float2(1.f, 1.f);
-    if (mypair >= 0) sinv = make_float2(pow2(30 - expo(spm[(b << 5) + c0])), pow2(30 - expo(spm[(b << 5) + c0 + 1])));
     if ((int)threadIdx.x < R) {
       sfwd[threadIdx.x] = pow2(expo(spm[(b << 5) + threadIdx.x]) - 30);
       spm[((b ^ 1) << 5) + threadIdx.x] = 0;   // the next tile's buffer (last read before the previous flush)
     }
     {
       // items (hex, active-pair slot); a thread's slot and pair are fixed (kBlock is a multiple of napw)
-      const int items = mypair >= 0 ? hexes(t) << lgw : 0;
-      float2 tdot2 = make_float2(0.f, 0.f);
-      for (int it = threadIdx.x; it < items; it += kBlock) {
-        const int hl = it >> lgw;
-        const uint4 lw = lw_next;
-        if (it + kBlock < items) lw_next = __ldg(ht.hex_local + (int64_t)t * ht.hex_per_tile + ((it + kBlock) >> lgw));
-        const int o[8] = {(int)(lw.x & 0xffff) * per_node + c0, (int)(lw.x >> 16) * per_node + c0,
-                          (int)(lw.y & 0xffff) * per_node + c0, (int)(lw.y >> 16) * per_node + c0,
-                          (int)(lw.z & 0xffff) * per_node + c0, (int)(lw.z >> 16) * per_node + c0,
-                          (int)(lw.w & 0xffff) * per_node + c0, (int)(lw.w >> 16) * per_node + c0};
-        hex_acc_p<DOT, R>(ps, qs, o, srb(b) + hl * 6 * kRec, aM, aK, sinv, tdot2);
+      const int pr = my_pair();
+      if (pr >= 0) {
+        const int c0 = pr << 1, nh = hexes(t);
+        const float2 sinv = make_float2(pow2(30 - expo(spm[(b << 5) + c0])), pow2(30 - expo(spm[(b << 5) + c0 + 1])));
+        for (int hl = threadIdx.x >> lg_slots(); hl < nh; hl += kBlock >> lg_slots()) {
+          const uint4 lw = slb(b)[hl];
+          const int o[8] = {(int)(lw.x & 0xffff) * per_node + c0, (int)(lw.x >> 16) * per_node + c0,
+                            (int)(lw.y & 0xffff) * per_node + c0, (int)(lw.y >> 16) * per_node + c0,
+                            (int)(lw.z & 0xffff) * per_node + c0, (int)(lw.z >> 16) * per_node + c0,
+                            (int)(lw.w & 0xffff) * per_node + c0, (int)(lw.w >> 16) * per_node + c0};
+          hex_acc_p<R>(ps, qs, o, srb(b) + hl * 6 * kRec, aM, aK, sinv);
+        }
       }
-      dot0 += (double)tdot2.x;
-      dot1 += (double)tdot2.y;
     }
     // (after the items: fewer registers live through them)
     load_nodes(tn + gridDim.x, nx);
-    lw_next = first_corners(tn);
     __syncthreads();
     // float4 pieces of the tile accumulator (four cases of one component of one node)
+    const int c4 = (threadIdx.x << 2) & (R - 1);
+    const float w4[4] = {sfwd[c4], sfwd[c4 + 1], sfwd[c4 + 2], sfwd[c4 + 3]};
+    float td[4] = {0.f, 0.f, 0.f, 0.f};
     for (int i = threadIdx.x; i < nl * F4; i += kBlock) {
-      const int l = i / F4, j = i - l * F4, kk = 4 * j / R, c4 = (i << 2) & (R - 1);
+      const int l = i / F4, j = i - l * F4, kk = 4 * j / R;
       const int raw = snode[l];
       const bool fixed = !dof_free((uint8_t)((raw >> 28) & 7), kk);
       float4* dst = reinterpret_cast<float4*>(q + (int64_t)(raw & 0x0fffffff) * per_node) + j;
       const int4 vi = reinterpret_cast<const int4*>(qs)[i];
-      const float4 v = make_float4((float)vi.x * sfwd[c4], (float)vi.y * sfwd[c4 + 1], (float)vi.z * sfwd[c4 + 2],
-                                   (float)vi.w * sfwd[c4 + 3]);
+      const float4 v = make_float4((float)vi.x * w4[0], (float)vi.y * w4[1], (float)vi.z * w4[2], (float)vi.w * w4[3]);
       reinterpret_cast<int4*>(qs)[i] = make_int4(0, 0, 0, 0);
+      if (DOT) {   // (the tile's rows: sum over its elements of p_e^T A_e p_e)
+        const float4 pv = reinterpret_cast<const float4*>(ps)[i];
+        td[0] = fmaf(pv.x, v.x, td[0]), td[1] = fmaf(pv.y, v.y, td[1]);
+        td[2] = fmaf(pv.z, v.z, td[2]), td[3] = fmaf(pv.w, v.w, td[3]);
+      }
       if (raw < 0) {
         if (!fixed) atomicAdd(dst, v);
       } else {
         *dst = fixed ? make_float4(0.f, 0.f, 0.f, 0.f) : v;
       }
     }
+    if (DOT) {
+      const bool hi = threadIdx.x & (R / 2), lo = threadIdx.x & (R / 4);
+      const float a0 = (hi ? td[2] : td[0]) + __shfl_xor_sync(0xffffffffu, hi ? td[0] : td[2], R / 2);
+      const float a1 = (hi ? td[3] : td[1]) + __shfl_xor_sync(0xffffffffu, hi ? td[1] : td[3], R / 2);
+      const float a = (lo ? a1 : a0) + __shfl_xor_sync(0xffffffffu, lo ? a0 : a1, R / 4);
+      sdot[(threadIdx.x & ~(R - 1)) + c4 + (hi ? 2 : 0) + (lo ? 1 : 0)] += (double)a;   // (its own word)
+    }
     nl = nl_next;
   }
   if (DOT) {
-    // slot sums over the warp's hexes, then over the warps (through the idle record buffer), then thread
-    // c < R takes case c (the layout of the block reduction); converged pairs give 0
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    double d0 = dot0, d1 = dot1;
-    for (int off = napw; off < 32; off <<= 1) {
-      d0 += __shfl_xor_sync(0xffffffffu, d0, off);
-      d1 += __shfl_xor_sync(0xffffffffu, d1, off);
-    }
-    double* spair = reinterpret_cast<double*>(smem_raw + L.rec0);   // [warp][16 slots][2]
     __syncthreads();
-    if (lane < napw) {
-      spair[(warp * 16 + lane) * 2] = d0;
-      spair[(warp * 16 + lane) * 2 + 1] = d1;
-    }
-    __syncthreads();
-    double vc = 0.0;
-    if ((int)threadIdx.x < R) {
-      const int pr = threadIdx.x >> 1;
-      if ((pmask >> pr) & 1u) {
-        const int sl = __popc(pmask & ((1u << pr) - 1u));
-        for (int w = 0; w < kBlock / 32; ++w) vc += spair[(w * 16 + sl) * 2 + (threadIdx.x & 1)];
-      }
-    }
-    double v[1] = {vc};
-    if (block_reduce_last<1>(v, R, red)) ebe_tail(red, sc, ptq_out, R);
+    double v[1] = {sdot[threadIdx.x]};   // (of case threadIdx.x mod R)
+    // (in the memory of the tile sums, no longer needed)
+    if (block_reduce_last_in<1>(reinterpret_cast<double(*)[kVecBlock]>(smem_raw + L.qs), v, R, red)) ebe_tail(red, sc, ptq_out, R);
   }
 }
 
@@ -1257,13 +1254,14 @@ size_t ebe_hex_staged_smem(const HexTiles& ht, const MeshView& m, int rpad) {
   return staged_layout<T>(ht.nloc_max, rpad, ht.hex_per_tile, m.seg ? m.nseg : 0).total;
 }
 template size_t ebe_hex_staged_smem<float>(const HexTiles&, const MeshView&, int);
+size_t ebe_hex_packed_extra(const HexTiles& ht) { return packed_extra(ht.hex_per_tile); }
 template size_t ebe_hex_staged_smem<double>(const HexTiles&, const MeshView&, int);
 
 template <typename T>
 cudaError_t launch_ebe_hex_staged(const HexTiles& ht, const MeshView& m, int rpad, const T* p, T* q, double aM,
                                   double aK, const Reducer* red, CgCase* sc, double* ptq_out, const int* gate,
                                   cudaStream_t s, int packed) {
-  const size_t smem = ebe_hex_staged_smem<T>(ht, m, rpad);
+  size_t smem = ebe_hex_staged_smem<T>(ht, m, rpad);
   if (smem == ~(size_t)0 || (reinterpret_cast<uintptr_t>(p) & 15) != 0) return cudaErrorInvalidValue;
   cudaError_t err = cudaMemsetAsync(q, 0, sizeof(T) * (size_t)m.N * 3 * rpad, s);
   if (err != cudaSuccess) return err;
@@ -1288,6 +1286,7 @@ cudaError_t launch_ebe_hex_staged(const HexTiles& ht, const MeshView& m, int rpa
   // (the tile flush writes float4 pieces); 1: registers capped for 16 warps an SM, 2: one block per SM
   if constexpr (sizeof(T) == 4) {
     if (packed && !m.seg && rpad >= 4 && (reinterpret_cast<uintptr_t>(q) & 15) == 0) {
+      smem += packed_extra(ht.hex_per_tile);
       auto go = [&](auto kfn, int grid, int block) {
         kfn<<<grid, block, smem, s>>>(ht, m, p, q, (float)aM, (float)aK, rd, csc, cptq, gate);
       };
