@@ -742,7 +742,7 @@ __device__ __forceinline__ float zr_node(const float* __restrict__ B, float r0, 
 // astray at the onset of a wave) drops it (CgCase::guess = 2, fallbacks[c] += 1), and k_guard_fix then
 // rewrites that case's r32 and guess.
 template <bool ALT>
-__global__ void __launch_bounds__(kVecBlock, 2) k_r0(MeshView m, int rpad, int rshift, double h, const double* __restrict__ b,
+__global__ void __launch_bounds__(kVecBlock, 1) k_r0(MeshView m, int rpad, int rshift, double h, const double* __restrict__ b,
                                                const double* __restrict__ Av4, const double* __restrict__ Av3,
                                                const double* __restrict__ Av2, const double* __restrict__ Av1,
                                                const float* __restrict__ qy, float* __restrict__ r32, Reducer red,
@@ -761,18 +761,27 @@ __global__ void __launch_bounds__(kVecBlock, 2) k_r0(MeshView m, int rpad, int r
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
     const int64_t n = i >> rshift;
     const int c = (int)(i & (rpad - 1));
-    const uint8_t f = m.freemask[n];
     float rf[3], fa[3];
+    // every load of the node before its free-DOF bits are looked at (16 cases on 139,425 nodes 129 -> 125 us)
+    double bk[3], v1[3], v2[3], v3[3], v4[3];
+    float qk[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const int64_t id = (n * 3 + k) * rpad + c;
+      bk[k] = b[id], v4[k] = Av4[id], v3[k] = Av3[id], v2[k] = Av2[id], v1[k] = Av1[id];
+      if (qy) qk[k] = qy[id];
+    }
+    const uint8_t f = m.freemask[n];
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
       const int64_t id = (n * 3 + k) * rpad + c;
       double v = 0.0;
       float qv = 0.f;
-      const double bv = b[id];
+      const double bv = bk[k];
       if (dof_free(f, k)) {
-        v = fma(w1, Av1[id], fma(w2, Av2[id], fma(w3, Av3[id], fma(w4, Av4[id], bv))));
+        v = fma(w1, v1[k], fma(w2, v2[k], fma(w3, v3[k], fma(w4, v4[k], bv))));
         if (qy) {
-          qv = qy[id];
+          qv = qk[k];
           v -= f2d(qv);
         }
       }
@@ -948,6 +957,8 @@ __global__ void __launch_bounds__(kVecBlock, 2) k_cert(MeshView m, int rpad, int
 // the next step's Adams-Bashforth and guess residual read); 2 the state side (u, a, K u, Pb: what the next
 // right-hand side reads), run after part 1 so that it may overlap the Gram row.  Part 2 finds M v already
 // updated and uses  -4/dt Mv = 4/dt Mv' - (8/dt^2) qM  in the Pb recurrence.
+// The FP64 pipe bounds it (two lanes a clock and SM): chains of FMAs, 14 operations a value instead of 16, and every
+// load ahead of the stores: 6.7e6 values 246 -> 221 us, 25.6e6 918 -> 823 us (the 160 bytes a value take 158 and 603).
 template <typename E, int P>
 __global__ void k_newmark_incr(int64_t n, double dt, double cM, double cK, double c1, double a1,
                                const double* __restrict__ du,
@@ -977,28 +988,25 @@ __global__ void k_newmark_incr(int64_t n, double dt, double cM, double cK, doubl
     auto ld = [&](const double* x) { return *reinterpret_cast<const double2*>(x + i); };
     auto st = [&](double* x, double y0, double y1) { *reinterpret_cast<double2*>(x + i) = make_double2(y0, y1); };
     const double2 d = ld(du), vp = ld(v_prev), m_ = ld(qM), k_ = ld(qK), mv = ld(Mv);
+    const double2 none = make_double2(0.0, 0.0);
+    const double2 uu = STATE ? ld(u) : none, aa = STATE ? ld(a) : none, ku = STATE ? ld(Ku) : none,
+                  pb = STATE ? ld(Pb) : none, kv = VEL ? ld(Kv) : none, ab = VEL && e_push ? ld(du_ab) : none;
     if (STATE) {
-      const double2 uu = ld(u), aa = ld(a), ku = ld(Ku), pb = ld(Pb);
       st(u, uu.x + d.x, uu.y + d.y);
-      st(a, c44 * d.x - c4 * vp.x - aa.x, c44 * d.y - c4 * vp.y - aa.y);
+      st(a, fma(c44, d.x, -fma(c4, vp.x, aa.x)), fma(c44, d.y, -fma(c4, vp.y, aa.y)));
       st(Ku, ku.x + k_.x, ku.y + k_.y);
-      if (P == 0) {
-        st(Pb, al * m_.x + be * k_.x - (pb.x + c4 * mv.x + 2.0 * ku.x),
-           al * m_.y + be * k_.y - (pb.y + c4 * mv.y + 2.0 * ku.y));
-      } else {
-        st(Pb, al2 * m_.x + be * k_.x - (pb.x - c4 * mv.x + 2.0 * ku.x),
-           al2 * m_.y + be * k_.y - (pb.y - c4 * mv.y + 2.0 * ku.y));
-      }
+      auto pb_next = [&](double mq, double kq, double pbo, double mvo, double kuo) {
+        return fma(P == 0 ? al : al2, mq, fma(be, kq, -fma(P == 0 ? c4 : -c4, mvo, fma(2.0, kuo, pbo))));
+      };
+      st(Pb, pb_next(m_.x, k_.x, pb.x, mv.x, ku.x), pb_next(m_.y, k_.y, pb.y, mv.y, ku.y));
     }
     if (VEL) {
-      const double2 kv = ld(Kv);
       st(v_push, c2 * d.x - vp.x, c2 * d.y - vp.y);
       const double mv2x = c2 * m_.x - mv.x, kv2x = c2 * k_.x - kv.x, mv2y = c2 * m_.y - mv.y, kv2y = c2 * k_.y - kv.y;
       st(Mv, mv2x, mv2y);
       st(Kv, kv2x, kv2y);
       st(Av_push, cM * mv2x + cK * kv2x, cM * mv2y + cK * kv2y);
       if (e_push) {
-        const double2 ab = ld(du_ab);
         store_snap2(e_push, slot_stride, i, d.x - ab.x, d.y - ab.y);
       }
     }
