@@ -218,7 +218,9 @@ fem_status fem_mesh_set_absorbing(fem_mesh* m, int64_t n_faces, const int32_t* f
 
 /*
  * Selects the EBE product implementation of a mesh (library tuning knob; the paper's EBE is one product,
- * Section 3.2, Eq. eqebefem).  ebe_variant: 0 = automatic, 1 = generic element kernel, 2 = tiled hex-patch
+ * Section 3.2, Eq. eqebefem).  ebe_variant: 0 = automatic (by the mesh's size, n_rhs and the precision), 1 = generic
+ * element kernel (on a mesh without hex patches, FP32 products of n_rhs >= 4 without p^T q sum in tiles of 256
+ * elements first), 2 = tiled hex-patch
  * kernel (available when the elements come in groups of six tets splitting a hexahedron with the Kuhn
  * topology, which fem_mesh_create detects), 3 = the tiled hex kernel with each tile's node values and
  * element records staged in shared memory first by bulk asynchronous copies (double-buffered), 4 = as 3
@@ -234,8 +236,8 @@ fem_status fem_mesh_set_absorbing(fem_mesh* m, int64_t n_faces, const int32_t* f
  * product the paper compares the EBE with, Section 3.3; built on first use and shared with the
  * certification product), FP64 blocks for FP64 products and their FP32 rounding for FP32 ones, any mesh,
  * not fused groups (those use 5, or 1 without hex patches).  hex_per_tile: 0 = automatic (largest tile
- * whose shared memory fits and that leaves a tile for every SM), or 64/128/256/512 hexes per tile.  Errors: FEM_ERR_ARG for other values or
- * variants 2-7 on a mesh without hex patches.
+ * whose shared memory fits and that leaves a tile for every SM), or 64/128/256/512 hexes per tile.  Errors:
+ * FEM_ERR_ARG for other values or variants 2-7 on a mesh without hex patches.
  */
 fem_status fem_mesh_tune(fem_mesh* m, int ebe_variant, int hex_per_tile);
 

@@ -493,7 +493,7 @@ struct fem_mesh {
       props.allocType = cudaMemAllocationTypePinned;
       props.location.type = cudaMemLocationTypeDevice;
       props.location.id = device;
-      uint64_t keep = UINT64_MAX;
+      uint64_t keep = (uint64_t)256 << 20;   // (a larger block's product takes far longer than its allocation)
       if (cudaMemPoolCreate(&pool, &props) != cudaSuccess) {
         cudaGetLastError();
         pool = nullptr;
@@ -2080,7 +2080,9 @@ static fem_status mesh_create(int64_t n_nodes, const double* xyz, int64_t n_elem
   if (!m->hex) {
     const cudaError_t ce = build_elem_tiles(
         npe, n_elems, n_nodes, npe == 10 ? m->conn10 : reinterpret_cast<const int32_t*>(m->conn), m->fm, m->rec32, &m->et, s);
-    if (ce != cudaSuccess) {
+    if (ce == cudaErrorMemoryAllocation) {
+      cudaGetLastError();   // no room for the tiles: the products take the element kernels
+    } else if (ce != cudaSuccess) {
       cudaGetLastError();
       return bail(fail(FEM_ERR_CUDA, std::string("element tiles: ") + cudaGetErrorString(ce)));
     }
