@@ -627,7 +627,7 @@ def run_ours(args):
                  "frac": fl / (avg32 * 1e-3) / 1e12 / alu32,
                  "peak_kind": "derived: %d SMs x 128 FP32 lanes x 2 flops x max SM clock" % n_sm,
                  "traffic": ncu_traffic("ebe_packed_f32_%s%d" % (args.config, rpad), EBE_SOURCES) if not args.variant else None,
-                 "kernel": ("k_ebe_hex_staged<float,1,0,1> (FP32 EBE product A p of the inner PCG, TMA-staged "
+                 "kernel": ("k_ebe_hex_packed (FP32 EBE product A p of the inner PCG, TMA-staged "
                             "hex tiles, two cases per thread; %d cases)" % rpad),
                  "avg_launch_ms": avg32, "launches": working32, "launches_issued": prof["ebe32_launches"],
                  "launch_note": "launches that did work (the slowest case's inner iterations + the correction's "
