@@ -458,7 +458,7 @@ struct fem_mesh {
       const HexTiles& t = tiles[i];
       if (t.n_tiles == 0) continue;
       if (hpt && t.hex_per_tile != hpt) continue;
-      size_t need, budget;
+      size_t need, budget, most = 220 * 1024;   // (most: for a tile size that was asked for)
       if (variant == 9) {
         need = elem_bytes == 4 ? ebe_hex_tc_smem(t, rpad) : ~(size_t)0;
         budget = 220 * 1024;
@@ -468,9 +468,10 @@ struct fem_mesh {
       } else if (variant == 3 || variant == 5 || variant == 6) {   // (6: one block per SM)
         need = elem_bytes == 4 ? ebe_hex_staged_smem<float>(t, view(), rpad) : ebe_hex_staged_smem<double>(t, view(), rpad);
         budget = variant == 6 ? 220 * 1024 : 110 * 1024;
-        if (variant == 5 && elem_bytes == 4 && need <= budget) {   // two blocks of the packed form still fit an SM
+        if (variant != 3 && elem_bytes == 4 && need <= most) {   // the packed form: two blocks an SM (6: one)
           need += ebe_hex_packed_extra(t);
-          budget = 113 * 1024;
+          most = 226 * 1024;
+          budget = variant == 6 ? most : 113 * 1024;
         }
       } else if (variant == 4) {   // one block per SM
         need = elem_bytes == 4 ? ebe_hex_cm_smem<float>(t, view(), rpad) : ebe_hex_cm_smem<double>(t, view(), rpad);
@@ -479,7 +480,7 @@ struct fem_mesh {
         need = (size_t)t.nloc_max * (3 * rpad * elem_bytes + 4);
         budget = elem_bytes == 4 ? 100 * 1024 : 200 * 1024;
       }
-      if (need > budget && !(hpt && need <= 220 * 1024)) continue;
+      if (need > budget && !(hpt && need <= most)) continue;
       if (!best || t.n_tiles >= sm_count()) best = &t;
     }
     return best;

@@ -21,13 +21,15 @@ def torch_dev():
     return torch
 
 
-def _check(torch, m, r, dtype, offset):
+def _check(torch, m, r, dtype, offset, tune=None):
     tp = wl.TimeParams()
     sysm, A = oracle.build_system(m, tp)
     cM, cK = 4.0 / tp.dt ** 2 + 2.0 * tp.a0 / tp.dt, 1.0 + 2.0 * tp.a1 / tp.dt
     vs = random_free_vectors(m, r, seed=r)
     h = fem.fem_mesh_create(m, tp)
     try:
+        if tune:
+            fem.fem_mesh_tune(h, *tune)
         n = 3 * m.n_nodes * r
         # offset 1: vectors that are not 8-byte (FP32) or 16-byte aligned
         p = torch.zeros(n + offset, dtype=dtype, device="cuda")[offset:]
@@ -67,3 +69,16 @@ def test_no_hex_patches(torch_dev, r, dtype, offset):
     order = np.random.default_rng(3).permutation(m.n_elems)
     m.conn, m.mat_id = np.ascontiguousarray(m.conn[order]), np.ascontiguousarray(m.mat_id[order])
     _check(torch_dev, m, r, getattr(torch_dev, dtype), offset)
+
+
+# Tile sizes that were asked for, at the edge of a block's shared memory: 490 nodes in a 256-hex tile (hexes in random
+# order) fit the staged form but not the packed one with its own words; 64 hexes of 8 cases fit both.
+@pytest.mark.parametrize("variant", [3, 5, 6])
+@pytest.mark.parametrize("hpt", [64, 128, 256, 512])
+@pytest.mark.parametrize("r", [4, 8, 16, 32])
+def test_requested_tile_sizes(torch_dev, variant, hpt, r):
+    m = small_mesh(6, 6, 9)
+    order = np.random.default_rng(7).permutation(m.n_elems // 6)
+    m.conn = np.ascontiguousarray(m.conn.reshape(-1, 6, 4)[order].reshape(-1, 4))
+    m.mat_id = np.ascontiguousarray(m.mat_id.reshape(-1, 6)[order].reshape(-1))
+    _check(torch_dev, m, r, torch_dev.float32, 0, (variant, hpt))
