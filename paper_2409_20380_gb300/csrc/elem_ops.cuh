@@ -13,6 +13,15 @@ __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 __device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
 
+// Fixed-point sums: a bound below 2^E takes the scale 2^(30 - E) in and 2^(E - 30) back.  E is at least -96, so that both
+// are normal FP32 numbers and their product is one (with each clamped by itself, sums of a bound below 2^-97 came back
+// doubled); a smaller bound's sums are then exact to 2^-127, half of FP32's smallest normal number, below which FP32
+// atomics flush to zero.  pow2 clamps to the normal range.
+__device__ __forceinline__ float pow2(int e) { return __uint_as_float((uint32_t)min(max(e + 127, 1), 254) << 23); }
+__device__ __forceinline__ int fixed_expo(float bound) {   // (bound < 2^(exponent field - 126))
+  return max((int)((__float_as_uint(bound) >> 23) & 0xffu) - 126, -96);
+}
+
 template <typename V> struct ScalarOf { using type = V; };
 template <> struct ScalarOf<float2> { using type = float; };
 template <typename V> __device__ __forceinline__ V vzero() { return (V)0; }

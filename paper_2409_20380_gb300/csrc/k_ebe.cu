@@ -970,11 +970,7 @@ __global__ void __launch_bounds__(kBlock, MINB) k_ebe_hex_packed(HexTiles ht, Me
     const int slot = threadIdx.x & ((1 << lg_slots()) - 1);
     return DOT ? slots[1 + slot] : slot;
   };
-  auto expo = [&](int mx) {   // the exponent field of bound_c gives bound_c < 2^(field - 126)
-    const uint32_t f = (__float_as_uint(bco * __int_as_float(mx)) >> 23) & 0xffu;
-    return f == 0u ? -126 : (int)f - 126;
-  };
-  auto pow2 = [](int e) { return __uint_as_float((uint32_t)min(max(e + 127, 1), 254) << 23); };
+  auto expo = [&](int mx) { return fixed_expo(bco * __int_as_float(mx)); };
   const int t0 = blockIdx.x;
   Nodes nx{};       // nodes of the next tile to copy
   int nl = 0;
@@ -1500,12 +1496,7 @@ __global__ void __launch_bounds__(kBlock, 2) k_ebe_hexmat(HexTiles ht, const flo
       }
     }
     __syncthreads();
-    // E_c from the exponent field of bound_c (bound_c < 2^(field - 126)); scale 2^(30 - E_c)
-    auto expo = [&](int c) {
-      const uint32_t f = (__float_as_uint(bco * __int_as_float(spm[c])) >> 23) & 0xffu;
-      return f == 0u ? -126 : (int)f - 126;
-    };
-    auto pow2 = [](int e) { return __uint_as_float((uint32_t)min(max(e + 127, 1), 254) << 23); };
+    auto expo = [&](int c) { return fixed_expo(bco * __int_as_float(spm[c])); };   // scale 2^(30 - E_c)
     const float sv = myc >= 0 ? pow2(30 - expo(myc)) : 1.f;
     const float2 sinv = make_float2(sv, sv);
     if ((int)threadIdx.x < rpad) sfwd[threadIdx.x] = pow2(expo(threadIdx.x) - 30);
@@ -2119,7 +2110,6 @@ __global__ void __launch_bounds__(kTcBlock, R == 8 ? 2 : 3) k_ebe_hex_tc(HexTile
   const uint32_t o_t1 = (uint32_t)(128 * 4 + r16);
   const uint32_t hs_u32 = smem_u32(hs);
   const float bco = fabsf(aM) * ht.abs_m + fabsf(aK) * ht.abs_k;
-  auto pow2 = [](int e) { return __uint_as_float((uint32_t)min(max(e + 127, 1), 254) << 23); };
   float4 tdot = make_float4(0.f, 0.f, 0.f, 0.f);
   double dd[4] = {0.0, 0.0, 0.0, 0.0};
   const int t0 = blockIdx.x;
@@ -2154,13 +2144,9 @@ __global__ void __launch_bounds__(kTcBlock, R == 8 ? 2 : 3) k_ebe_hex_tc(HexTile
     const int* spm_b = spm + (b << 5);
     // per case: E (the fixed-point bound 2^E), ep (max |p| < 2^ep); p enters FP16 as p 2^(14 - ep), sums
     // leave to fixed point by 2^(30 - E - (14 - ep))
-    auto expo_b = [&](int c) {
-      const uint32_t fb = (__float_as_uint(bco * __int_as_float(spm_b[c])) >> 23) & 0xffu;
-      return fb == 0u ? -126 : (int)fb - 126;
-    };
-    auto expo_p = [&](int c) {
-      const uint32_t fp = ((uint32_t)spm_b[c] >> 23) & 0xffu;
-      return fp == 0u ? -126 : (int)fp - 126;
+    auto expo_b = [&](int c) { return fixed_expo(bco * __int_as_float(spm_b[c])); };
+    auto expo_p = [&](int c) {   // (2^(14 - ep) is in FP32's range too)
+      return max((int)(((uint32_t)spm_b[c] >> 23) & 0xffu) - 126, -112);
     };
     float s_in[R / 8], f_out0[R / 8], f_out1[R / 8];
 #pragma unroll

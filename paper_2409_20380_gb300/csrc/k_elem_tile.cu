@@ -233,9 +233,8 @@ __global__ void __launch_bounds__(kBlock, NPE == 4 ? 4 : 2) k_elem_tile(ElemTile
     for (int i = threadIdx.x * 16; i < ne * kRec * 4; i += kBlock * 16) cp_async16(smem + L.rec + b * L.rec_sz + i, gr + i);
     for (int i = threadIdx.x * 16; i < ne * NPE * 2; i += kBlock * 16) cp_async16(smem + L.loc + b * L.loc_sz + i, gl + i);
   };
-  auto pow2 = [](int x) { return __uint_as_float((uint32_t)min(max(x + 127, 1), 254) << 23); };
   auto field = [&](int m) { return (int)((__float_as_uint(bco * __int_as_float(m)) >> 23) & 0xffu); };
-  auto expo = [](int f) { return f == 0 ? -126 : f - 126; };         // bound < 2^expo
+  auto expo = [](int f) { return max(f - 126, -96); };               // bound < 2^expo (fixed_expo)
   double dot = 0.0;
   int* spm0 = reinterpret_cast<int*>(smem);
   if (threadIdx.x < 64) spm0[threadIdx.x] = 0;
