@@ -219,8 +219,7 @@ fem_status fem_mesh_set_absorbing(fem_mesh* m, int64_t n_faces, const int32_t* f
 /*
  * Selects the EBE product implementation of a mesh (library tuning knob; the paper's EBE is one product,
  * Section 3.2, Eq. eqebefem).  ebe_variant: 0 = automatic (by the mesh's size, n_rhs and the precision), 1 = generic
- * element kernel (on a mesh without hex patches, FP32 products of n_rhs >= 4 without p^T q sum in tiles of 256
- * elements first), 2 = tiled hex-patch
+ * element kernel, 2 = tiled hex-patch
  * kernel (available when the elements come in groups of six tets splitting a hexahedron with the Kuhn
  * topology, which fem_mesh_create detects), 3 = the tiled hex kernel with each tile's node values and
  * element records staged in shared memory first by bulk asynchronous copies (double-buffered), 4 = as 3

@@ -9,8 +9,7 @@
 // from int L_0^a L_1^b L_2^c L_3^d dV = 6 V a! b! c! d! / (a + b + c + d + 3)! for the preconditioner's
 // diagonal, applied in the product through the seven distinct values of 420 m_ij.
 // Local order: corners 0-3, edges (0,1), (1,2), (0,2), (0,3), (1,3), (2,3).  One thread per (element,
-// case); sums scatter with global atomics into a zeroed q, Dirichlet DOFs skipped (the FP32 products of four cases
-// and more go through the tiles of k_elem_tile.cu).
+// case); sums scatter with global atomics into a zeroed q, Dirichlet DOFs skipped.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -259,13 +258,9 @@ template <typename T>
 cudaError_t launch_ebe10_gated(int64_t E, int64_t N, int rpad, const int32_t* conn10, const float* rec32,
                                const double* rec64, const uint8_t* fm, const T* pm, const T* pk, T* q, double aM,
                                double aK, const Reducer* red, CgCase* sc, double* ptq, const int* gate,
-                               cudaStream_t s, const ElemTiles* et) {
+                               cudaStream_t s) {
   cudaError_t e = cudaMemsetAsync(q, 0, sizeof(T) * (size_t)N * 3 * rpad, s);
   if (e != cudaSuccess) return e;
-  if constexpr (sizeof(T) == 4) {
-    if (!pk && et && elem_tile_fits(10, *et, rpad, pm, q))
-      return launch_elem_tile(10, *et, E, rpad, rec32, pm, q, aM, aK, red, sc, ptq, gate, s);
-  }
   const int rs = lg2i(rpad);
   const bool i32 = N * 3 * rpad < ((int64_t)1 << 31);
   const Reducer none{nullptr, nullptr, nullptr};
@@ -287,10 +282,10 @@ cudaError_t launch_ebe10_gated(int64_t E, int64_t N, int rpad, const int32_t* co
 }
 template cudaError_t launch_ebe10_gated<float>(int64_t, int64_t, int, const int32_t*, const float*, const double*,
                                                const uint8_t*, const float*, const float*, float*, double, double,
-                                               const Reducer*, CgCase*, double*, const int*, cudaStream_t, const ElemTiles*);
+                                               const Reducer*, CgCase*, double*, const int*, cudaStream_t);
 template cudaError_t launch_ebe10_gated<double>(int64_t, int64_t, int, const int32_t*, const float*, const double*,
                                                 const uint8_t*, const double*, const double*, double*, double, double,
-                                                const Reducer*, CgCase*, double*, const int*, cudaStream_t, const ElemTiles*);
+                                                const Reducer*, CgCase*, double*, const int*, cudaStream_t);
 
 cudaError_t launch_diag10(int64_t E, const int32_t* conn10, const double* rec64, double aM, double aK, double* D,
                           cudaStream_t s) {
@@ -326,9 +321,7 @@ struct fem_mesh10 {
   unsigned* counter = nullptr;
   double* out = nullptr;
   Mass10 mc{};
-  ElemTiles et;               // tiles of the FP32 products
   ~fem_mesh10() {
-    free_elem_tiles(&et);
     cudaFree(conn); cudaFree(rec32); cudaFree(rec64); cudaFree(fm); cudaFree(partial); cudaFree(counter); cudaFree(out);
   }
 };
@@ -395,12 +388,6 @@ fem_status fem_mesh10_create(int64_t n_nodes, const double* xyz, int64_t n_elems
     if (e != cudaSuccess) return set_error(FEM_ERR_CUDA, std::string("tet10 mesh: ") + cudaGetErrorString(e));
     return set_error(FEM_ERR_ARG, h_err & 2 ? "degenerate or inverted corner tet" : "bad material id");
   }
-  e = build_elem_tiles(10, n_elems, n_nodes, m->conn, m->fm, m->rec32, &m->et, s);
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    delete m;
-    return set_error(FEM_ERR_CUDA, std::string("tet10 tiles: ") + cudaGetErrorString(e));
-  }
   double mm[10][10];
   mass10_host(mm);
   for (int i = 0; i < 10; ++i)
@@ -429,7 +416,7 @@ fem_status fem_ebe10_apply(fem_mesh10* m, int precision, const void* p_dev, void
           ? launch_ebe10_gated<double>(m->E, m->N, n_rhs, m->conn, m->rec32, m->rec64, m->fm, (const double*)p_dev,
                                        nullptr, (double*)q_dev, alpha_M, alpha_K, rd, nullptr, ptq_dev, nullptr, s)
           : launch_ebe10_gated<float>(m->E, m->N, n_rhs, m->conn, m->rec32, m->rec64, m->fm, (const float*)p_dev, nullptr,
-                                      (float*)q_dev, alpha_M, alpha_K, rd, nullptr, ptq_dev, nullptr, s, &m->et);
+                                      (float*)q_dev, alpha_M, alpha_K, rd, nullptr, ptq_dev, nullptr, s);
   if (e != cudaSuccess) return set_error(FEM_ERR_CUDA, std::string("tet10 product: ") + cudaGetErrorString(e));
   return FEM_OK;
 }
@@ -474,7 +461,7 @@ fem_status pcg10_solve(fem_mesh10* m, int precision, const double* b_dev, double
   auto product32 = [&](const float* in, float* out) {   // FP32 product with p^T q and the step length
     if (e == cudaSuccess)
       e = launch_ebe10_gated<float>(m->E, m->N, rpad, m->conn, m->rec32, m->rec64, m->fm, in, nullptr, out, alpha_M,
-                                    alpha_K, &red, sc, nullptr, n_active, s, &m->et);
+                                    alpha_K, &red, sc, nullptr, n_active, s);
   };
   auto product = [&](const double* in, double* out, bool dot) {
     if (e == cudaSuccess)

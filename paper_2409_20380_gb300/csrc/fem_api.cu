@@ -272,7 +272,6 @@ struct fem_mesh {
   static constexpr int kNTile = 5;
   HexTiles tiles[kNTile];          // hex_per_tile 32, 64, 128, 256, 512
   std::vector<void*> tile_bufs;
-  ElemTiles et;                    // element tiles (meshes without hex patches, quadratic tets)
   int ebe_variant = 0;             // 0 auto, 1 generic, 2 tiled hex, 3 staged, 4 case-major, 5/6 packed staged,
                                    // 7 hex element matrices, 8 assembled 3x3 blocks (CRS-style comparator)
   float* hexmat = nullptr;         // [ceil(H / 2)][300][2] hex matrices for (cM, cK) (built on first use)
@@ -414,7 +413,6 @@ struct fem_mesh {
     for (auto* w : ws) delete w;
     if (pool) cudaMemPoolDestroy(pool);
     for (void* b : tile_bufs) cudaFree(b);
-    free_elem_tiles(&et);
   }
   // Tiling for a product on T with rpad cases: the largest tile whose accumulator fits the budget.
   // EBE implementation of a product on elements of elem_bytes with rpad cases: an explicit fem_mesh_tune
@@ -547,7 +545,7 @@ static cudaError_t ebe_elem_product(const fem_mesh* m, int rpad, const T* p, T* 
   }
   if (m->npe == 10 && v != 8)   // quadratic tets: the tet10 element kernel (or the assembled blocks, variant 8)
     return launch_ebe10_gated<T>(m->E, m->N, rpad, m->conn10, m->rec32, m->rec64, m->fm, p, nullptr, q, aM, aK, red,
-                                 sc, ptq, gate, s, &m->et);
+                                 sc, ptq, gate, s);
   if (v == 8) {   // assembled 3x3 blocks (built outside stream capture only); not for fused groups
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     if (!m->seg && (m->row_ptr || (cudaStreamIsCapturing(s, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone &&
@@ -556,7 +554,7 @@ static cudaError_t ebe_elem_product(const fem_mesh* m, int rpad, const T* p, T* 
                                   ptq, gate, s);
     if (m->npe == 10)
       return launch_ebe10_gated<T>(m->E, m->N, rpad, m->conn10, m->rec32, m->rec64, m->fm, p, nullptr, q, aM, aK,
-                                   red, sc, ptq, gate, s, &m->et);
+                                   red, sc, ptq, gate, s);
     v = m->hex ? 5 : 1, h = 0;
   }
   if (v == 7) {   // hex element matrices: FP32, the mesh's own coefficients, no fused groups, aligned vectors
@@ -586,14 +584,6 @@ static cudaError_t ebe_elem_product(const fem_mesh* m, int rpad, const T* p, T* 
   }
   if (const HexTiles* t = m->tiles_for(sizeof(T), rpad, v, h))
     return launch_ebe_hex<T>(*t, m->view(), rpad, p, q, aM, aK, red, sc, ptq, gate, s);
-  if constexpr (sizeof(T) == 4) {
-    // Element tiles, without p^T q only: its FP32 sums of a thread stay those of the element kernel.
-    if (!red && !m->seg && elem_tile_fits(4, m->et, rpad, p, q)) {
-      const cudaError_t e = cudaMemsetAsync(q, 0, sizeof(T) * (size_t)m->N * 3 * rpad, s);
-      if (e != cudaSuccess) return e;
-      return launch_elem_tile(4, m->et, m->E, rpad, m->rec32, p, q, aM, aK, nullptr, nullptr, nullptr, gate, s);
-    }
-  }
   return launch_ebe_gated<T>(m->view(), rpad, p, nullptr, q, aM, aK, red, sc, ptq, gate, s);
 }
 
@@ -2077,16 +2067,6 @@ static fem_status mesh_create(int64_t n_nodes, const double* xyz, int64_t n_elem
     }
     if (!ok) return bail(fail(FEM_ERR_OOM, "tile allocation failed"));
     m->hex = true;
-  }
-  if (!m->hex) {
-    const cudaError_t ce = build_elem_tiles(
-        npe, n_elems, n_nodes, npe == 10 ? m->conn10 : reinterpret_cast<const int32_t*>(m->conn), m->fm, m->rec32, &m->et, s);
-    if (ce == cudaErrorMemoryAllocation) {
-      cudaGetLastError();   // no room for the tiles: the products take the element kernels
-    } else if (ce != cudaSuccess) {
-      cudaGetLastError();
-      return bail(fail(FEM_ERR_CUDA, std::string("element tiles: ") + cudaGetErrorString(ce)));
-    }
   }
   *out = m;
   return FEM_OK;

@@ -52,15 +52,6 @@ struct HexTiles {                    // device view
   // of |M^e_ij| and |K^e_ij| (bounds on any partial sum of a product's element contributions to a row)
   float abs_m = 0.0f, abs_k = 0.0f;
 };
-// Tiles of consecutive elements of a mesh without hex patches (k_elem_tile.cu), device arrays.
-struct ElemTiles {
-  int n_tiles = 0;                   // 0: not built (few elements, no locality, too many nodes for the entries)
-  int per_tile = 0, nloc_max = 0;
-  const int* count = nullptr;        // [n_tiles] distinct nodes
-  const int* nodes = nullptr;        // tile t's from t x per_tile x npe: node id (bits 0-27), free-DOF bits (28-30)
-  const uint16_t* loc = nullptr;     // [E][nodes per element] tile-local node index
-  float abs_m = 0.0f, abs_k = 0.0f;  // as HexTiles'
-};
 bool detect_hex_patches(const int32_t* conn, int64_t E);
 bool build_hex_tiles(const int32_t* conn, int64_t E, int64_t N, int hex_per_tile, HexTilesHost* out);
 
@@ -173,19 +164,6 @@ int wide_grid_cap();
 int grid_for(int64_t items, int cap = -1);   // cap < 0: red_grid_cap()
 // Largest element-wise absolute row sums of M and K over the mesh's nodes (see HexTiles::abs_m).
 cudaError_t elem_abs_row_bounds(const MeshView& m, double* abs_m, double* abs_k, cudaStream_t s);
-// FP32 absolute row sums of linear tets' M and K per node ([N] and [N][3], zeroed by the caller); the largest |v|.
-cudaError_t launch_abs_rows4(int64_t E, const int4* conn, const float* rec32, float* mrow, float* krow, cudaStream_t s);
-cudaError_t launch_max_abs(int64_t n, const float* v, int* out, cudaStream_t s);
-// Tiles of a mesh of npe-node elements (conn [E][npe] on the device).  Synchronises s.
-cudaError_t build_elem_tiles(int npe, int64_t E, int64_t N, const int32_t* conn, const uint8_t* fm, const float* rec32,
-                             ElemTiles* out, cudaStream_t s);
-void free_elem_tiles(ElemTiles* t);
-// Whether the tiled element product applies to rpad cases and these vectors, and the FP32 product q += (aM M +
-// aK K) p with it (q zeroed by the caller; red, p^T q and the CG step length: quadratic tets only).
-bool elem_tile_fits(int npe, const ElemTiles& et, int rpad, const void* p, const void* q);
-cudaError_t launch_elem_tile(int npe, const ElemTiles& et, int64_t E, int rpad, const float* rec32, const float* p,
-                             float* q, double aM, double aK, const Reducer* red, CgCase* sc, double* ptq,
-                             const int* gate, cudaStream_t s);
 // Grid of grid-stride kernel `fn` (blocks of `block` threads, no dynamic shared memory): at most one wave of
 // the blocks that fit on the GPU at once, so no partial second wave.
 int grid_resident(const void* fn, int block, int64_t items);
@@ -452,7 +430,7 @@ template <typename T>
 cudaError_t launch_ebe10_gated(int64_t E, int64_t N, int rpad, const int32_t* conn10, const float* rec32,
                                const double* rec64, const uint8_t* fm, const T* pm, const T* pk, T* q, double aM,
                                double aK, const Reducer* red, CgCase* sc, double* ptq, const int* gate,
-                               cudaStream_t s, const ElemTiles* et = nullptr);
+                               cudaStream_t s);
 cudaError_t launch_diag10(int64_t E, const int32_t* conn10, const double* rec64, double aM, double aK, double* D,
                           cudaStream_t s);
 cudaError_t launch_bcsr_assemble10(int64_t E, const int32_t* conn10, const double* rec64, const int32_t* row_ptr,

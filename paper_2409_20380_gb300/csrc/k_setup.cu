@@ -259,24 +259,18 @@ __global__ void k_max_abs(int64_t n, const float* __restrict__ v, int* __restric
   if ((threadIdx.x & 31) == 0) atomicMax(out, __float_as_int(mx));
 }
 
-cudaError_t launch_abs_rows4(int64_t E, const int4* conn, const float* rec32, float* mrow, float* krow, cudaStream_t s) {
-  k_abs_rows<<<grid_for(E, wide_grid_cap()), kBlock, 0, s>>>(E, conn, rec32, mrow, krow);
-  return cudaGetLastError();
-}
-cudaError_t launch_max_abs(int64_t n, const float* v, int* out, cudaStream_t s) {
-  k_max_abs<<<grid_for(n), kBlock, 0, s>>>(n, v, out);
-  return cudaGetLastError();
-}
-
 cudaError_t elem_abs_row_bounds(const MeshView& m, double* abs_m, double* abs_k, cudaStream_t s) {
   float* rows = nullptr;
   const int64_t n = m.N;
   cudaError_t e = cudaMalloc(&rows, sizeof(float) * (4 * n + 2));
   if (e == cudaSuccess) e = cudaMemsetAsync(rows, 0, sizeof(float) * (4 * n + 2), s);
   int* mx = reinterpret_cast<int*>(rows + 4 * n);
-  if (e == cudaSuccess) e = launch_abs_rows4(m.E, m.conn, m.rec32, rows + 3 * n, rows, s);
-  if (e == cudaSuccess) e = launch_max_abs(3 * n, rows, mx, s);
-  if (e == cudaSuccess) e = launch_max_abs(n, rows + 3 * n, mx + 1, s);
+  if (e == cudaSuccess) {
+    k_abs_rows<<<grid_for(m.E, wide_grid_cap()), kBlock, 0, s>>>(m.E, m.conn, m.rec32, rows + 3 * n, rows);
+    k_max_abs<<<grid_for(3 * n), kBlock, 0, s>>>(3 * n, rows, mx);
+    k_max_abs<<<grid_for(n), kBlock, 0, s>>>(n, rows + 3 * n, mx + 1);
+    e = cudaGetLastError();
+  }
   float h[2] = {0.f, 0.f};
   if (e == cudaSuccess) e = cudaMemcpyAsync(h, mx, sizeof(h), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
