@@ -99,15 +99,16 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? 2 : 1) k_ebe10(int64_
     const int64_t e = it >> rshift;
     const int c = (int)(it & (rpad - 1));
     I off[10];   // offset of node i's first value of case c
-    int fr[10];
+    int fr = 0;   // free-DOF bits of the nodes, three each
 #pragma unroll
     for (int i = 0; i < 10; ++i) {
       const int nd = __ldg(conn + e * 10 + i);
       off[i] = (I)nd * (I)(3 * rpad) + (I)c;
-      fr[i] = fm[nd];
+      fr |= (fm[nd] & 7) << (3 * i);
     }
     T r[12];
     load_rec(recs + e * kRec, r);
+    T S[10][3];
     T hd = (T)0;   // (the element's p^T q in the product's precision, one conversion an element: FP64
                    // conversions and adds run on GB300's narrow FP64 pipe)
     elem10<DOT, T, T>(
@@ -117,10 +118,23 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? 2 : 1) k_ebe10(int64_
         },
         [&](int i, const T (&Q)[3]) {
 #pragma unroll
-          for (int k = 0; k < 3; ++k)
-            if (dof_free((uint8_t)fr[i], k)) atomicAdd(q + off[i] + (I)(k * rpad), Q[k]);
+          for (int k = 0; k < 3; ++k) S[i][k] = Q[k];
         },
         r, aM, aK, hd);
+    // One branch an element, taken by the few at the boundary: thirty atomics with a condition each cost more than the
+    // separate Dirichlet pass they replaced (16 cases on 786,432 elements: 642 us against 531, with p^T q 685 against 595).
+    if (fr == 0x3fffffff) {
+#pragma unroll
+      for (int i = 0; i < 10; ++i)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) atomicAdd(q + off[i] + (I)(k * rpad), S[i][k]);
+    } else {
+#pragma unroll
+      for (int i = 0; i < 10; ++i)
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+          if (fr >> (3 * i + k) & 1) atomicAdd(q + off[i] + (I)(k * rpad), S[i][k]);
+    }
     if (DOT) dot += (double)hd;
   }
   if (DOT) {
