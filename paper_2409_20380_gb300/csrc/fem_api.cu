@@ -272,6 +272,7 @@ struct fem_mesh {
   static constexpr int kNTile = 5;
   HexTiles tiles[kNTile];          // hex_per_tile 32, 64, 128, 256, 512
   std::vector<void*> tile_bufs;
+  static constexpr int kHexElem = 10, kHexSplit = 11;   // the hex element kernels (chosen by resolve only)
   int ebe_variant = 0;             // 0 auto, 1 generic, 2 tiled hex, 3 staged, 4 case-major, 5/6 packed staged,
                                    // 7 hex element matrices, 8 assembled 3x3 blocks (CRS-style comparator)
   float* hexmat = nullptr;         // [ceil(H / 2)][300][2] hex matrices for (cM, cK) (built on first use)
@@ -426,23 +427,15 @@ struct fem_mesh {
       const Tuned& t = tuned[elem_bytes == 4 ? 0 : 1][lg];
       if (t.variant) *variant = t.variant, *hpt = t.hpt;
     }
-    if (*variant == 0 && *hpt == 0 && hex && !seg) {
-      // Automatic choice on hex patches by the hexes H and the cases r, both sides measured alone:
-      //   FP32: packed staged tiles (5), with 1 or 2 cases (no 16-byte node rows) unstaged tiles, but the element
-      //   kernel for those up to H r = 8192 (H = 512, r = 1: 8.4 us against 12.2; 4096: 10.8 against 12.8; 15,283:
-      //   17.8 against 14.7), where the tiles would leave most SMs idle.
-      //   FP64 (bound by the FP64 pipe): tiles of at most 128 hexes from 50,000 hexes on, three tiles an SM
-      //   (110,593 hexes, 4 cases: 586 us against 620 staged, 638 element kernel; 1 case 153 against 204, 178), the
-      //   element kernel below, whose threads spread over all SMs (512 hexes, 1 case: 12.5 us against 33.5 for 64-hex
-      //   tiles and 103 for one 512-hex tile; 15,283 hexes, 16 cases: 354 against 403).
-      if (elem_bytes == 4) {
-        if (rpad <= 2 && (E / 6) * rpad <= 8192) *variant = 1;
-      } else {
-        *variant = E / 6 < 50000 ? 1 : 2;
-        *hpt = *variant == 2 ? 128 : 0;
-        if (*variant == 2 && !tiles_for(elem_bytes, rpad, 2, 128)) *hpt = 0;
-      }
-    }
+    // Automatic choice on hex patches, both sides measured alone.  FP32: packed staged tiles (5), with 1 or 2 cases (no
+    // 16-byte node rows) unstaged ones.  FP64 (bound by the FP64 pipe), by the hexes H and the cases r: the hex element
+    // kernel (against the best of 64- and 128-hex tiles, r = 1, 4, 16: H = 6912 30 us against 34, 42 against 60, 139 against
+    // 194; 25,920 42 against 46, 140 against 147, 486 against 559; 50,688 75 against 79, 270 against 284, 916 against
+    // 1105; 1,048,576, r = 1, 4: 1198 against 1269, 4662 against 4987; tiles ahead at two sizes of all measured, by the last
+    // wave: 131,072, r = 1, 189 against 171, and 98,304, r = 2, 272 against 259), up to H r = 8192 with a thread a tet
+    // (H = 512, r = 1: 14.0 against 28.8; 4800, r = 1: 17 against 30, 2 29 against 30; 6912, r = 2: 34 against 29).
+    if (elem_bytes == 8 && *variant == 0 && *hpt == 0 && hex && !seg)
+      *variant = (E / 6) * rpad <= 8192 ? kHexSplit : kHexElem;
     if (*variant == 0) *variant = hex ? 5 : 1;       // packed staged tiles where they apply (else 3, 2, 1)
     if (!hex && *variant != 8) *variant = 1;
   }
@@ -570,6 +563,10 @@ static cudaError_t ebe_elem_product(const fem_mesh* m, int rpad, const T* p, T* 
         return launch_ebe_hexmat(*t, m->view(), m->hexmat, rpad, p, q, aM, aK, red, sc, ptq, gate, s);
     }
     v = 5, h = 0;
+  }
+  if constexpr (sizeof(T) == 8) {
+    if (v == fem_mesh::kHexSplit) return launch_hex_split(m->view(), rpad, p, q, aM, aK, red, sc, ptq, gate, s);
+    if (v == fem_mesh::kHexElem) return launch_hex_atomic(m->view(), rpad, p, q, aM, aK, red, sc, ptq, gate, s);
   }
   if (v == 4) {   // case-major staged tiles (converged cases skipped); same requirements as 3, no fused groups
     const HexTiles* t = (reinterpret_cast<uintptr_t>(p) & 15) == 0 ? m->tiles_for(sizeof(T), rpad, 4, h) : nullptr;

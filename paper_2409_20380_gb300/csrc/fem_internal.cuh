@@ -330,6 +330,12 @@ cudaError_t launch_ebe_hex_staged(const HexTiles& ht, const MeshView& m, int rpa
 template <typename T>
 size_t ebe_hex_staged_smem(const HexTiles& ht, const MeshView& m, int rpad);   // ~0 when not applicable
 size_t ebe_hex_packed_extra(const HexTiles& ht);   // more, for the packed form
+// FP64 products without tiles (meshes of hex patches, not fused groups): one thread a hex and case, and one thread a
+// tet and case with the sums by hexes (very small meshes).
+cudaError_t launch_hex_atomic(const MeshView& m, int rpad, const double* p, double* q, double aM, double aK,
+                              const Reducer* red, CgCase* sc, double* ptq_out, const int* gate, cudaStream_t s);
+cudaError_t launch_hex_split(const MeshView& m, int rpad, const double* p, double* q, double aM, double aK,
+                             const Reducer* red, CgCase* sc, double* ptq_out, const int* gate, cudaStream_t s);
 // Case-major staged variant: warps of 32 hexes of one case; converged cases (sc[c].active == 0) skipped.
 template <typename T>
 cudaError_t launch_ebe_hex_cm(const HexTiles& ht, const MeshView& m, int rpad, const T* p, T* q, double aM, double aK,

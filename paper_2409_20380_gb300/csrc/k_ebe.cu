@@ -115,23 +115,27 @@ __global__ void __launch_bounds__(kBlock) k_ebe_atomic(MeshView m, int rpad, int
   }
 }
 
+// Grid of the element kernels.  Small meshes: blocks small enough that the items cover the SMs twice (3072 tets, one
+// case: 96 blocks of a warp instead of 12 of 256 threads; FP64 product 12.5 us), but of at least 8 rpad threads, so that
+// the last block of the p^T q reduction has eight threads a case.
+static void elem_grid(int64_t items, int rpad, bool reduces, int* grid, int* block) {
+  int b = kBlock;
+  while (b > 32 && b > 8 * rpad && items < (int64_t)b * 2 * sm_count()) b >>= 1;
+  const int cap = reduces ? vec_grid_cap() * (kBlock / b) : red_grid_cap();
+  *grid = (int)std::min((items + b - 1) / b, (int64_t)std::min(cap, kMaxRedBlocks));
+  *block = b;
+}
+
 template <typename T, int NC>
 static cudaError_t ebe_atomic_nc(const MeshView& m, int rpad, const T* pm, const T* pk, T* q, T aM, T aK,
                                  const Reducer* red, CgCase* sc, double* ptq_out, const int* gate, cudaStream_t s) {
   const int gs = log2i(rpad / NC);
-  // Small meshes: blocks small enough that the items cover the SMs twice (3072 tets, one case: 96 blocks of a
-  // warp instead of 12 of 256 threads; FP64 product 12.5 us), but of at least 8 rpad threads, so that the last
-  // block of the p^T q reduction has eight threads a case.
-  const int64_t items = m.E << gs;
-  int block = kBlock;
-  while (block > 32 && block > 8 * rpad && items < (int64_t)block * 2 * sm_count()) block >>= 1;
-  const int cap = red ? vec_grid_cap() * (kBlock / block) : red_grid_cap();
-  int64_t grid = (items + block - 1) / block;
-  if (grid > std::min(cap, kMaxRedBlocks)) grid = std::min(cap, kMaxRedBlocks);
+  int grid, block;
+  elem_grid(m.E << gs, rpad, red != nullptr, &grid, &block);
   const Reducer rd = red ? *red : Reducer{nullptr, nullptr, nullptr};
   const bool i32 = m.N * 3 * rpad < ((int64_t)1 << 31);
   auto run = [&](auto kfn) {
-    kfn<<<(int)grid, block, 0, s>>>(m, rpad, gs, pm, pk ? pk : pm, q, aM, aK, rd, red ? sc : nullptr,
+    kfn<<<grid, block, 0, s>>>(m, rpad, gs, pm, pk ? pk : pm, q, aM, aK, rd, red ? sc : nullptr,
                                     red ? ptq_out : nullptr, gate);
     return cudaGetLastError();
   };
@@ -409,6 +413,154 @@ __device__ __forceinline__ void hex_elem(LD ld, FL fl, RC rc, T aM, T aK, T& hd)
       fl(sl, Q[sl]);
     }
   }
+}
+
+// FP64 products, one thread per (hex, case), without tiles: the corners' sums over the hex's tets stay in registers, and
+// 27 of them instead of 72 element sums go to global memory.  The FP64 pipe bounds it, with nothing to stage or flush
+// and no barrier beside it (sizes: the automatic choice in fem_api.cu).  A sum over tets kept in registers rounds
+// less often than one in global memory: off by 1.75e-16 to 1.88e-16 of the rms value, as from the tiles, where one
+// thread a tet gives 2.0e-16 to 2.2e-16.
+template <bool DOT, typename I>
+__global__ void __launch_bounds__(kBlock) k_hex_atomic(MeshView m, int rpad, int rshift, const double* __restrict__ p,
+                                                       double* __restrict__ q, double aM, double aK, Reducer red,
+                                                       CgCase* sc, double* ptq_out, const int* gate) {
+  if (gate && *gate == 0) return;
+  const int64_t total = (m.E / 6) << rshift;
+  const int c = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) & (rpad - 1));
+  double dot = 0.0;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t h = i >> rshift;
+    // the eight corners, from three of the tets (kHexTet)
+    const int4 t0 = __ldg(m.conn + 6 * h), t3 = __ldg(m.conn + 6 * h + 3), t4 = __ldg(m.conn + 6 * h + 4);
+    const int nd[8] = {t0.x, t0.y, t0.z, t0.w, t4.z, t3.y, t3.z, t4.y};
+    I off[8];
+    int fr = 0;       // free-DOF bits of the corners, three each
+#pragma unroll
+    for (int a = 0; a < 8; ++a) {
+      off[a] = (I)nd[a] * (I)(3 * rpad) + (I)c;
+      fr |= (m.freemask[nd[a]] & 7) << (3 * a);
+    }
+    const double* re = m.rec64 + h * 6 * kRec;
+    hex_apply<DOT>(
+        [&](int sl, double (&P)[3]) {
+#pragma unroll
+          for (int k = 0; k < 3; ++k) P[k] = p[off[sl] + (I)(k * rpad)];
+        },
+        [&](int sl, const double (&Q)[3]) {
+          if ((fr >> (3 * sl) & 7) == 7) {
+#pragma unroll
+            for (int k = 0; k < 3; ++k) atomicAdd(q + off[sl] + (I)(k * rpad), Q[k]);
+          } else {
+#pragma unroll
+            for (int k = 0; k < 3; ++k)
+              if (fr >> (3 * sl + k) & 1) atomicAdd(q + off[sl] + (I)(k * rpad), Q[k]);
+          }
+        },
+        [&](int t, double (&r)[12]) { load_rec(re + t * kRec, r); }, aM, aK, dot);
+  }
+  if constexpr (DOT) {
+    double v[1] = {dot};
+    if (block_reduce_last<1>(v, rpad, red)) ebe_tail(red, sc, ptq_out, rpad);
+  }
+}
+
+// The same for very few hexes in FP64, where the chain of a whole hex (700 operations of long latency: 20 us) is what
+// bounds: one thread a tet, the hex's corner sums over its tets through shared memory.  A block takes nb items, a
+// multiple of the cases, on threads t nb + j (tet t of item j), so a thread's case is threadIdx.x mod rpad.
+// 512 hexes, one case: 14.0 us against 28.8.
+struct HexRefs {
+  int n[8], ref[8][6];     // per corner: its tets, as 4 tet + corner in the tet
+};
+constexpr HexRefs hex_refs() {
+  HexRefs r{};
+  for (int t = 0; t < 6; ++t)
+    for (int a = 0; a < 4; ++a) {
+      const int s = kHexTet[t][a];
+      r.ref[s][r.n[s]++] = 4 * t + a;
+    }
+  return r;
+}
+__constant__ HexRefs c_hex_refs = hex_refs();
+constexpr int kSplitItems = 32;
+
+template <bool DOT>
+__global__ void __launch_bounds__(6 * kSplitItems) k_hex_split(MeshView m, int rpad, int rshift, int nb,
+                                                               const double* __restrict__ p, double* __restrict__ q,
+                                                               double aM, double aK, Reducer red, CgCase* sc,
+                                                               double* ptq_out, const int* gate) {
+  if (gate && *gate == 0) return;
+  __shared__ double part[kSplitItems][73];       // (one more than 72: the items' words on different banks)
+  __shared__ int node[kSplitItems][24];
+  const int64_t total = (m.E / 6) << rshift;
+  const int t = threadIdx.x / nb, j = threadIdx.x % nb;
+  double dot = 0.0;
+  for (int64_t base = (int64_t)blockIdx.x * nb; base < total; base += (int64_t)gridDim.x * nb) {
+    const int64_t i = base + j;
+    if (t < 6 && i < total) {
+      const int64_t e = (i >> rshift) * 6 + t;
+      const int c = (int)(i & (rpad - 1));
+      const int4 cn = __ldg(m.conn + e);
+      const int nd[4] = {cn.x, cn.y, cn.z, cn.w};
+      const int fr[4] = {m.freemask[cn.x] & 7, m.freemask[cn.y] & 7, m.freemask[cn.z] & 7, m.freemask[cn.w] & 7};
+      double r[12];
+      load_rec(m.rec64 + e * kRec, r);
+      auto ld = [&](int a, double (&P)[3]) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) P[k] = p[((int64_t)nd[a] * 3 + k) * rpad + c];
+      };
+      auto fl = [&](int a, const double (&Q)[3]) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) part[j][(4 * t + a) * 3 + k] = Q[k];
+        node[j][4 * t + a] = nd[a] | fr[a] << 28;
+      };
+      elem4<DOT, false, double, double>(ld, ld, fl, r, aM, aK, dot);
+    }
+    __syncthreads();
+    for (int o = threadIdx.x; o < nb * 24; o += blockDim.x) {
+      const int jo = o / 24, s = o % 24 / 3, k = o % 3;
+      if (base + jo >= total) break;
+      const int* ref = c_hex_refs.ref[s];
+      const double* w = part[jo] + k;
+      const int n = node[jo][ref[0]];
+      double v = w[ref[0] * 3] + w[ref[1] * 3];                // (two tets, or all six at corners 0 and 3)
+      if (c_hex_refs.n[s] == 6) v += (w[ref[2] * 3] + w[ref[3] * 3]) + (w[ref[4] * 3] + w[ref[5] * 3]);
+      if (n >> (28 + k) & 1) atomicAdd(q + ((int64_t)(n & 0x0fffffff) * 3 + k) * rpad + ((base + jo) & (rpad - 1)), v);
+    }
+    __syncthreads();
+  }
+  if constexpr (DOT) {
+    double v[1] = {dot};
+    if (block_reduce_last<1>(v, rpad, red)) ebe_tail(red, sc, ptq_out, rpad);
+  }
+}
+
+cudaError_t launch_hex_split(const MeshView& m, int rpad, const double* p, double* q, double aM, double aK,
+                             const Reducer* red, CgCase* sc, double* ptq_out, const int* gate, cudaStream_t s) {
+  const cudaError_t err = cudaMemsetAsync(q, 0, sizeof(double) * (size_t)m.N * 3 * rpad, s);
+  if (err != cudaSuccess) return err;
+  const int rs = log2i(rpad), nb = rpad <= 4 ? 5 * rpad : std::max(16, rpad);
+  const int64_t items = (m.E / 6) << rs;
+  const int grid = (int)std::min((items + nb - 1) / nb, (int64_t)red_grid_cap());
+  const Reducer rd = red ? *red : Reducer{nullptr, nullptr, nullptr};
+  auto kfn = red ? k_hex_split<true> : k_hex_split<false>;
+  kfn<<<grid, (6 * nb + 31) & ~31, 0, s>>>(m, rpad, rs, nb, p, q, aM, aK, rd, red ? sc : nullptr, red ? ptq_out : nullptr,
+                                          gate);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_hex_atomic(const MeshView& m, int rpad, const double* p, double* q, double aM, double aK,
+                              const Reducer* red, CgCase* sc, double* ptq_out, const int* gate, cudaStream_t s) {
+  const cudaError_t err = cudaMemsetAsync(q, 0, sizeof(double) * (size_t)m.N * 3 * rpad, s);
+  if (err != cudaSuccess) return err;
+  const int rs = log2i(rpad);
+  int grid, block;
+  elem_grid((m.E / 6) << rs, rpad, red != nullptr, &grid, &block);
+  const Reducer rd = red ? *red : Reducer{nullptr, nullptr, nullptr};
+  const bool i32 = m.N * 3 * rpad < ((int64_t)1 << 31);
+  auto kfn = red ? (i32 ? k_hex_atomic<true, int32_t> : k_hex_atomic<true, int64_t>)
+                 : (i32 ? k_hex_atomic<false, int32_t> : k_hex_atomic<false, int64_t>);
+  kfn<<<grid, block, 0, s>>>(m, rpad, rs, p, q, aM, aK, rd, red ? sc : nullptr, red ? ptq_out : nullptr, gate);
+  return cudaGetLastError();
 }
 
 template <typename T, bool DOT, bool SEG>
