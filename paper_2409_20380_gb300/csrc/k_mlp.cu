@@ -52,6 +52,7 @@ __device__ __forceinline__ float gelu_grad_f(float z) {
 // for 8 output columns, so no shared-memory staging and no barrier between K steps.
 // ------------------------------------------------------------------------------------------------------
 constexpr int kRows = 32;                      // samples a block (two m16 tiles)
+constexpr int kNBias = kL1 + kL2 + kL3;
 constexpr int kMlpBlock = 256;                 // 8 warps: 32 of a layer's 256 columns each
 constexpr int kSX = kL0 + 8, kSA = kL1 + 8, kSD = kL3 + 8;   // padded rows (16 bytes mod 128: conflict-free ldmatrix)
 
@@ -112,7 +113,7 @@ struct MlpPass {
   float* out;              // forward only: [B][32]
   const float* t;          // training: [n_src][32] targets, or residual-space samples [n_src][kNRes]
   bf16 *X0, *A1, *A2, *dZ1, *dZ2, *dZ3;    // training: row-major, for the weight gradients
-  float* grad;             // training: bias gradients are added here (the caller has zeroed it)
+  float* bsum;             // training: [blocks][kNBias] bias gradients of each block's samples (b1, b2, b3)
   double* loss;
 };
 
@@ -127,6 +128,7 @@ __global__ void __launch_bounds__(kMlpBlock) k_mlp_pass(MlpPass g) {
   __shared__ float sr[kMlpBlock / 32][kL3];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, gq = lane >> 2, tq = lane & 3;
   const int64_t row0 = (int64_t)blockIdx.x * kRows;
+  float* bsum = g.bsum + (size_t)blockIdx.x * kNBias;
   auto sample = [&](int r) -> int64_t {   // source row of batch row row0 + r, -1: none
     const int64_t b = row0 + r;
     if (b >= g.B) return -1;
@@ -232,7 +234,7 @@ __global__ void __launch_bounds__(kMlpBlock) k_mlp_pass(MlpPass g) {
     float c = 0.0f;
 #pragma unroll 8
     for (int r = 0; r < kRows; ++r) c += sO[r][lane];
-    atomicAdd(g.grad + kOffB3 + lane, c);
+    bsum[kL1 + kL2 + lane] = c;
   }
   put(sD, kSD, kL3, g.dZ3);
   // dZ = (dZ_next W) * GELU'(Z): BF16 into dst, the FP32 column sums (bias gradient) into gb
@@ -254,18 +256,15 @@ __global__ void __launch_bounds__(kMlpBlock) k_mlp_pass(MlpPass g) {
         s0 += __shfl_xor_sync(0xffffffffu, s0, o);
         s1 += __shfl_xor_sync(0xffffffffu, s1, o);
       }
-      if (gq == 0) {
-        atomicAdd(gb + c, s0);
-        atomicAdd(gb + c + 1, s1);
-      }
+      if (gq == 0) gb[c] = s0, gb[c + 1] = s1;
     }
   };
   layer_mma<kL3, 2, 4>(sD, kSD, g.P3T, 4 * warp, acc);
-  back(g2, sB, g.grad + kOffB2);      // (rows past the batch have dL/dout = 0, so their dZ is zero)
+  back(g2, sB, bsum + kL1);      // (rows past the batch have dL/dout = 0, so their dZ is zero)
   __syncthreads();
   put(sB, kSA, kL2, g.dZ2);
   layer_mma<kL2, 2, 4>(sB, kSA, g.P2T, 4 * warp, acc);
-  back(g1, sA, g.grad + kOffB1);
+  back(g1, sA, bsum);
   __syncthreads();
   put(sA, kSA, kL1, g.dZ1);
 }
@@ -273,18 +272,34 @@ __global__ void __launch_bounds__(kMlpBlock) k_mlp_pass(MlpPass g) {
 // Weight gradients: C[m][n] += sum_b P[b][m] Q[b][n] over the batch rows b, 64 x 64 tiles of the three outputs
 // (dW2 = dZ2^T A1: 16 tiles; dW1 = dZ1^T X0: 4; dW3 = dZ3^T A2, as its transpose A2^T dZ3 with 32 columns: 4),
 // each with its batch split over gridDim.y blocks that add into the zeroed gradient (so that the grid covers the
-// SMs twice).  Both operands lie row-major by sample: ldmatrix.trans turns them.  A block stages 32 samples at a
+// SMs twice; from 512 samples on, so that smaller batches have one writer and repeat bitwise).  The blocks behind the
+// tiles sum the bias gradients of the pass's blocks, 32 columns each, in a fixed order.  Both operands lie row-major by sample: ldmatrix.trans turns them.  A block stages 32 samples at a
 // time, double-buffered by cp.async.
 constexpr int kWgStride = 72;                  // BF16 values a staged row of 64 (144 bytes: conflict-free)
 struct MlpWgrad {
   const bf16 *X0, *A1, *A2, *dZ1, *dZ2, *dZ3;
+  const float* bsum;
   float* grad;
-  int steps;                                   // batch rows / 32
+  int steps;                                   // batch rows / 32, the blocks of the pass
 };
+constexpr int kWgTiles = 24;
+static_assert(kRows == 32 && kNBias % 32 == 0, "one row of bias sums a step, 32 columns a block");
 __global__ void __launch_bounds__(128) k_mlp_wgrad(MlpWgrad g) {
   __shared__ __align__(16) bf16 sP[2][32 * kWgStride], sQ[2][32 * kWgStride];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, gq = lane >> 2, tq = lane & 3;
   const int tile = blockIdx.x;
+  if (tile >= kWgTiles) {
+    if (blockIdx.y) return;
+    float* sb = reinterpret_cast<float*>(sP);  // [4][32]
+    const int c = (tile - kWgTiles) * 32 + lane;
+    float s = 0.0f;
+    for (int b = warp; b < g.steps; b += 4) s += g.bsum[(size_t)b * kNBias + c];
+    sb[tid] = s;
+    __syncthreads();
+    const int64_t off = c < kL1 ? kOffB1 + c : c < kL1 + kL2 ? kOffB2 + c - kL1 : kOffB3 + c - kL1 - kL2;
+    if (warp == 0) g.grad[off] = (sb[lane] + sb[lane + 32]) + (sb[lane + 64] + sb[lane + 96]);
+    return;
+  }
   const bf16 *P, *Q;
   float* C;
   int ldp, ldq, nq = 64, rs, cs;               // C[m * rs + n * cs]
@@ -408,6 +423,7 @@ struct fem_mlp {
   bf16 *P1 = nullptr, *P2 = nullptr, *P3 = nullptr, *P3T = nullptr, *P2T = nullptr;   // packed weights (k_pack)
   int64_t cap = 0;                     // rows of the training workspace (multiple of kRows)
   bf16 *X0 = nullptr, *A1 = nullptr, *A2 = nullptr, *dZ1 = nullptr, *dZ2 = nullptr, *dZ3 = nullptr;
+  float* bsum = nullptr;
   int64_t out_cap = 0;                 // rows of OUT
   float* OUT = nullptr;
   double* loss_acc = nullptr;
@@ -415,9 +431,10 @@ struct fem_mlp {
   std::mutex mu;
 
   void free_ws() {
-    for (void* p : {(void*)X0, (void*)A1, (void*)A2, (void*)dZ1, (void*)dZ2, (void*)dZ3})
+    for (void* p : {(void*)X0, (void*)A1, (void*)A2, (void*)dZ1, (void*)dZ2, (void*)dZ3, (void*)bsum})
       if (p) cudaFree(p);
     X0 = A1 = A2 = dZ1 = dZ2 = dZ3 = nullptr;
+    bsum = nullptr;
     cap = 0;
   }
   ~fem_mlp() {
@@ -453,6 +470,7 @@ cudaError_t ensure_cap(fem_mlp* n, int64_t rows) {
   };
   A(&n->X0, rows * kL0); A(&n->A1, rows * kL1); A(&n->A2, rows * kL2);
   A(&n->dZ1, rows * kL1); A(&n->dZ2, rows * kL2); A(&n->dZ3, rows * kL3);
+  A(&n->bsum, rows / kRows * kNBias);
   if (e != cudaSuccess) {
     cudaGetLastError();
     n->free_ws();
@@ -491,7 +509,7 @@ cudaError_t loss_grad(fem_mlp* n, const float* x, const float* t, const int32_t*
   MlpPass g = pass_args(n, x, idx, n_src, B);
   CE(ensure_cap(n, g.Mpad));
   CE(cudaMemsetAsync(grad, 0, sizeof(float) * kNParams, s));
-  g.t = t, g.grad = grad, g.loss = n->loss_acc;
+  g.t = t, g.bsum = n->bsum, g.loss = n->loss_acc;
   g.X0 = n->X0, g.A1 = n->A1, g.A2 = n->A2, g.dZ1 = n->dZ1, g.dZ2 = n->dZ2, g.dZ3 = n->dZ3;
   const unsigned blocks = (unsigned)(g.Mpad / kRows);
   if (residual)
@@ -499,11 +517,11 @@ cudaError_t loss_grad(fem_mlp* n, const float* x, const float* t, const int32_t*
   else
     k_mlp_pass<1><<<blocks, kMlpBlock, 0, s>>>(g);
   CE(cudaGetLastError());
-  // 24 tiles; the batch split so that the grid covers the SMs twice, at least 4 of the 32-row steps a block
-  MlpWgrad w{n->X0, n->A1, n->A2, n->dZ1, n->dZ2, n->dZ3, grad, (int)(g.Mpad / 32)};
-  int split = (2 * sm_count() + 23) / 24;
-  if (split > w.steps / 4) split = w.steps / 4;
-  k_mlp_wgrad<<<dim3(24, split < 1 ? 1 : split), 128, 0, s>>>(w);
+  // 24 tiles; the batch split so that the grid covers the SMs twice, at least 8 of the 32-row steps a block
+  MlpWgrad w{n->X0, n->A1, n->A2, n->dZ1, n->dZ2, n->dZ3, n->bsum, grad, (int)(g.Mpad / 32)};
+  int split = (2 * sm_count() + kWgTiles - 1) / kWgTiles;
+  if (split > w.steps / 8) split = w.steps / 8;
+  k_mlp_wgrad<<<dim3(kWgTiles + kNBias / 32, split < 1 ? 1 : split), 128, 0, s>>>(w);
   return cudaGetLastError();
 }
 
