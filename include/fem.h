@@ -262,8 +262,10 @@ fem_status fem_mesh_autotune(fem_mesh* m, int precision, int n_rhs, void* stream
  *       device from the same FP64 element records (built on first use and kept with the mesh);
  *   3 = the assembled operators in double-float arithmetic.
  * Modes 0 and 2 round like FP64; 1 and 3 to about 1e-14 of the largest term.  Modes 2/3 need
- * ~84 bytes x 15 x n_nodes of device memory for the operators.  Mode 3 takes a temporary input
- * copy from the mesh's own stream-ordered memory pool (given back with the mesh; not during stream capture).
+ * ~84 bytes x 15 x n_nodes of device memory for the operators.  Stream-ordered: the call does not wait for the
+ * product (but for the operators, the first time).  Mode 3 takes a temporary input copy from the mesh's own
+ * stream-ordered memory pool, of which up to 256 MB stay with the mesh for the next call and go back with it; not
+ * during stream capture.
  */
 fem_status fem_mesh_split_product(fem_mesh* m, int mode, const double* p_dev, double* qM_dev, double* qK_dev,
                                   int n_rhs, void* stream);
