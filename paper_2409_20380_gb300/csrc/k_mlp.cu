@@ -480,6 +480,23 @@ cudaError_t ensure_cap(fem_mlp* n, int64_t rows) {
   return cudaSuccess;
 }
 
+// OUT for `rows` rows.
+cudaError_t ensure_out(fem_mlp* n, int64_t rows) {
+  if (rows <= n->out_cap) return cudaSuccess;
+  CE(cudaDeviceSynchronize());      // (the old buffer may still be read by work queued on another stream)
+  if (n->OUT) cudaFree(n->OUT);
+  n->OUT = nullptr, n->out_cap = 0;
+  CE(alloc_n(&n->OUT, rows * kL3));
+  n->out_cap = rows;
+  return cudaSuccess;
+}
+
+// Whether the results of `out` may overwrite values of `in` that other blocks still read.
+bool overlap(const void* out, size_t out_bytes, const void* in, size_t in_bytes) {
+  const uintptr_t a = reinterpret_cast<uintptr_t>(out), b = reinterpret_cast<uintptr_t>(in);
+  return a < b + in_bytes && b < a + out_bytes;
+}
+
 cudaError_t pack_weights(fem_mlp* n, cudaStream_t s) {
   k_pack<<<grid_of(kNParams + kL2 * kL1), 256, 0, s>>>(n->th, n->P1, n->P2, n->P3, n->P3T, n->P2T);
   return cudaGetLastError();
@@ -778,13 +795,7 @@ cudaError_t mlp_features(const PredView& p, int n_pairs, const float4* case_src,
 
 cudaError_t mlp_propose(fem_mlp* net, const float* F, int64_t rows, int n_pairs, double* dw, cudaStream_t s) {
   std::lock_guard<std::mutex> lk(net->mu);
-  if (rows > net->out_cap) {
-    CE(cudaDeviceSynchronize());      // (the old buffer may still be read by work queued on another stream)
-    if (net->OUT) cudaFree(net->OUT);
-    net->OUT = nullptr, net->out_cap = 0;
-    CE(alloc_n(&net->OUT, rows * kL3));
-    net->out_cap = rows;
-  }
+  CE(ensure_out(net, rows));
   CE(forward(net, F, rows, net->OUT, s));
   k_coef_delta<<<grid_of(rows * kMaxSlots), 256, 0, s>>>(rows, n_pairs, net->OUT, dw);
   return cudaGetLastError();
@@ -900,7 +911,11 @@ fem_status fem_mlp_forward(fem_mlp* n, const float* x_dev, int64_t B, float* out
   if (!n || (B > 0 && (!x_dev || !out_dev)) || B < 0) return set_error(FEM_ERR_ARG, "fem_mlp_forward: bad argument");
   if (B == 0) return FEM_OK;
   std::lock_guard<std::mutex> lk(n->mu);
-  MCU(forward(n, x_dev, B, out_dev, n->s));
+  const size_t bytes = sizeof(float) * kL3 * B;
+  const bool apart = !overlap(out_dev, bytes, x_dev, sizeof(float) * kL0 * B);
+  if (!apart) MCU(ensure_out(n, B));
+  MCU(forward(n, x_dev, B, apart ? out_dev : n->OUT, n->s));
+  if (!apart) MCU(cudaMemcpyAsync(out_dev, n->OUT, bytes, cudaMemcpyDeviceToDevice, n->s));
   return FEM_OK;
 }
 
@@ -911,7 +926,12 @@ static fem_status mlp_loss_grad_any(fem_mlp* n, const float* x_dev, const float*
   if (!n || !x_dev || !t_dev || B <= 0) return set_error(FEM_ERR_ARG, "fem_mlp_loss_grad: bad argument");
   std::lock_guard<std::mutex> lk(n->mu);
   MCU(cudaMemsetAsync(n->loss_acc, 0, sizeof(double), n->s));
-  MCU(loss_grad(n, x_dev, t_dev, nullptr, B, B, grad_dev ? grad_dev : n->grad, n->s, residual));
+  // (grad_dev may lie in the inputs' memory: it is written once they have been read)
+  const size_t gbytes = sizeof(float) * kNParams;
+  const bool apart = grad_dev && !overlap(grad_dev, gbytes, x_dev, sizeof(float) * kL0 * B) &&
+                     !overlap(grad_dev, gbytes, t_dev, sizeof(float) * (residual ? kNRes : kL3) * B);
+  MCU(loss_grad(n, x_dev, t_dev, nullptr, B, B, apart ? grad_dev : n->grad, n->s, residual));
+  if (grad_dev && !apart) MCU(cudaMemcpyAsync(grad_dev, n->grad, gbytes, cudaMemcpyDeviceToDevice, n->s));
   double acc = 0.0;
   MCU(cudaMemcpyAsync(&acc, n->loss_acc, sizeof(double), cudaMemcpyDeviceToHost, n->s));
   MCU(cudaStreamSynchronize(n->s));

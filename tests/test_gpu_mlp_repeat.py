@@ -1,5 +1,5 @@
 """Gradients of the learned proposal's network repeat bitwise where their sums have a fixed order: all of them for batches
-below 512 samples (one writer an entry), the bias gradients for every batch."""
+below 512 samples (one writer an entry), the bias gradients for every batch.  Results may be written over the inputs."""
 import numpy as np
 import pytest
 
@@ -41,5 +41,31 @@ def test_gradient_repeats(torch_dev, B, residual):
                 first = g
             assert torch.equal(g[biases], first[biases])
             assert B >= 512 or torch.equal(g, first)
+    finally:
+        fem.fem_mlp_destroy(net)
+
+
+def test_results_over_inputs(torch_dev):
+    torch = torch_dev
+    B = 40000      # more blocks than run at once
+    rng = np.random.default_rng(1)
+    x = torch.tensor(rng.standard_normal((B, 64)).astype(np.float32), device="cuda")
+    t = torch.tensor(rng.standard_normal((B, 32)).astype(np.float32), device="cuda")
+    net = fem.fem_mlp_create(wl.mlp_init_weights(5).astype(np.float32))
+    try:
+        out, g = torch.empty((B, 32), device="cuda"), torch.empty(fem.FEM_MLP_N_PARAMS, device="cuda")
+        fem.fem_mlp_forward(net, x, out)
+        loss = fem.fem_mlp_loss_grad(net, x, t, g)
+        both = torch.empty(96 * B, device="cuda")     # x, then t
+        for over in (0, 1000, 64 * B - 90000, 64 * B - 16, 64 * B):
+            both[:64 * B], both[64 * B:] = x.reshape(-1), t.reshape(-1)
+            y = both[over:over + 32 * B]
+            fem.fem_mlp_forward(net, both[:64 * B].reshape(B, 64), y.reshape(B, 32))
+            assert torch.equal(y.reshape(B, 32), out), over
+            both[:64 * B], both[64 * B:] = x.reshape(-1), t.reshape(-1)
+            y = both[over:over + fem.FEM_MLP_N_PARAMS]
+            got = fem.fem_mlp_loss_grad(net, both[:64 * B].reshape(B, 64), both[64 * B:].reshape(B, 32), y)
+            assert abs(got - loss) <= 1e-12 * abs(loss)
+            assert float((y - g).abs().max()) <= 1e-6 * float(g.abs().max()), over   # (the order of 13 atomic adds)
     finally:
         fem.fem_mlp_destroy(net)
