@@ -210,28 +210,6 @@ template cudaError_t launch_mask<float>(int64_t, int, const uint8_t*, float*, cu
 // of the tile's nodes.  The flush stores nodes only this tile touches and adds (global red) the others;
 // q must be zero beforehand for those.  Dirichlet DOFs of q are written as zero.
 // ------------------------------------------------------------------------------------------------------
-template <typename T> struct Vec4;
-template <> struct Vec4<float> {
-  __device__ __forceinline__ static void load12(const float* __restrict__ src, float (&r)[12]) {
-    const float4* s4 = reinterpret_cast<const float4*>(src);
-    const float4 a = __ldg(s4), b = __ldg(s4 + 1), c = __ldg(s4 + 2);
-    r[0] = a.x; r[1] = a.y; r[2] = a.z; r[3] = a.w;
-    r[4] = b.x; r[5] = b.y; r[6] = b.z; r[7] = b.w;
-    r[8] = c.x; r[9] = c.y; r[10] = c.z; r[11] = c.w;
-  }
-};
-template <> struct Vec4<double> {
-  __device__ __forceinline__ static void load12(const double* __restrict__ src, double (&r)[12]) {
-    const double2* s2 = reinterpret_cast<const double2*>(src);
-#pragma unroll
-    for (int i = 0; i < 6; ++i) {
-      const double2 v = __ldg(s2 + i);
-      r[2 * i] = v.x;
-      r[2 * i + 1] = v.y;
-    }
-  }
-};
-
 // One hex in FP64: q += (aM M + aK K) p over its six tets.  ld(slot, P) gives a corner's values, rc(t, r) the
 // record of tet t, fl(slot, Q) takes a corner's sums.  The tets are visited around the cycle of their middle
 // corners (the diagonal corners 0 and 3 are in all six): a middle corner's values are loaded just before its
@@ -614,7 +592,7 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? 2 : 1) k_ebe_hex(HexT
 #pragma unroll
             for (int k = 0; k < 3; ++k) atomicAdd(qs + ls[sl] * per_node + k * rpad + c, Q[k]);
           },
-          [&](int t, T (&r)[12]) { Vec4<T>::load12(re + t * kRec, r); }, aM, aK, hdot);
+          [&](int t, T (&r)[12]) { load_rec(re + t * kRec, r); }, aM, aK, hdot);
       if (seg) {
         double v1[1] = {(double)hdot};
         seg_add<1>(sacc, m.nseg, m.seg[snode[ls[0]] & 0x0fffffff], v1);
@@ -1893,7 +1871,7 @@ __global__ void __launch_bounds__(kBlock) k_ebe_split(MeshView m, int rpad, int 
     const int4 cn = __ldg(m.conn + e);
     const int64_t nd[4] = {cn.x, cn.y, cn.z, cn.w};
     double r[12];
-    Vec4<double>::load12(m.rec64 + e * kRec, r);
+    load_rec(m.rec64 + e * kRec, r);
     double P[4][3];
 #pragma unroll
     for (int a = 0; a < 4; ++a)
