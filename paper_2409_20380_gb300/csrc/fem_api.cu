@@ -2026,9 +2026,11 @@ static fem_status mesh_create(int64_t n_nodes, const double* xyz, int64_t n_elem
   if (npe == 4 && n_nodes < (int64_t(1) << 28) && detect_hex_patches(conn, n_elems)) {
     const int sizes[fem_mesh::kNTile] = {32, 64, 128, 256, 512};
     bool ok = true;
-    double abs_m = 0.0, abs_k = 0.0;   // scale bounds of the packed kernel's fixed-point tile sums
+    float* rows = nullptr;             // the nodes' absolute row sums, for the scales of the fixed-point tile sums
+    if ((st = dalloc(&rows, 4 * n_nodes)) != FEM_OK) return bail(st);
+    m->tile_bufs.push_back(rows);      // (given back below)
     {
-      cudaError_t ce = elem_abs_row_bounds(m->view(), &abs_m, &abs_k, s);
+      cudaError_t ce = launch_abs_rows(m->view(), rows, s);
       if (ce != cudaSuccess) return bail(fail(FEM_ERR_CUDA, std::string("row bounds: ") + cudaGetErrorString(ce)));
     }
     for (int i = 0; i < fem_mesh::kNTile && ok; ++i) {
@@ -2040,15 +2042,19 @@ static fem_status mesh_create(int64_t n_nodes, const double* xyz, int64_t n_elem
       }
       int *d_hoff = nullptr, *d_noff = nullptr, *d_nodes = nullptr;
       uint4* d_loc = nullptr;
+      float4* d_bound = nullptr;
       ok = dalloc(&d_hoff, th.tile_hex_off.size()) == FEM_OK && dalloc(&d_noff, th.tile_node_off.size()) == FEM_OK &&
-           dalloc(&d_nodes, th.tile_nodes.size()) == FEM_OK && dalloc(&d_loc, (size_t)th.n_hex) == FEM_OK;
-      for (void* b : {(void*)d_hoff, (void*)d_noff, (void*)d_nodes, (void*)d_loc})
+           dalloc(&d_nodes, th.tile_nodes.size()) == FEM_OK && dalloc(&d_loc, (size_t)th.n_hex) == FEM_OK &&
+           dalloc(&d_bound, (size_t)th.n_tiles) == FEM_OK;
+      for (void* b : {(void*)d_hoff, (void*)d_noff, (void*)d_nodes, (void*)d_loc, (void*)d_bound})
         if (b) m->tile_bufs.push_back(b);
       if (!ok) break;
-      cudaError_t ce = cudaMemcpy(d_hoff, th.tile_hex_off.data(), sizeof(int) * th.tile_hex_off.size(), cudaMemcpyHostToDevice);
-      if (ce == cudaSuccess) ce = cudaMemcpy(d_noff, th.tile_node_off.data(), sizeof(int) * th.tile_node_off.size(), cudaMemcpyHostToDevice);
-      if (ce == cudaSuccess) ce = cudaMemcpy(d_nodes, th.tile_nodes.data(), sizeof(int) * th.tile_nodes.size(), cudaMemcpyHostToDevice);
-      if (ce == cudaSuccess) ce = cudaMemcpy(d_loc, th.hex_local.data(), sizeof(uint16_t) * th.hex_local.size(), cudaMemcpyHostToDevice);
+      auto up = [&](void* dst, const void* src, size_t bytes) { return cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, s); };
+      cudaError_t ce = up(d_hoff, th.tile_hex_off.data(), sizeof(int) * th.tile_hex_off.size());
+      if (ce == cudaSuccess) ce = up(d_noff, th.tile_node_off.data(), sizeof(int) * th.tile_node_off.size());
+      if (ce == cudaSuccess) ce = up(d_nodes, th.tile_nodes.data(), sizeof(int) * th.tile_nodes.size());
+      if (ce == cudaSuccess) ce = up(d_loc, th.hex_local.data(), sizeof(uint16_t) * th.hex_local.size());
+      if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);   // (the host arrays end with this size)
       if (ce != cudaSuccess) return bail(fail(FEM_ERR_CUDA, std::string("tile upload: ") + cudaGetErrorString(ce)));
       HexTiles& t = m->tiles[i];
       t.n_tiles = th.n_tiles;
@@ -2058,11 +2064,15 @@ static fem_status mesh_create(int64_t n_nodes, const double* xyz, int64_t n_elem
       t.tile_node_off = d_noff;
       t.tile_nodes = d_nodes;
       t.hex_local = d_loc;
-      // (rounded up to FP32 and given 1% more for the FP32 rounding of the records and products)
-      t.abs_m = (float)(abs_m * 1.01);
-      t.abs_k = (float)(abs_k * 1.01);
+      ce = launch_tile_bounds(t, n_nodes, rows, d_bound, s);
+      if (ce != cudaSuccess) return bail(fail(FEM_ERR_CUDA, std::string("tile bounds: ") + cudaGetErrorString(ce)));
+      t.bound = d_bound;
     }
     if (!ok) return bail(fail(FEM_ERR_OOM, "tile allocation failed"));
+    const cudaError_t ce = cudaStreamSynchronize(s);
+    if (ce != cudaSuccess) return bail(fail(FEM_ERR_CUDA, std::string("tile bounds: ") + cudaGetErrorString(ce)));
+    m->tile_bufs.erase(std::find(m->tile_bufs.begin(), m->tile_bufs.end(), (void*)rows));
+    cudaFree(rows);
     m->hex = true;
   }
   *out = m;

@@ -48,9 +48,9 @@ struct HexTiles {                    // device view
   const int* tile_node_off = nullptr;
   const int* tile_nodes = nullptr;   // per entry: node id (bits 0-27), free-DOF bits (28-30), shared (31)
   const uint4* hex_local = nullptr;  // 8 x uint16 per hex
-  // largest element-wise absolute row sums over the nodes: sum over the elements e of a node i and over j
-  // of |M^e_ij| and |K^e_ij| (bounds on any partial sum of a product's element contributions to a row)
-  float abs_m = 0.0f, abs_k = 0.0f;
+  // per tile: the largest element-wise absolute row sums over its nodes, the sum over the elements e of a node i and
+  // over j of |M^e_ij| (x) and |K^e_ij| (y), bounds on any partial sum of a product's element contributions to a row
+  const float4* bound = nullptr;
 };
 bool detect_hex_patches(const int32_t* conn, int64_t E);
 bool build_hex_tiles(const int32_t* conn, int64_t E, int64_t N, int hex_per_tile, HexTilesHost* out);
@@ -162,8 +162,9 @@ int vec_grid_cap();
 int red_grid_cap();
 int wide_grid_cap();
 int grid_for(int64_t items, int cap = -1);   // cap < 0: red_grid_cap()
-// Largest element-wise absolute row sums of M and K over the mesh's nodes (see HexTiles::abs_m).
-cudaError_t elem_abs_row_bounds(const MeshView& m, double* abs_m, double* abs_k, cudaStream_t s);
+// Element-wise absolute row sums of the nodes, rows: [N][3] of K, then [N] of M; their maxima over each tile's nodes.
+cudaError_t launch_abs_rows(const MeshView& m, float* rows, cudaStream_t s);
+cudaError_t launch_tile_bounds(const HexTiles& t, int64_t N, const float* rows, float4* bound, cudaStream_t s);
 // Grid of grid-stride kernel `fn` (blocks of `block` threads, no dynamic shared memory): at most one wave of
 // the blocks that fit on the GPU at once, so no partial second wave.
 int grid_resident(const void* fn, int block, int64_t items);

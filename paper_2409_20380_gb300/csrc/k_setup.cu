@@ -250,35 +250,35 @@ __global__ void k_abs_rows(int64_t E, const int4* __restrict__ conn, const float
   }
 }
 
-// Largest |v| (ordered as integers).
-__global__ void k_max_abs(int64_t n, const float* __restrict__ v, int* __restrict__ out) {
-  float mx = 0.f;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    mx = fmaxf(mx, fabsf(v[i]));
-  for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  if ((threadIdx.x & 31) == 0) atomicMax(out, __float_as_int(mx));
+cudaError_t launch_abs_rows(const MeshView& m, float* rows, cudaStream_t s) {
+  const cudaError_t e = cudaMemsetAsync(rows, 0, sizeof(float) * 4 * m.N, s);
+  if (e != cudaSuccess) return e;
+  k_abs_rows<<<grid_for(m.E, wide_grid_cap()), kBlock, 0, s>>>(m.E, m.conn, m.rec32, rows + 3 * m.N, rows);
+  return cudaGetLastError();
 }
 
-cudaError_t elem_abs_row_bounds(const MeshView& m, double* abs_m, double* abs_k, cudaStream_t s) {
-  float* rows = nullptr;
-  const int64_t n = m.N;
-  cudaError_t e = cudaMalloc(&rows, sizeof(float) * (4 * n + 2));
-  if (e == cudaSuccess) e = cudaMemsetAsync(rows, 0, sizeof(float) * (4 * n + 2), s);
-  int* mx = reinterpret_cast<int*>(rows + 4 * n);
-  if (e == cudaSuccess) {
-    k_abs_rows<<<grid_for(m.E, wide_grid_cap()), kBlock, 0, s>>>(m.E, m.conn, m.rec32, rows + 3 * n, rows);
-    k_max_abs<<<grid_for(3 * n), kBlock, 0, s>>>(3 * n, rows, mx);
-    k_max_abs<<<grid_for(n), kBlock, 0, s>>>(n, rows + 3 * n, mx + 1);
-    e = cudaGetLastError();
+// One block a tile (1% more for the FP32 rounding of the records, the bounds and the products).
+__global__ void __launch_bounds__(128) k_tile_bounds(HexTiles t, int64_t N, const float* __restrict__ rows,
+                                                     float4* __restrict__ bound) {
+  __shared__ int mx[2];            // (sums of absolute values are ordered as integers, NaN above infinity)
+  if (threadIdx.x < 2) mx[threadIdx.x] = 0;
+  __syncthreads();
+  int m = 0, k = 0;
+  for (int l = t.tile_node_off[blockIdx.x] + threadIdx.x; l < t.tile_node_off[blockIdx.x + 1]; l += blockDim.x) {
+    const int64_t n = t.tile_nodes[l] & 0x0fffffff;
+    for (int i = 0; i < 3; ++i) k = max(k, __float_as_int(rows[3 * n + i]));
+    m = max(m, __float_as_int(rows[3 * N + n]));
   }
-  float h[2] = {0.f, 0.f};
-  if (e == cudaSuccess) e = cudaMemcpyAsync(h, mx, sizeof(h), cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  cudaFree(rows);
-  if (e != cudaSuccess) return e;
-  *abs_k = h[0];
-  *abs_m = h[1];
-  return cudaSuccess;
+  atomicMax(mx, m);
+  atomicMax(mx + 1, k);
+  __syncthreads();
+  if (threadIdx.x == 0)
+    bound[blockIdx.x] = make_float4(1.01f * __int_as_float(mx[0]), 1.01f * __int_as_float(mx[1]), 0.f, 0.f);
+}
+
+cudaError_t launch_tile_bounds(const HexTiles& t, int64_t N, const float* rows, float4* bound, cudaStream_t s) {
+  k_tile_bounds<<<t.n_tiles, 128, 0, s>>>(t, N, rows, bound);
+  return cudaGetLastError();
 }
 
 }  // namespace fem
