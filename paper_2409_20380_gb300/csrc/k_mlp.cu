@@ -45,7 +45,7 @@ __device__ __forceinline__ float gelu_grad_f(float z) {
 // thread owns the same entries of a layer on the way forward and back), and a second kernel forms the three
 // weight gradients.  What bounds both is latency (2.2 GFLOP a training pass at 4096 samples, ~2 us of tensor
 // time), so passes and launches are what is saved: 4096 samples took 246 us in 13 launches (three column sums of
-// 60 us on 1 to 8 blocks among them), and take 47 us in 2 launches now (66,560 samples: 3332 -> 331 us; forward
+// 60 us on 1 to 8 blocks among them), and take 46 us in 2 launches now (66,560 samples: 3332 -> 330 us; forward
 // alone at 4096: 37 -> 10 us).  32 samples a block (128 blocks at 4096) leave the
 // tensor cores mostly idle either way; tcgen05's smallest tile (128 rows) would leave 120 of 152 SMs without work.
 // Weights come straight from L2 in the order of the MMA's B fragments (k_pack): 16 bytes a lane cover 32 of K
