@@ -2064,7 +2064,8 @@ cudaError_t launch_ebe_split_df(const MeshView& m, const float* rec_df, int rpad
 // lower blocks as transposes (.trans) of the stored upper ones.  With the component-major order a lane's B
 // operand needs only corner slots 2tq and 2tq + 1, and its outputs are the three components of corner slot
 // gq.  Sums go to the tile accumulator in the packed kernel's fixed point; p^T q is taken at the flush from
-// the tile's sums and its FP32 values of p.  FP16 operands carry ~2.4e-4 of relative error into a product
+// the tile's sums and its FP32 values of p, with one FP64 addition a thread and tile (with four in registers, and
+// the Dirichlet rows branched around, it took 98 of 389 us at 8 cases on 6,291,456 tets, now 41).  FP16 operands carry ~2.4e-4 of relative error into a product
 // (FP32 accumulation): a refinement pass takes this product only when its reduction targets are 1e-3 or
 // coarser, and the FP64 certification removes the rest.  Blocks of 256 threads (two an SM with 64-hex tiles at 8 cases, three with 32-hex tiles at 16):
 // the node rows are double-buffered, the records single-buffered (the next tile's records are requested
@@ -2208,7 +2209,7 @@ __global__ void __launch_bounds__(kTcBlock, R == 8 ? 2 : 3) k_ebe_hex_tc(HexTile
   uint64_t* mbar = reinterpret_cast<uint64_t*>(smem_raw);
   int* spm = reinterpret_cast<int*>(smem_raw + 32);          // [2][32] per-case max |p| bits, per tile parity
   float* sfwd = reinterpret_cast<float*>(smem_raw + 288);    // [32] fixed point back to FP32
-  double* sdot = reinterpret_cast<double*>(smem_raw + 768);  // [32] p^T q sums of the block
+  __shared__ double sdot[kTcBlock];                          // p^T q, a word a thread
   int* qs = reinterpret_cast<int*>(smem_raw + L.qs);
   unsigned char* hs = smem_raw + L.hm;
   auto psb = [&](int b) { return reinterpret_cast<float*>(smem_raw + (b ? L.ps1 : L.ps0)); };
@@ -2223,7 +2224,7 @@ __global__ void __launch_bounds__(kTcBlock, R == 8 ? 2 : 3) k_ebe_hex_tc(HexTile
   }
   for (int i = tid; i < ht.nloc_max * f4; i += kTcBlock) reinterpret_cast<int4*>(qs)[i] = make_int4(0, 0, 0, 0);
   if (tid < 64) spm[tid] = 0;
-  if (tid < 32) sdot[tid] = 0.0;
+  if (DOT) sdot[tid] = 0.0;
   __syncthreads();
   // node rows and corner tables of tile t into buffer b (bytes of the tile's records counted too: they are
   // requested by request_records once the record buffer is free)
@@ -2263,8 +2264,6 @@ __global__ void __launch_bounds__(kTcBlock, R == 8 ? 2 : 3) k_ebe_hex_tc(HexTile
   const uint32_t o_t1 = (uint32_t)(128 * 4 + r16);
   const uint32_t hs_u32 = smem_u32(hs);
   auto sbd = [&](int b) { return reinterpret_cast<float2*>(smem_raw + 416 + 16 * b); };   // the tile's row bounds
-  float4 tdot = make_float4(0.f, 0.f, 0.f, 0.f);
-  double dd[4] = {0.0, 0.0, 0.0, 0.0};
   const int t0 = blockIdx.x;
   if (t0 < ht.n_tiles) {
     issue(t0, 0);
@@ -2353,6 +2352,13 @@ __global__ void __launch_bounds__(kTcBlock, R == 8 ? 2 : 3) k_ebe_hex_tc(HexTile
     if (tn < ht.n_tiles) request_records(tn, b ^ 1);   // the record buffer is free: the next tile's records
     // flush: float4 pieces (four cases of one component of one node) to the output; p^T q from the tile's
     // sums and its FP32 values of p (a thread's four cases are fixed: 4 kTcBlock is a multiple of R)
+    float td[4] = {0.f, 0.f, 0.f, 0.f};
+    const int c4 = (tid << 2) & (R - 1);
+    float w4[4];
+    if (DOT)
+      for (int u = 0; u < 4; ++u) w4[u] = sfwd[c4 + u];
+    // (the factors in registers with p^T q only: 297 against 290 us without it)
+    auto back = [&](int x, int u, int i) { return (float)x * (DOT ? w4[u] : sfwd[((i << 2) & (R - 1)) + u]); };
     for (int i = tid; i < nl * f4; i += kTcBlock) {
       const int l = i / f4, kk = (i - l * f4) / (R / 4);
       const int raw = snode[l];
@@ -2360,34 +2366,33 @@ __global__ void __launch_bounds__(kTcBlock, R == 8 ? 2 : 3) k_ebe_hex_tc(HexTile
       const bool fixed = !dof_free((uint8_t)((raw >> 28) & 7), kk);
       float4* dstg = reinterpret_cast<float4*>(q + g * per_node) + (i - l * f4);
       const int4 vi = reinterpret_cast<const int4*>(qs)[i];
-      const int c4 = (i << 2) & (R - 1);
-      const float4 v = make_float4((float)vi.x * sfwd[c4], (float)vi.y * sfwd[c4 + 1], (float)vi.z * sfwd[c4 + 2],
-                                   (float)vi.w * sfwd[c4 + 3]);
+      const float4 v = make_float4(back(vi.x, 0, i), back(vi.y, 1, i), back(vi.z, 2, i), back(vi.w, 3, i));
+      const float4 w = fixed ? make_float4(0.f, 0.f, 0.f, 0.f) : v;
       reinterpret_cast<int4*>(qs)[i] = make_int4(0, 0, 0, 0);
-      if (DOT && !fixed) {
+      if (DOT) {
         const float4 pv = reinterpret_cast<const float4*>(ps)[i];
-        tdot.x = fmaf(pv.x, v.x, tdot.x), tdot.y = fmaf(pv.y, v.y, tdot.y);
-        tdot.z = fmaf(pv.z, v.z, tdot.z), tdot.w = fmaf(pv.w, v.w, tdot.w);
+        td[0] = fmaf(pv.x, w.x, td[0]), td[1] = fmaf(pv.y, w.y, td[1]);
+        td[2] = fmaf(pv.z, w.z, td[2]), td[3] = fmaf(pv.w, w.w, td[3]);
       }
       if (raw < 0) {
         if (!fixed) atomicAdd(dstg, v);
       } else {
-        *dstg = fixed ? make_float4(0.f, 0.f, 0.f, 0.f) : v;
+        *dstg = w;
       }
     }
-    if (DOT) {
-      dd[0] += (double)tdot.x, dd[1] += (double)tdot.y, dd[2] += (double)tdot.z, dd[3] += (double)tdot.w;
-      tdot = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (DOT) {   // (as in the packed kernel: over four lanes in FP32, each of which goes on with one case in FP64)
+      const bool hi = tid & (R / 2), lo = tid & (R / 4);
+      const float a0 = (hi ? td[2] : td[0]) + __shfl_xor_sync(0xffffffffu, hi ? td[0] : td[2], R / 2);
+      const float a1 = (hi ? td[3] : td[1]) + __shfl_xor_sync(0xffffffffu, hi ? td[1] : td[3], R / 2);
+      const float a = (lo ? a1 : a0) + __shfl_xor_sync(0xffffffffu, lo ? a0 : a1, R / 4);
+      sdot[(tid & ~(R - 1)) + c4 + (hi ? 2 : 0) + (lo ? 1 : 0)] += (double)a;   // (its own word)
     }
     __syncthreads();
   }
   if (DOT) {
-    const int c4 = (tid << 2) & (R - 1);
-#pragma unroll
-    for (int j = 0; j < 4; ++j) atomicAdd(sdot + c4 + j, dd[j]);
-    __syncthreads();
-    double v[1] = {tid < R ? sdot[tid] : 0.0};
-    if (block_reduce_last<1>(v, R, red)) ebe_tail(red, sc, ptq_out, R);
+    double v[1] = {sdot[tid]};   // (of case tid mod R; behind the loop's last barrier)
+    // (in the memory of the tile sums, no longer needed)
+    if (block_reduce_last_in<1>(reinterpret_cast<double(*)[kVecBlock]>(smem_raw + L.qs), v, R, red)) ebe_tail(red, sc, ptq_out, R);
   }
 }
 
