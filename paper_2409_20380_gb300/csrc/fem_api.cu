@@ -429,11 +429,11 @@ struct fem_mesh {
     }
     // Automatic choice on hex patches, both sides measured alone.  FP32: packed staged tiles (5), with 1 or 2 cases (no
     // 16-byte node rows) unstaged ones.  FP64 (bound by the FP64 pipe), by the hexes H and the cases r: the hex element
-    // kernel (against the best of 64- and 128-hex tiles, r = 1, 4, 16: H = 6912 30 us against 34, 42 against 60, 139 against
-    // 194; 25,920 42 against 46, 140 against 147, 486 against 559; 50,688 75 against 79, 270 against 284, 916 against
-    // 1105; 1,048,576, r = 1, 4: 1198 against 1269, 4662 against 4987; tiles ahead at two sizes of all measured, by the last
-    // wave: 131,072, r = 1, 189 against 171, and 98,304, r = 2, 272 against 259), up to H r = 8192 with a thread a tet
-    // (H = 512, r = 1: 14.0 against 28.8; 4800, r = 1: 17 against 30, 2 29 against 30; 6912, r = 2: 34 against 29).
+    // kernel, at every size measured ahead of 64- and 128-hex tiles and of staged ones (r = 1, 4, 16: H = 15,138 31 us
+    // against 36, 94 against 102, 286 against 378; 50,688 75 against 79, 245 against 284, 911 against 1105; 131,072 163
+    // against 171, 591 against 650, 2332 against 2552; 442,368, r = 1, 4: 508 against 568, 1972 against 2142), up to H r =
+    // 8192 with a thread a tet (H = 512, r = 1: 14.0 against 28.8; 4800, r = 1: 17 against 30, r = 2: 29 against 29; 6912,
+    // r = 2: 34 against 29).
     if (elem_bytes == 8 && *variant == 0 && *hpt == 0 && hex && !seg)
       *variant = (E / 6) * rpad <= 8192 ? kHexSplit : kHexElem;
     if (*variant == 0) *variant = hex ? 5 : 1;       // packed staged tiles where they apply (else 3, 2, 1)

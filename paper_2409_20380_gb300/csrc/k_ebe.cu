@@ -115,23 +115,18 @@ __global__ void __launch_bounds__(kBlock) k_ebe_atomic(MeshView m, int rpad, int
   }
 }
 
-// Grid of the element kernels.  Small meshes: blocks small enough that the items cover the SMs twice (3072 tets, one
-// case: 96 blocks of a warp instead of 12 of 256 threads; FP64 product 12.5 us), but of at least 8 rpad threads, so that
-// the last block of the p^T q reduction has eight threads a case.
-static void elem_grid(int64_t items, int rpad, bool reduces, int* grid, int* block) {
-  int b = kBlock;
-  while (b > 32 && b > 8 * rpad && items < (int64_t)b * 2 * sm_count()) b >>= 1;
-  const int cap = reduces ? vec_grid_cap() * (kBlock / b) : red_grid_cap();
-  *grid = (int)std::min((items + b - 1) / b, (int64_t)std::min(cap, kMaxRedBlocks));
-  *block = b;
-}
-
 template <typename T, int NC>
 static cudaError_t ebe_atomic_nc(const MeshView& m, int rpad, const T* pm, const T* pk, T* q, T aM, T aK,
                                  const Reducer* red, CgCase* sc, double* ptq_out, const int* gate, cudaStream_t s) {
   const int gs = log2i(rpad / NC);
-  int grid, block;
-  elem_grid(m.E << gs, rpad, red != nullptr, &grid, &block);
+  // Small meshes: blocks small enough that the items cover the SMs twice (3072 tets, one case: 96 blocks of a
+  // warp instead of 12 of 256 threads; FP64 product 12.5 us), but of at least 8 rpad threads, so that the last
+  // block of the p^T q reduction has eight threads a case.
+  const int64_t items = m.E << gs;
+  int block = kBlock;
+  while (block > 32 && block > 8 * rpad && items < (int64_t)block * 2 * sm_count()) block >>= 1;
+  const int cap = red ? vec_grid_cap() * (kBlock / block) : red_grid_cap();
+  const int grid = (int)std::min((items + block - 1) / block, (int64_t)std::min(cap, kMaxRedBlocks));
   const Reducer rd = red ? *red : Reducer{nullptr, nullptr, nullptr};
   const bool i32 = m.N * 3 * rpad < ((int64_t)1 << 31);
   auto run = [&](auto kfn) {
@@ -531,8 +526,12 @@ cudaError_t launch_hex_atomic(const MeshView& m, int rpad, const double* p, doub
   const cudaError_t err = cudaMemsetAsync(q, 0, sizeof(double) * (size_t)m.N * 3 * rpad, s);
   if (err != cudaSuccess) return err;
   const int rs = log2i(rpad);
-  int grid, block;
-  elem_grid((m.E / 6) << rs, rpad, red != nullptr, &grid, &block);
+  // Blocks of 128 threads, two an SM by registers (256: up to 15% slower by the last wave, 131,072 hexes, one case, 189
+  // against 163 us), smaller while the items leave SMs idle, of at least four threads a case for the reduction.
+  const int64_t items = (m.E / 6) << rs;
+  int block = kBlock / 2;
+  while (block > 32 && block > 4 * rpad && items < (int64_t)block * 2 * sm_count()) block >>= 1;
+  const int grid = (int)std::min((items + block - 1) / block, (int64_t)kMaxRedBlocks);
   const Reducer rd = red ? *red : Reducer{nullptr, nullptr, nullptr};
   const bool i32 = m.N * 3 * rpad < ((int64_t)1 << 31);
   auto kfn = red ? (i32 ? k_hex_atomic<true, int32_t> : k_hex_atomic<true, int64_t>)
