@@ -775,7 +775,7 @@ def run_kernel(args):
                       "variant": args.variant, "hex_per_tile": args.hex_per_tile, "mesh_info": info,
                       "ms_per_launch": ms, "alg_gbs": bytes_launch / (ms * 1e-3) / 1e9,
                       "alg_tflops": FLOP_PER_ELEM_CASE * E * r / (ms * 1e-3) / 1e12,
-                      "note": "includes the q zero-fill and the Dirichlet mask pass of fem_ebe_apply"}), flush=True)
+                      "note": "includes the q zero-fill of fem_ebe_apply"}), flush=True)
     fem.fem_mesh_destroy(h)
 
 
@@ -826,8 +826,7 @@ def run_kernel10(args):
                       "alg_gbs": bytes_launch / (ms * 1e-3) / 1e9,
                       "alg_tflops": FLOP_PER_TET10_CASE * E * r / (ms * 1e-3) / 1e12,
                       "flop_per_elem_case": FLOP_PER_TET10_CASE,
-                      "note": "one thread per (element, case), global atomics; includes the q zero-fill and "
-                              "the Dirichlet mask pass"}), flush=True)
+                      "note": "one thread per (element, case), global atomics; includes the q zero-fill"}), flush=True)
     fem.fem_mesh10_destroy(h)
 
 

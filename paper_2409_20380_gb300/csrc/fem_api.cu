@@ -432,10 +432,10 @@ struct fem_mesh {
     // kernel, at every size measured ahead of 64- and 128-hex tiles and of staged ones (r = 1, 4, 16: H = 15,138 31 us
     // against 36, 94 against 102, 286 against 378; 50,688 75 against 79, 245 against 284, 911 against 1105; 131,072 163
     // against 171, 591 against 650, 2332 against 2552; 442,368, r = 1, 4: 508 against 568, 1972 against 2142), up to H r =
-    // 8192 with a thread a tet (H = 512, r = 1: 14.0 against 28.8; 4800, r = 1: 17 against 30, r = 2: 29 against 29; 6912,
-    // r = 2: 34 against 29).
+    // 11,000 with a thread a tet (H = 512, r = 1: 12.4 against 28.8; 4800, r = 2: 25 against 30; 1152, r = 8: 21 against 30;
+    // 3072, r = 4: 31 against 30; 6912, r = 2: 31 against 30).
     if (elem_bytes == 8 && *variant == 0 && *hpt == 0 && hex && !seg)
-      *variant = (E / 6) * rpad <= 8192 ? kHexSplit : kHexElem;
+      *variant = (E / 6) * rpad <= 11000 ? kHexSplit : kHexElem;
     if (*variant == 0) *variant = hex ? 5 : 1;       // packed staged tiles where they apply (else 3, 2, 1)
     if (!hex && *variant != 8) *variant = 1;
   }

@@ -440,20 +440,25 @@ __global__ void __launch_bounds__(kBlock) k_hex_atomic(MeshView m, int rpad, int
 // The same for very few hexes in FP64, where the chain of a whole hex (700 operations of long latency: 20 us) is what
 // bounds: one thread a tet, the hex's corner sums over its tets through shared memory.  A block takes nb items, a
 // multiple of the cases, on threads t nb + j (tet t of item j), so a thread's case is threadIdx.x mod rpad.
-// 512 hexes, one case: 14.0 us against 28.8.
-struct HexRefs {
-  int n[8], ref[8][6];     // per corner: its tets, as 4 tet + corner in the tet
-};
-constexpr HexRefs hex_refs() {
-  HexRefs r{};
+// 512 hexes, one case: 12.4 us against 28.8.
+// Of the hex's sums, thread t of an item takes those of a middle corner (two tets) and one component of corner 0 or 3
+// (all six tets).  The places 4 tet + corner of a hex corner in its tets, five bits each, are compile-time words.
+constexpr int corner_ref(int s, int i) {    // corner s in the i-th of its tets
   for (int t = 0; t < 6; ++t)
-    for (int a = 0; a < 4; ++a) {
-      const int s = kHexTet[t][a];
-      r.ref[s][r.n[s]++] = 4 * t + a;
-    }
+    for (int a = 0; a < 4; ++a)
+      if (kHexTet[t][a] == s && i-- == 0) return 4 * t + a;
+  return 0;
+}
+constexpr uint32_t end_refs(int s) {        // corner 0 or 3: its six tets
+  uint32_t r = 0;
+  for (int i = 0; i < 6; ++i) r |= (uint32_t)corner_ref(s, i) << (5 * i);
   return r;
 }
-__constant__ HexRefs c_hex_refs = hex_refs();
+constexpr uint32_t middle_refs(int i) {     // corners 1, 2, 4, 5, 6, 7: the i-th of their two tets
+  uint32_t r = 0;
+  for (int t = 0; t < 6; ++t) r |= (uint32_t)corner_ref(t < 2 ? t + 1 : t + 2, i) << (5 * t);
+  return r;
+}
 constexpr int kSplitItems = 32;
 
 template <bool DOT>
@@ -489,15 +494,23 @@ __global__ void __launch_bounds__(6 * kSplitItems) k_hex_split(MeshView m, int r
       elem4<DOT, false, double, double>(ld, ld, fl, r, aM, aK, dot);
     }
     __syncthreads();
-    for (int o = threadIdx.x; o < nb * 24; o += blockDim.x) {
-      const int jo = o / 24, s = o % 24 / 3, k = o % 3;
-      if (base + jo >= total) break;
-      const int* ref = c_hex_refs.ref[s];
-      const double* w = part[jo] + k;
-      const int n = node[jo][ref[0]];
-      double v = w[ref[0] * 3] + w[ref[1] * 3];                // (two tets, or all six at corners 0 and 3)
-      if (c_hex_refs.n[s] == 6) v += (w[ref[2] * 3] + w[ref[3] * 3]) + (w[ref[4] * 3] + w[ref[5] * 3]);
-      if (n >> (28 + k) & 1) atomicAdd(q + ((int64_t)(n & 0x0fffffff) * 3 + k) * rpad + ((base + jo) & (rpad - 1)), v);
+    if (t < 6 && i < total) {
+      constexpr uint32_t R0 = middle_refs(0), R1 = middle_refs(1), C0 = end_refs(0), C3 = end_refs(3);
+      const int c = (int)(i & (rpad - 1)), r0 = (int)(R0 >> (5 * t)) & 31, r1 = (int)(R1 >> (5 * t)) & 31;
+      const uint32_t rc = t < 3 ? C0 : C3;
+      const int kc = t < 3 ? t : t - 3;       // (corner 0 or 3: its component)
+      auto add = [&](int n, int k, double v) {
+        if (n >> (28 + k) & 1) atomicAdd(q + ((int64_t)(n & 0x0fffffff) * 3 + k) * rpad + c, v);
+      };
+      double x[6], y[3];
+#pragma unroll
+      for (int u = 0; u < 6; ++u) x[u] = part[j][((rc >> (5 * u)) & 31) * 3 + kc];
+#pragma unroll
+      for (int k = 0; k < 3; ++k) y[k] = part[j][r0 * 3 + k] + part[j][r1 * 3 + k];
+      const int nm = node[j][r0], nc = node[j][rc & 31];
+#pragma unroll
+      for (int k = 0; k < 3; ++k) add(nm, k, y[k]);
+      add(nc, kc, (x[0] + x[1]) + ((x[2] + x[3]) + (x[4] + x[5])));
     }
     __syncthreads();
   }

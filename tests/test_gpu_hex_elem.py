@@ -1,6 +1,6 @@
 """The kernels that fem_ebe_apply chooses by itself on hex patches for FP32 products of one or two cases and for FP64
 products: as exact as the tiled ones (whose corner sums over a hex's tets stay in registers), Dirichlet rows zero, sizes
-at the edges of the choice (H r = 8192) and of a block.
+at the edges of the choice (H r = 11,000) and of a block.
 
 The rms error against wider arithmetic, a mean over 20 vectors (its own spread is below 1%), is at most 6% above the
 tiles'; one atomic add a tet instead of a hex is 10% to 45% above.  The reference of FP64 products is summed in
@@ -52,7 +52,7 @@ def _operator(m, dtype, cM=CM, cK=CK):
 
 
 @pytest.mark.parametrize("dtype,dims,r", [("float32", (8, 8, 8), 1), ("float32", (12, 11, 10), 2), ("float64", (8, 8, 8), 1),
-                                          ("float64", (9, 8, 7), 4), ("float64", (11, 10, 10), 8)])
+                                          ("float64", (9, 8, 7), 4), ("float64", (12, 12, 10), 8)])
 def test_as_exact_as_tiles(torch_dev, dtype, dims, r):
     torch = torch_dev
     m, tp = wl.config2_mesh(*dims), wl.config2_time_params()
@@ -76,10 +76,10 @@ def test_as_exact_as_tiles(torch_dev, dtype, dims, r):
         fem.fem_mesh_destroy(h)
 
 
-# hexes x cases at and above 8192, one hex, blocks with a remainder
+# hexes x cases at and above 11,000, one hex, blocks with a remainder
 @pytest.mark.parametrize("dtype,dims,r", [("float64", (1, 1, 1), 1), ("float64", (1, 1, 1), 32), ("float64", (3, 2, 5), 2),
                                           ("float64", (7, 3, 3), 4), ("float64", (8, 8, 8), 16), ("float64", (9, 9, 7), 16),
-                                          ("float64", (16, 16, 16), 2), ("float64", (17, 16, 16), 2), ("float64", (8, 8, 4), 32),
+                                          ("float64", (11, 10, 25), 4), ("float64", (11, 10, 26), 4), ("float64", (8, 8, 4), 32),
                                           ("float32", (1, 1, 1), 2), ("float32", (27, 27, 27), 2), ("float32", (28, 27, 27), 2)])
 def test_edges(torch_dev, dtype, dims, r):
     torch = torch_dev
